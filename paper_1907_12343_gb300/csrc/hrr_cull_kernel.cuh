@@ -32,9 +32,9 @@
 //
 // Memory: the kernel is bound by the L1 data pipe (one scattered record per lane per
 // step), so each record is fetched with 256-bit loads that do not allocate in L1. A node's
-// range minimum is attained at its argmin, which lies in exactly one child; carrying the
-// argmin with each stack entry means only the other children's minima have to be
-// computed. Accepted pairs are staged
+// range minimum is attained at one index, which lies in exactly one child; carrying the
+// minimum with each stack entry (its index is brev(v - r)) means only the other children's
+// minima have to be computed. Accepted pairs are staged
 // per warp in shared memory and appended to the output with one atomic per frame and
 // coalesced 8-byte stores.
 //
@@ -49,7 +49,7 @@
 // much for each, so a node below the root is visited iff its own test passes, whatever its
 // ancestors' results. The head counts the root and the visited nodes above the deepest top
 // level as visits, tests the top's leaves, and pushes the visited nodes of the deepest top
-// level (with their argmins) as the stack the walk starts from: the same visited set, visit
+// level (with their range minima) as the stack the walk starts from: the same visited set, visit
 // count and accepted set as a walk from the root.
 //
 // One launch may cover many frames (a batch): the eye cursor then runs over the eyes of all
@@ -183,14 +183,16 @@ __device__ __forceinline__ void emit(const Frame *F, uint2 *wbuf, uint16_t *wfr,
     __syncwarp();
 }
 
-// Argmin of the range minimum of (brev(i) + r) over [a, b); c = brev(2^32 - r).
+// Range minimum of (brev(i) + r) over the L >= 1 indices from a; c = brev(2^32 - r).
 template <int VARIANT>
-__device__ __forceinline__ uint32_t range_argmin(uint32_t a, uint32_t b, uint32_t r, uint32_t c) {
+__device__ __forceinline__ uint32_t range_min(uint32_t a, uint32_t L, uint32_t r, uint32_t c) {
+    if (VARIANT == 0) return hrr_range_min_value(a, L, r, 0u - r, c);
     uint32_t k;
-    if (VARIANT == 0) return hrr_range_argmin_select(a, b, c);
-    hrr_rangemin_closed(a, b, r, &k);
-    return k;
+    return hrr_rangemin_closed(a, a + L, r, &k);
 }
+
+// The index at which brev(i) + r is v.
+__device__ __forceinline__ uint32_t index_of(uint32_t v, uint32_t r) { return __brev(v - r); }
 
 // The eye a traversal works on.
 struct Eye {
@@ -199,26 +201,26 @@ struct Eye {
     uint32_t r, c;  // shift and brev(2^32 - r)
 };
 
-// What one lane's visit produces: up to W children to push (node, argmin of its range
-// minimum) and up to W accepted leaves.
+// What one lane's visit produces: up to W children to push (node, range minimum) and up to W
+// accepted leaves.
 template <int W>
 struct Visit {
     bool go[W];
-    uint32_t node[W], karg[W], acc[W];
+    uint32_t node[W], vmin[W], acc[W];
 };
 
 // Test one child slot: an internal child (range of more than one leaf) survives unless
-// its range minimum at argmin k culls it; the box is (lo, imax, hi).
-__device__ __forceinline__ bool survives(const Eye &E, const float4 &lo, const float4 &hi, uint32_t k) {
+// its range minimum v culls it; the box is (lo, imax, hi).
+__device__ __forceinline__ bool survives(const Eye &E, const float4 &lo, const float4 &hi, uint32_t v) {
     float den, rhs;
     hrr_node_bound(E.scale, lo.x, lo.y, lo.z, hi.x, hi.y, hi.z, lo.w, E.x, E.y, E.z, den, rhs);
-    return !hrr_node_culls(__brev(k) + E.r, den, rhs);
+    return !hrr_node_culls(v, den, rhs);
 }
 
 // A visit of binary node `node`: its 64-byte record holds both children (box low corner
 // with the maximum intensity, box high corner with `split` / the range's other end).
 template <int VARIANT>
-__device__ __forceinline__ void visit(const float4 *nodes, uint32_t n_lights, uint32_t node, uint32_t kmin,
+__device__ __forceinline__ void visit(const float4 *nodes, uint32_t n_lights, uint32_t node, uint32_t vmin,
                                       const Eye &E, unsigned long long *flags, Visit<2> &V) {
     float4 q0, q1, q2, q3;
     load32(&nodes[4 * (size_t)node], q0, q1);
@@ -231,16 +233,16 @@ __device__ __forceinline__ void visit(const float4 *nodes, uint32_t n_lights, ui
         return;
     }
     const bool int0 = first != split, int1 = split + 1u != last;
-    const bool kin0 = kmin <= split;
-    // the other child's argmin (unused when that child is a leaf: computing it anyway
+    const bool in0 = index_of(vmin, E.r) <= split;
+    // the other child's minimum (unused when that child is a leaf: computing it anyway
     // keeps the warp on one path)
-    const uint32_t knew = range_argmin<VARIANT>(kin0 ? split + 1u : first, kin0 ? last + 1u : split + 1u, E.r, E.c);
-    V.karg[0] = kin0 ? kmin : knew;
-    V.karg[1] = kin0 ? knew : kmin;
+    const uint32_t vnew = range_min<VARIANT>(in0 ? split + 1u : first, in0 ? last - split : split - first + 1u, E.r, E.c);
+    V.vmin[0] = in0 ? vmin : vnew;
+    V.vmin[1] = in0 ? vnew : vmin;
     V.node[0] = split;
     V.node[1] = split + 1u;
-    V.go[0] = int0 && survives(E, q0, q1, V.karg[0]);
-    V.go[1] = int1 && survives(E, q2, q3, V.karg[1]);
+    V.go[0] = int0 && survives(E, q0, q1, V.vmin[0]);
+    V.go[1] = int1 && survives(E, q2, q3, V.vmin[1]);
     if (!int0 || !int1) {  // leaf children: one test site, a second for two leaves
         const uint32_t i = !int0 ? split : last;
         const float4 ql = !int0 ? q0 : q2;
@@ -253,11 +255,11 @@ __device__ __forceinline__ void visit(const float4 *nodes, uint32_t n_lights, ui
 
 // A visit of node g read with width four: its 128-byte record holds the four grandchild
 // slots [first, s0], [s0 + 1, split], [split + 1, s1], [s1 + 1, last] (a leaf child fills its
-// first slot and leaves the second empty). The parent's argmin lies in one child; one range
-// minimum gives the other child's, and one more per internal child splits it between that
-// child's two slots.
+// first slot and leaves the second empty). The parent's minimum is attained in one child; one
+// more range minimum gives the other child's, and one more per internal child splits it
+// between that child's two slots.
 template <int VARIANT>
-__device__ __forceinline__ void visit(const float4 *wide, uint32_t n_lights, uint32_t g, uint32_t kmin,
+__device__ __forceinline__ void visit(const float4 *wide, uint32_t n_lights, uint32_t g, uint32_t vmin,
                                       const Eye &E, unsigned long long *flags, Visit<4> &V) {
     float4 q[8];
     load32(&wide[8 * (size_t)g], q[0], q[1]);
@@ -275,21 +277,21 @@ __device__ __forceinline__ void visit(const float4 *wide, uint32_t n_lights, uin
         atomicOr(flags, HRR_FLAG_TOPOLOGY);  // corrupt record
         return;
     }
-    const bool kin0 = kmin <= split;
-    const uint32_t kc = range_argmin<VARIANT>(kin0 ? split + 1u : first, kin0 ? last + 1u : split + 1u, E.r, E.c);
-    const uint32_t kA = kin0 ? kmin : kc, kB = kin0 ? kc : kmin;  // argmins of children 0 and 1
-    uint32_t k[4] = {kA, kA, kB, kB};
+    const bool in0 = index_of(vmin, E.r) <= split;
+    const uint32_t vc = range_min<VARIANT>(in0 ? split + 1u : first, in0 ? last - split : split - first + 1u, E.r, E.c);
+    const uint32_t vA = in0 ? vmin : vc, vB = in0 ? vc : vmin;  // range minima of children 0 and 1
+    uint32_t v[4] = {vA, vA, vB, vB};
     if (c0int) {
-        const bool in0 = kA <= s0;
-        const uint32_t kx = range_argmin<VARIANT>(in0 ? s0 + 1u : first, in0 ? split + 1u : s0 + 1u, E.r, E.c);
-        k[0] = in0 ? kA : kx;
-        k[1] = in0 ? kx : kA;
+        const bool at0 = index_of(vA, E.r) <= s0;
+        const uint32_t vx = range_min<VARIANT>(at0 ? s0 + 1u : first, at0 ? split - s0 : s0 - first + 1u, E.r, E.c);
+        v[0] = at0 ? vA : vx;
+        v[1] = at0 ? vx : vA;
     }
     if (c1int) {
-        const bool in2 = kB <= s1;
-        const uint32_t ky = range_argmin<VARIANT>(in2 ? s1 + 1u : split + 1u, in2 ? last + 1u : s1 + 1u, E.r, E.c);
-        k[2] = in2 ? kB : ky;
-        k[3] = in2 ? ky : kB;
+        const bool at2 = index_of(vB, E.r) <= s1;
+        const uint32_t vy = range_min<VARIANT>(at2 ? s1 + 1u : split + 1u, at2 ? last - s1 : s1 - split, E.r, E.c);
+        v[2] = at2 ? vB : vy;
+        v[3] = at2 ? vy : vB;
     }
     const uint32_t a[4] = {first, s0 + 1u, split + 1u, s1 + 1u};
     const uint32_t b[4] = {s0, split, s1, last};  // inclusive; a > b: an empty slot
@@ -300,8 +302,8 @@ __device__ __forceinline__ void visit(const float4 *wide, uint32_t n_lights, uin
     bool any_leaf = false;
 #pragma unroll
     for (int t = 0; t < 4; ++t) {
-        V.karg[t] = k[t];
-        V.go[t] = a[t] < b[t] && survives(E, q[2 * t], q[2 * t + 1], k[t]);
+        V.vmin[t] = v[t];
+        V.go[t] = a[t] < b[t] && survives(E, q[2 * t], q[2 * t + 1], v[t]);
         any_leaf |= a[t] == b[t];
     }
     if (any_leaf) {
@@ -332,7 +334,7 @@ __device__ __forceinline__ uint32_t head(const float4 *top, const Eye &E, const 
         uint32_t acc[W];
 #pragma unroll
         for (int t = 0; t < W; ++t) acc[t] = kNone;
-        uint32_t node = 0, karg = 0;
+        uint32_t node = 0, vmin = 0;
         if (s < HRR_TOP_SLOTS) {
             float4 a, h, x;
             if constexpr (BATCH) {
@@ -347,8 +349,8 @@ __device__ __forceinline__ uint32_t head(const float4 *top, const Eye &E, const 
             const uint32_t kind = __float_as_uint(x.z);
             const uint32_t first = __float_as_uint(h.w), last = __float_as_uint(x.x);
             if (kind == HRR_TOP_INTERNAL) {
-                karg = range_argmin<VARIANT>(first, last + 1u, E.r, E.c);
-                vis = survives(E, a, h, karg);
+                vmin = range_min<VARIANT>(first, last - first + 1u, E.r, E.c);
+                vis = survives(E, a, h, vmin);
                 node = __float_as_uint(x.y);
             } else if (kind == HRR_TOP_LEAF &&
                        hrr_leaf_accepts(__brev(first) + E.r, E.tau, E.scale, a.x, a.y, a.z, a.w, E.x, E.y, E.z)) {
@@ -358,7 +360,7 @@ __device__ __forceinline__ uint32_t head(const float4 *top, const Eye &E, const 
         const bool deep = s >= kDeep;
         visits += __popc(__ballot_sync(0xFFFFFFFFu, vis && !deep));
         const unsigned bp = __ballot_sync(0xFFFFFFFFu, vis && deep);
-        if (vis && deep) ring[n + __popc(bp & lt)] = make_uint2(node, karg);
+        if (vis && deep) ring[n + __popc(bp & lt)] = make_uint2(node, vmin);
         n += __popc(bp);
         if (__any_sync(0xFFFFFFFFu, acc[0] != kNone)) emit<BATCH, W>(F, wbuf, wfr, cnt, lane, f, j, acc);
     }
@@ -382,7 +384,7 @@ __device__ __forceinline__ void traverse(const Launch &Lc, const Frame *F) {
     static_assert(TOP == 0 || (TOP == (int)HRR_TOP_LEVELS && W == 2 && kRing >= 32), "top levels");
     __shared__ uint2 buf[kWarps][kBuf];
     __shared__ uint16_t buf_frame[BATCH ? kWarps : 1][BATCH ? kBuf : 1];
-    __shared__ uint2 ring_all[kWarps][kRing];  // (node, argmin of its range minimum)
+    __shared__ uint2 ring_all[kWarps][kRing];  // (node, its range minimum)
     constexpr bool kTopShared = TOP > 0 && !BATCH;
     __shared__ float4 top_s[kTopShared ? 3 * HRR_TOP_SLOTS : 1];
     if constexpr (kTopShared) {  // the top slots follow the frame's binary records
@@ -455,7 +457,7 @@ __device__ __forceinline__ void traverse(const Launch &Lc, const Frame *F) {
             visits = head<VARIANT, BATCH, W>(top, E, F, wbuf, wfr, cnt, lane, f, j, ring, S);
             R = S;
         } else {
-            if (lane == 0) ring[0] = make_uint2(0u, range_argmin<VARIANT>(0u, n_lights, E.r, E.c));
+            if (lane == 0) ring[0] = make_uint2(0u, range_min<VARIANT>(0u, n_lights, E.r, E.c));
             __syncwarp();
         }
         while (S > 0) {
@@ -485,7 +487,7 @@ __device__ __forceinline__ void traverse(const Launch &Lc, const Frame *F) {
             for (int t = 0; t < W; ++t) {
                 V.go[t] = false;
                 V.node[t] = 0;
-                V.karg[t] = 0;
+                V.vmin[t] = 0;
                 V.acc[t] = kNone;
             }
             if (active) visit<VARIANT>(nodes, n_lights, e.x, e.y, E, Lc.flags, V);
@@ -517,7 +519,7 @@ __device__ __forceinline__ void traverse(const Launch &Lc, const Frame *F) {
                 for (int t = 0; t < W; ++t) pos += __popc(bal[t] & lt);
 #pragma unroll
                 for (int t = 0; t < W; ++t) {
-                    if (V.go[t]) ring[pos & kRingMask] = make_uint2(V.node[t], V.karg[t]);
+                    if (V.go[t]) ring[pos & kRingMask] = make_uint2(V.node[t], V.vmin[t]);
                     pos += V.go[t] ? 1u : 0u;
                 }
                 S += n;

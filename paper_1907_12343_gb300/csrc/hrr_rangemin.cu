@@ -16,8 +16,9 @@ __device__ __forceinline__ uint32_t one_query(uint32_t a, uint32_t b, uint32_t r
         return 0xFFFFFFFFu;
     }
     if (VARIANT == 0) {
-        *k = hrr_range_argmin_select(a, b, __brev(0u - r));
-        return __brev(*k) + r;
+        const uint32_t T = 0u - r, v = hrr_range_min_value(a, b - a, r, T, __brev(T));
+        *k = __brev(v + T);
+        return v;
     }
     return hrr_rangemin_closed(a, b, r, k);
 }

@@ -208,14 +208,14 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) cull_samples_kernel(cons
                 if (valid && ((e.y >> s) & 1u)) {
                     const uint32_t bit = 1u << s;
                     if (int0) {
-                        const uint32_t k = hrr_range_argmin_select(first, split + 1u, cs);
-                        if (!hrr_node_culls(__brev(k) + rs, den0, rhs0)) mask0 |= bit;
+                        const uint32_t v = hrr_range_min_value(first, split + 1u - first, rs, 0u - rs, cs);
+                        if (!hrr_node_culls(v, den0, rhs0)) mask0 |= bit;
                     } else if (hrr_leaf_accepts(__brev(split) + rs, tau, scale, q0.x, q0.y, q0.z, q0.w, ex, ey, ez)) {
                         acc0 |= bit;
                     }
                     if (int1) {
-                        const uint32_t k = hrr_range_argmin_select(split + 1u, last + 1u, cs);
-                        if (!hrr_node_culls(__brev(k) + rs, den1, rhs1)) mask1 |= bit;
+                        const uint32_t v = hrr_range_min_value(split + 1u, last - split, rs, 0u - rs, cs);
+                        if (!hrr_node_culls(v, den1, rhs1)) mask1 |= bit;
                     } else if (hrr_leaf_accepts(__brev(last) + rs, tau, scale, q2.x, q2.y, q2.z, q2.w, ex, ey, ez)) {
                         acc1 |= bit;
                     }
