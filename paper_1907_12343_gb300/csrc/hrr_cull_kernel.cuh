@@ -4,10 +4,12 @@
 //
 // For eye j with shift r_j (tile entry at its pixel), the traversal starts at the root and,
 // at every visited node, tests the node's children from one record:
-//   * a leaf child i is accepted iff brev(i) + r_j < ceil(p_ij 2^32) (exact float32 p);
-//   * an internal child with leaf range [a, b) is descended unless the range minimum
+//   * a child with leaf range [a, b) survives unless the range minimum
 //     v(a, b) = min_{i in [a,b)} (brev(i) + r_j) mod 2^32 passes the conservative cull test
-//     (v is at least the threshold of every light below; then none can be accepted).
+//     (v is at least the threshold of every light below; then none can be accepted);
+//   * a surviving internal child is descended; a surviving leaf child i (whose box is the
+//     light's position and whose minimum is its own value) is accepted iff
+//     brev(i) + r_j < ceil(p_ij 2^32) (exact float32 p).
 // The accepted set therefore equals flat Russian roulette over all pairs.
 //
 // Node width. The hierarchy is binary; a traversal reads it either with binary nodes
@@ -22,8 +24,11 @@
 // warp traverses one eye at a time. The warp's stack of pending nodes is a ring in shared
 // memory; every step pops up to 32 nodes, one per lane, and the lanes push the children
 // that survive their tests back as one compacted run (ballot + popc). All lanes of a step
-// execute the same node test on the same eye, so the warp stays converged except at leaf
-// children. When the ring would overflow, its oldest entries move to a per-warp area in
+// execute the same test on the same eye, leaf children included, so the warp stays
+// converged. A leaf child that survives (about one in a hundred visits, nearly all of them
+// accepted) is queued in shared memory, and the exact pair test runs on 32 queued leaves at
+// a time, and on the rest when the eye is done. Testing leaves in the step itself took a
+// divergent branch with one or two lanes in two of three steps. When the ring would overflow, its oldest entries move to a per-warp area in
 // global memory, and they come back when the ring runs low. The stack never exceeds
 // (w - 1) * 32 * L + 32 entries for node width w and L depth levels of pushed nodes (each
 // remainder of a pushed run below the top holds at most (w - 1) * 32 entries, and the
@@ -34,9 +39,8 @@
 // step), so each record is fetched with 256-bit loads that do not allocate in L1. A node's
 // range minimum is attained at one index, which lies in exactly one child; carrying the
 // minimum with each stack entry (its index is brev(v - r)) means only the other children's
-// minima have to be computed. Accepted pairs are staged
-// per warp in shared memory and appended to the output with one atomic per frame and
-// coalesced 8-byte stores.
+// minima have to be computed. The accepted pairs of one batch of queued leaves are appended
+// to the output with one atomic and neighbouring 8-byte stores.
 //
 // The head (forms with top levels, binary records): each eye starts by evaluating the 62
 // nodes below the root of the top HRR_TOP_LEVELS levels, one per lane in two passes,
@@ -64,13 +68,7 @@
 
 namespace {
 
-#ifndef HRR_CULL_BUF
-#define HRR_CULL_BUF 128  // staged output pairs per warp
-#endif
-
-constexpr int kBuf = HRR_CULL_BUF;
 constexpr uint32_t kMaxFrames = HRR_CULL_MAX_FRAMES;  // frames of one batched launch
-constexpr uint32_t kNone = 0xFFFFFFFFu;
 
 // Resident threads per SM each instantiation is compiled for (the register budget):
 // 40 registers for binary records (6 blocks of 256 threads), 64 for width four.
@@ -114,75 +112,6 @@ __device__ __forceinline__ void load32(const float4 *p, float4 &a, float4 &b) {
         : "l"(p));
 }
 
-// Append the warp's staged pairs to their frames' outputs: one atomic per frame present in
-// each 32-entry chunk (a chunk rarely holds more than one frame). The pairs are written
-// once and never read by the kernel, so they are stored with the streaming (evict-first)
-// hint: the output stream then does not push the node records out of L2.
-template <bool BATCH>
-__device__ __forceinline__ void flush(const Frame *F, const uint2 *wbuf, const uint16_t *wfr, uint32_t cnt,
-                                      int lane) {
-    if constexpr (!BATCH) {
-        unsigned long long base = 0;
-        if (lane == 0) base = atomicAdd(&F[0].counts[0], (unsigned long long)cnt);
-        base = __shfl_sync(0xFFFFFFFFu, base, 0);
-        for (uint32_t k = lane; k < cnt; k += 32) {
-            const unsigned long long o = base + k;
-            if (o < F[0].cap) __stcs(&F[0].pairs[o], wbuf[k]);
-        }
-    } else {
-        for (uint32_t k0 = 0; k0 < cnt; k0 += 32) {
-            const uint32_t k = k0 + lane;
-            const bool has = k < cnt;
-            const uint32_t f = has ? wfr[k] : 0xFFFFFFFFu;
-            const unsigned grp = __match_any_sync(0xFFFFFFFFu, f);
-            const int leader = __ffs(grp) - 1;
-            const uint32_t rank = __popc(grp & ((1u << lane) - 1u));
-            unsigned long long base = 0;
-            if (has && lane == leader)
-                base = atomicAdd(&frame_at<BATCH>(F, f).counts[0], (unsigned long long)__popc(grp));
-            base = __shfl_sync(0xFFFFFFFFu, base, leader);
-            if (has) {
-                const Frame &fr = frame_at<BATCH>(F, f);
-                const unsigned long long o = base + rank;
-                if (o < fr.cap) __stcs(&fr.pairs[o], wbuf[k]);
-            }
-        }
-    }
-    __syncwarp();
-}
-
-// Stage the accepted leaves (up to W per lane, kNone for none) of eye j (warp-collective).
-template <bool BATCH, int W>
-__device__ __forceinline__ void emit(const Frame *F, uint2 *wbuf, uint16_t *wfr, uint32_t &cnt, int lane,
-                                     uint32_t f, uint32_t j, const uint32_t (&acc)[W]) {
-    unsigned bal[W];
-    uint32_t tot = 0;
-#pragma unroll
-    for (int k = 0; k < W; ++k) {
-        bal[k] = __ballot_sync(0xFFFFFFFFu, acc[k] != kNone);
-        tot += __popc(bal[k]);
-    }
-    if (tot == 0) return;
-    if (cnt + tot > (uint32_t)kBuf) {  // tot <= 32 W <= kBuf
-        flush<BATCH>(F, wbuf, wfr, cnt, lane);
-        cnt = 0;
-    }
-    const unsigned lt = (1u << lane) - 1u;
-    const uint32_t *perm = frame_at<BATCH>(F, f).perm;
-    uint32_t base = cnt;
-#pragma unroll
-    for (int k = 0; k < W; ++k) {
-        if (acc[k] != kNone) {
-            const uint32_t o = base + __popc(bal[k] & lt);
-            wbuf[o] = make_uint2(j, __ldg(&perm[acc[k]]));
-            if constexpr (BATCH) wfr[o] = (uint16_t)f;
-        }
-        base += __popc(bal[k]);
-    }
-    cnt += tot;
-    __syncwarp();
-}
-
 // Range minimum of (brev(i) + r) over the L >= 1 indices from a; c = brev(2^32 - r).
 template <int VARIANT>
 __device__ __forceinline__ uint32_t range_min(uint32_t a, uint32_t L, uint32_t r, uint32_t c) {
@@ -202,15 +131,15 @@ struct Eye {
 };
 
 // What one lane's visit produces: up to W children to push (node, range minimum) and up to W
-// accepted leaves.
+// surviving leaves.
 template <int W>
 struct Visit {
-    bool go[W];
-    uint32_t node[W], vmin[W], acc[W];
+    bool go[W], leaf[W];
+    uint32_t node[W], vmin[W], light[W];
 };
 
-// Test one child slot: an internal child (range of more than one leaf) survives unless
-// its range minimum v culls it; the box is (lo, imax, hi).
+// Test one child slot: it survives unless its range minimum v culls it; the box is (lo, imax,
+// hi), for a leaf the light itself, which fails this test only if the pair is rejected.
 __device__ __forceinline__ bool survives(const Eye &E, const float4 &lo, const float4 &hi, uint32_t v) {
     float den, rhs;
     hrr_node_bound(E.scale, lo.x, lo.y, lo.z, hi.x, hi.y, hi.z, lo.w, E.x, E.y, E.z, den, rhs);
@@ -234,23 +163,19 @@ __device__ __forceinline__ void visit(const float4 *nodes, uint32_t n_lights, ui
     }
     const bool int0 = first != split, int1 = split + 1u != last;
     const bool in0 = index_of(vmin, E.r) <= split;
-    // the other child's minimum (unused when that child is a leaf: computing it anyway
-    // keeps the warp on one path)
+    // the other child's minimum (of a leaf: its own value)
     const uint32_t vnew = range_min<VARIANT>(in0 ? split + 1u : first, in0 ? last - split : split - first + 1u, E.r, E.c);
     V.vmin[0] = in0 ? vmin : vnew;
     V.vmin[1] = in0 ? vnew : vmin;
     V.node[0] = split;
     V.node[1] = split + 1u;
-    V.go[0] = int0 && survives(E, q0, q1, V.vmin[0]);
-    V.go[1] = int1 && survives(E, q2, q3, V.vmin[1]);
-    if (!int0 || !int1) {  // leaf children: one test site, a second for two leaves
-        const uint32_t i = !int0 ? split : last;
-        const float4 ql = !int0 ? q0 : q2;
-        if (hrr_leaf_accepts(__brev(i) + E.r, E.tau, E.scale, ql.x, ql.y, ql.z, ql.w, E.x, E.y, E.z)) V.acc[0] = i;
-        if (!int0 && !int1 &&
-            hrr_leaf_accepts(__brev(last) + E.r, E.tau, E.scale, q2.x, q2.y, q2.z, q2.w, E.x, E.y, E.z))
-            V.acc[1] = last;
-    }
+    const bool s0 = survives(E, q0, q1, V.vmin[0]), s1 = survives(E, q2, q3, V.vmin[1]);
+    V.go[0] = s0 && int0;
+    V.go[1] = s1 && int1;
+    V.leaf[0] = s0 && !int0;
+    V.leaf[1] = s1 && !int1;
+    V.light[0] = split;
+    V.light[1] = last;
 }
 
 // A visit of node g read with width four: its 128-byte record holds the four grandchild
@@ -299,44 +224,74 @@ __device__ __forceinline__ void visit(const float4 *wide, uint32_t n_lights, uin
     V.node[1] = s0 + 1u;
     V.node[2] = s1;
     V.node[3] = s1 + 1u;
-    bool any_leaf = false;
 #pragma unroll
     for (int t = 0; t < 4; ++t) {
         V.vmin[t] = v[t];
-        V.go[t] = a[t] < b[t] && survives(E, q[2 * t], q[2 * t + 1], v[t]);
-        any_leaf |= a[t] == b[t];
-    }
-    if (any_leaf) {
-#pragma unroll
-        for (int t = 0; t < 4; ++t)
-            if (a[t] == b[t] &&
-                hrr_leaf_accepts(__brev(a[t]) + E.r, E.tau, E.scale, q[2 * t].x, q[2 * t].y, q[2 * t].z, q[2 * t].w, E.x,
-                                 E.y, E.z))
-                V.acc[t] = a[t];
+        const bool s = a[t] <= b[t] && survives(E, q[2 * t], q[2 * t + 1], v[t]);
+        V.go[t] = s && a[t] < b[t];
+        V.leaf[t] = s && a[t] == b[t];
+        V.light[t] = a[t];
     }
 }
 
+// The exact test of one light per lane (`has`: the lane has one, at position (x, y, z) of
+// intensity w and sorted index i) for eye j, and the accepted pairs appended to the frame's
+// output: one atomic, neighbouring stores (warp-collective). The pairs are written once and
+// never read by the kernel, so they are stored with the streaming (evict-first) hint: the
+// output stream then does not push the node records out of L2.
+__device__ __forceinline__ void take(const Frame &fr, const Eye &E, uint32_t j, int lane, bool has, const float4 &l,
+                                     uint32_t i) {
+    const bool acc = has && hrr_pair_accepts(__brev(i) + E.r, E.tau, l.x, l.y, l.z, l.w, E.x, E.y, E.z);
+    const unsigned bal = __ballot_sync(0xFFFFFFFFu, acc);
+    if (bal == 0u) return;
+    unsigned long long base = 0;
+    if (lane == 0) base = atomicAdd(&fr.counts[0], (unsigned long long)__popc(bal));
+    base = __shfl_sync(0xFFFFFFFFu, base, 0);
+    const unsigned long long o = base + __popc(bal & ((1u << lane) - 1u));
+    if (acc && o < fr.cap) __stcs(&fr.pairs[o], make_uint2(j, __ldg(&fr.perm[i])));
+}
+
+// A queued leaf: the node whose record holds it, its slot t there and its sorted index, with
+// the bits of t in the words' top bits (nodes and lights number less than 2^31).
+__device__ __forceinline__ uint2 queued(uint32_t node, uint32_t t, uint32_t light) {
+    return make_uint2(node | (t >> 1 << 31), light | (t << 31));
+}
+
+// Take the n <= 32 newest of the warp's queued leaves.
+template <int W>
+__device__ __forceinline__ void take_queued(const Frame &fr, const Eye &E, uint32_t j, int lane, const uint2 *q,
+                                            uint32_t n) {
+    const bool has = (uint32_t)lane < n;
+    float4 l = make_float4(0.f, 0.f, 0.f, 0.f);
+    uint32_t i = 0;
+    if (has) {
+        const uint2 e = q[lane];
+        const uint32_t t = (e.x >> 31 << 1) | (e.y >> 31);
+        i = e.y & 0x7FFFFFFFu;
+        l = __ldg(&fr.nodes[(size_t)(2 * W) * (e.x & 0x7FFFFFFFu) + 2u * t]);
+    }
+    __syncwarp();
+    take(fr, E, j, lane, has, l, i);
+}
+
 // The head of eye j's traversal over the top slots `top` (shared memory for a single frame,
-// global memory for a batch): stages the top's accepted leaves, pushes the visited nodes of
+// global memory for a batch): takes the top's surviving leaves, pushes the visited nodes of
 // the deepest top level onto the empty ring, and returns the visits it accounts for (the
 // root and the visited nodes above that level).
-template <int VARIANT, bool BATCH, int W>
-__device__ __forceinline__ uint32_t head(const float4 *top, const Eye &E, const Frame *F, uint2 *wbuf, uint16_t *wfr,
-                                         uint32_t &cnt, int lane, uint32_t f, uint32_t j, uint2 *ring,
-                                         uint32_t &pushed) {
+template <int VARIANT, bool BATCH>
+__device__ __forceinline__ uint32_t head(const float4 *top, const Eye &E, const Frame &fr, int lane, uint32_t j,
+                                         uint2 *ring, uint32_t &pushed) {
     constexpr uint32_t kDeep = HRR_TOP_SLOTS / 2;  // first slot of the deepest top level
     const unsigned lt = (1u << lane) - 1u;
     uint32_t visits = 1, n = 0;  // the root
 #pragma unroll
     for (uint32_t p = 0; p < (HRR_TOP_SLOTS + 31) / 32; ++p) {
         const uint32_t s = 1u + (uint32_t)lane + 32u * p;  // slots 1 .. HRR_TOP_SLOTS - 1
-        bool vis = false;
-        uint32_t acc[W];
-#pragma unroll
-        for (int t = 0; t < W; ++t) acc[t] = kNone;
-        uint32_t node = 0, vmin = 0;
+        bool vis = false, leaf = false;
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+        uint32_t node = 0, vmin = 0, light = 0;
         if (s < HRR_TOP_SLOTS) {
-            float4 a, h, x;
+            float4 h, x;
             if constexpr (BATCH) {
                 a = __ldg(&top[3 * s]);
                 h = __ldg(&top[3 * s + 1]);
@@ -348,13 +303,13 @@ __device__ __forceinline__ uint32_t head(const float4 *top, const Eye &E, const 
             }
             const uint32_t kind = __float_as_uint(x.z);
             const uint32_t first = __float_as_uint(h.w), last = __float_as_uint(x.x);
-            if (kind == HRR_TOP_INTERNAL) {
+            if (kind != HRR_TOP_EMPTY) {
                 vmin = range_min<VARIANT>(first, last - first + 1u, E.r, E.c);
-                vis = survives(E, a, h, vmin);
+                const bool s = survives(E, a, h, vmin);
+                vis = s && kind == HRR_TOP_INTERNAL;
+                leaf = s && kind == HRR_TOP_LEAF;
                 node = __float_as_uint(x.y);
-            } else if (kind == HRR_TOP_LEAF &&
-                       hrr_leaf_accepts(__brev(first) + E.r, E.tau, E.scale, a.x, a.y, a.z, a.w, E.x, E.y, E.z)) {
-                acc[0] = first;
+                light = first;
             }
         }
         const bool deep = s >= kDeep;
@@ -362,7 +317,7 @@ __device__ __forceinline__ uint32_t head(const float4 *top, const Eye &E, const 
         const unsigned bp = __ballot_sync(0xFFFFFFFFu, vis && deep);
         if (vis && deep) ring[n + __popc(bp & lt)] = make_uint2(node, vmin);
         n += __popc(bp);
-        if (__any_sync(0xFFFFFFFFu, acc[0] != kNone)) emit<BATCH, W>(F, wbuf, wfr, cnt, lane, f, j, acc);
+        if (__any_sync(0xFFFFFFFFu, leaf)) take(fr, E, j, lane, leaf, a, light);
     }
     __syncwarp();
     pushed = n;
@@ -379,11 +334,10 @@ __device__ __forceinline__ void traverse(const Launch &Lc, const Frame *F) {
     // a step pushes at most 32 W entries; making room for them must only move entries that
     // are resident (see the spill below), which needs kRing >= 32 W + 31
     static_assert((kRing & kRingMask) == 0 && kRing >= 32 * W + 32, "ring size");
-    static_assert(kBuf >= 32 * W, "output staging buffer");
+    constexpr uint32_t kQueue = 32 * W + 32;  // a step queues at most 32 W leaves onto fewer than 32
     // the head reads the frames' binary records and pushes at most 32 entries
     static_assert(TOP == 0 || (TOP == (int)HRR_TOP_LEVELS && W == 2 && kRing >= 32), "top levels");
-    __shared__ uint2 buf[kWarps][kBuf];
-    __shared__ uint16_t buf_frame[BATCH ? kWarps : 1][BATCH ? kBuf : 1];
+    __shared__ uint2 queue_all[kWarps][kQueue];  // surviving leaves of the eye (see queued)
     __shared__ uint2 ring_all[kWarps][kRing];  // (node, its range minimum)
     constexpr bool kTopShared = TOP > 0 && !BATCH;
     __shared__ float4 top_s[kTopShared ? 3 * HRR_TOP_SLOTS : 1];
@@ -397,12 +351,11 @@ __device__ __forceinline__ void traverse(const Launch &Lc, const Frame *F) {
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
-    uint2 *wbuf = buf[warp];
-    uint16_t *wfr = BATCH ? buf_frame[warp] : nullptr;
+    uint2 *queue = queue_all[warp];
     uint2 *ring = ring_all[warp];
     // This warp's spill area (formed where it is used, so that it holds no registers).
 #define HRR_WARP_SPILL (Lc.spill + ((size_t)blockIdx.x * kWarps + warp) * Lc.spill_cap)
-    uint32_t cnt = 0, f = 0;
+    uint32_t f = 0;
     unsigned long long visit_acc = 0;  // visits of finished eyes of frame f, not yet published
 
     for (;;) {
@@ -437,24 +390,18 @@ __device__ __forceinline__ void traverse(const Launch &Lc, const Frame *F) {
         const uint32_t tx = fr.px[j] % fr.tile_w, ty = fr.py[j] % fr.tile_h;
         E.r = fr.tile[ty * fr.tile_w + tx] + fr.shift_offset;
         if (n_lights == 1) {  // the root is a leaf (record 0, slot 0, in either layout)
-            uint32_t acc[W];
-#pragma unroll
-            for (int t = 0; t < W; ++t) acc[t] = kNone;
-            if (lane == 0) {
-                const float4 q0 = __ldg(&nodes[0]);
-                if (hrr_leaf_accepts(__brev(0u) + E.r, E.tau, E.scale, q0.x, q0.y, q0.z, q0.w, E.x, E.y, E.z)) acc[0] = 0;
-                if (fr.eye_visits) fr.eye_visits[j] = 0;
-            }
-            emit<BATCH, W>(F, wbuf, wfr, cnt, lane, f, j, acc);
+            if (lane == 0 && fr.eye_visits) fr.eye_visits[j] = 0;
+            take(fr, E, j, lane, lane == 0, __ldg(&nodes[0]), 0u);
             continue;
         }
         E.c = __brev(0u - E.r);
         // Stack: logical entries [0, S); the newest R of them are in the ring at index & mask,
         // the others in the spill area at their logical index.
         uint32_t S = 1, R = 1, visits = 0;
+        uint32_t queued_n = 0;  // surviving leaves of this eye still to be taken
         if constexpr (TOP > 0) {
             const float4 *top = kTopShared ? top_s : nodes + 4 * (size_t)(n_lights - 1u);
-            visits = head<VARIANT, BATCH, W>(top, E, F, wbuf, wfr, cnt, lane, f, j, ring, S);
+            visits = head<VARIANT, BATCH>(top, E, fr, lane, j, ring, S);
             R = S;
         } else {
             if (lane == 0) ring[0] = make_uint2(0u, range_min<VARIANT>(0u, n_lights, E.r, E.c));
@@ -485,10 +432,8 @@ __device__ __forceinline__ void traverse(const Launch &Lc, const Frame *F) {
             Visit<W> V;
 #pragma unroll
             for (int t = 0; t < W; ++t) {
-                V.go[t] = false;
-                V.node[t] = 0;
-                V.vmin[t] = 0;
-                V.acc[t] = kNone;
+                V.go[t] = V.leaf[t] = false;
+                V.node[t] = V.vmin[t] = V.light[t] = 0;
             }
             if (active) visit<VARIANT>(nodes, n_lights, e.x, e.y, E, Lc.flags, V);
             // Push the surviving children as one compacted run.
@@ -526,18 +471,30 @@ __device__ __forceinline__ void traverse(const Launch &Lc, const Frame *F) {
                 R += n;
                 __syncwarp();
             }
-            bool any_acc = false;
+            bool any_leaf = false;
 #pragma unroll
-            for (int t = 0; t < W; ++t) any_acc |= V.acc[t] != kNone;
-            if (__any_sync(0xFFFFFFFFu, any_acc)) emit<BATCH, W>(F, wbuf, wfr, cnt, lane, f, j, V.acc);
+            for (int t = 0; t < W; ++t) any_leaf |= V.leaf[t];
+            if (__any_sync(0xFFFFFFFFu, any_leaf)) {
+#pragma unroll
+                for (int t = 0; t < W; ++t) {
+                    const unsigned b = __ballot_sync(0xFFFFFFFFu, V.leaf[t]);
+                    if (V.leaf[t]) queue[queued_n + __popc(b & lt)] = queued(e.x, (uint32_t)t, V.light[t]);
+                    queued_n += __popc(b);
+                }
+                __syncwarp();
+                while (queued_n >= 32u) {
+                    queued_n -= 32u;
+                    take_queued<W>(fr, E, j, lane, queue + queued_n, 32u);
+                }
+            }
         }
+        if (queued_n) take_queued<W>(fr, E, j, lane, queue, queued_n);
         if (lane == 0) {
             uint32_t *ev = frame_at<BATCH>(F, f).eye_visits;
             if (ev) ev[j] = visits;
         }
         visit_acc += visits;
     }
-    if (cnt) flush<BATCH>(F, wbuf, wfr, cnt, lane);
     if (lane == 0 && visit_acc) {
         if constexpr (BATCH) atomicAdd(&frame_at<BATCH>(F, f).counts[1], visit_acc);
         else atomicAdd(&F[0].counts[1], visit_acc);

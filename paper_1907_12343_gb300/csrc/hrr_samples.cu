@@ -147,7 +147,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) cull_samples_kernel(cons
             uint32_t acc = 0;
             for (uint32_t s = 0; s < P.n_samples; ++s) {
                 const uint32_t rs = __shfl_sync(0xFFFFFFFFu, rl, s);
-                if (lane == 0 && hrr_leaf_accepts(__brev(0u) + rs, tau, scale, q0.x, q0.y, q0.z, q0.w, ex, ey, ez))
+                if (lane == 0 && hrr_pair_accepts(__brev(0u) + rs, tau, q0.x, q0.y, q0.z, q0.w, ex, ey, ez))
                     acc |= 1u << s;
             }
             emit(P, wbuf, wsmp, cnt, lane, j, 0u, acc);
@@ -207,17 +207,17 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) cull_samples_kernel(cons
                 const uint32_t rs = __shfl_sync(0xFFFFFFFFu, rl, s), cs = __shfl_sync(0xFFFFFFFFu, cl, s);
                 if (valid && ((e.y >> s) & 1u)) {
                     const uint32_t bit = 1u << s;
-                    if (int0) {
-                        const uint32_t v = hrr_range_min_value(first, split + 1u - first, rs, 0u - rs, cs);
-                        if (!hrr_node_culls(v, den0, rhs0)) mask0 |= bit;
-                    } else if (hrr_leaf_accepts(__brev(split) + rs, tau, scale, q0.x, q0.y, q0.z, q0.w, ex, ey, ez)) {
-                        acc0 |= bit;
+                    // a leaf's minimum is its own value, its box the light: few leaves
+                    // survive the node test, and only those take the exact one
+                    const uint32_t v0 = hrr_range_min_value(first, split + 1u - first, rs, 0u - rs, cs);
+                    if (!hrr_node_culls(v0, den0, rhs0)) {
+                        if (int0) mask0 |= bit;
+                        else if (hrr_pair_accepts(v0, tau, q0.x, q0.y, q0.z, q0.w, ex, ey, ez)) acc0 |= bit;
                     }
-                    if (int1) {
-                        const uint32_t v = hrr_range_min_value(split + 1u, last - split, rs, 0u - rs, cs);
-                        if (!hrr_node_culls(v, den1, rhs1)) mask1 |= bit;
-                    } else if (hrr_leaf_accepts(__brev(last) + rs, tau, scale, q2.x, q2.y, q2.z, q2.w, ex, ey, ez)) {
-                        acc1 |= bit;
+                    const uint32_t v1 = hrr_range_min_value(split + 1u, last - split, rs, 0u - rs, cs);
+                    if (!hrr_node_culls(v1, den1, rhs1)) {
+                        if (int1) mask1 |= bit;
+                        else if (hrr_pair_accepts(v1, tau, q2.x, q2.y, q2.z, q2.w, ex, ey, ez)) acc1 |= bit;
                     }
                 }
             }
