@@ -10,11 +10,10 @@
 //   4. topology_kernel   binary radix tree over (key, sorted position) in parallel: every
 //                        internal node finds its range and split from its neighbours'
 //                        common-prefix lengths (Karras, HPG 2012);
-//   5. refit_kernel      bottom-up boxes / maximum intensities with one atomic counter per
-//                        node (the second child to finish computes the parent), written
-//                        straight into the parent's 64-byte record.
+//   5. the box pass      boxes, maximum intensities and the records (hrr_boxes.cuh).
 #include <algorithm>
 
+#include "hrr_boxes.cuh"
 #include "hrr_internal.cuh"
 
 namespace {
@@ -166,16 +165,24 @@ __global__ void __launch_bounds__(kThreads) radix_scatter_kernel(
     }
 }
 
+// Positions and intensities in leaf order, and the box pass's scratch reset (leaf i's entries
+// by thread i, in place of three memory sets).
+template <bool CHECK>
 __global__ void __launch_bounds__(kThreads) gather_kernel(const float *__restrict__ x,
                                                           const float *__restrict__ y,
                                                           const float *__restrict__ z,
                                                           const float *__restrict__ inten,
                                                           const uint32_t *__restrict__ perm,
-                                                          uint32_t n, float4 *__restrict__ spos) {
+                                                          uint32_t n, float4 *__restrict__ spos,
+                                                          BoxScratch s, unsigned long long *flags) {
     const uint32_t i = blockIdx.x * kThreads + threadIdx.x;
     if (i >= n) return;
     const uint32_t v = perm[i];
-    spos[i] = make_float4(x[v], y[v], z[v], inten[v]);
+    const float4 p = make_float4(x[v], y[v], z[v], inten[v]);
+    if (CHECK && (!isfinite(p.x) || !isfinite(p.y) || !isfinite(p.z) || !isfinite(p.w)))
+        atomicOr(flags, HRR_FLAG_NONFINITE);
+    spos[i] = p;
+    box_reset(s, i, n);
 }
 
 // Common-prefix length of the ordering keys (Morton key, sorted position) of leaves i, j;
@@ -225,65 +232,10 @@ __device__ __forceinline__ void store_slot(hrr_node *node, uint32_t slot, const 
     f[4] = hi[0]; f[5] = hi[1]; f[6] = hi[2];
 }
 
-__global__ void __launch_bounds__(kThreads) refit_kernel(const float4 *__restrict__ spos,
-                                                         uint32_t n, hrr_node *nodes,
-                                                         const uint32_t *__restrict__ leaf_parent,
-                                                         const uint32_t *__restrict__ int_parent,
-                                                         uint32_t *arrivals, uint32_t *child_height,
-                                                         uint32_t *root_height,
-                                                         unsigned long long *flags) {
-    const uint32_t leaf = blockIdx.x * kThreads + threadIdx.x;
-    if (leaf >= n || (*(volatile unsigned long long *)flags & HRR_FLAG_NONFINITE)) return;
-    const float4 p = spos[leaf];
-    float lo[3] = {p.x, p.y, p.z}, hi[3] = {p.x, p.y, p.z};
-    float imax = p.w;
-    uint32_t h = 0;
-    uint32_t code = leaf_parent[leaf];
-    for (;;) {
-        const uint32_t node = code >> 1, slot = code & 1u;
-        if (code == 0xFFFFFFFFu || node >= n - 1) {  // every link is set by topology_kernel
-            atomicOr(flags, HRR_FLAG_TOPOLOGY);
-            return;
-        }
-        store_slot(&nodes[node], slot, lo, hi, imax);
-        child_height[2ull * node + slot] = h;
-        __threadfence();
-        if (atomicAdd(&arrivals[node], 1u) == 0u) return;  // the sibling finishes the node
-        __threadfence();
-        const float *f = reinterpret_cast<const float *>(&nodes[node]);
-        for (int c = 0; c < 3; ++c) {
-            lo[c] = fminf(__ldcg(f + c), __ldcg(f + 8 + c));
-            hi[c] = fmaxf(__ldcg(f + 4 + c), __ldcg(f + 12 + c));
-        }
-        imax = fmaxf(__ldcg(f + 3), __ldcg(f + 11));
-        h = 1u + max(__ldcg(&child_height[2ull * node]), __ldcg(&child_height[2ull * node + 1]));
-        if (node == 0) {
-            *root_height = h;
-            return;
-        }
-        code = int_parent[node];
-    }
-}
-
 // Refit for moved lights: the leaves keep their order, so gather the new positions into
 // that order (flagging non-finite values), rebuild the parent links from the records, and
-// run refit_kernel again. The last two skip their work when the gather raised a flag, so
+// run the box pass again. The later ones skip their work when the gather raised a flag, so
 // the hierarchy is left as it was.
-__global__ void __launch_bounds__(kThreads) gather_check_kernel(const float *__restrict__ x,
-                                                                const float *__restrict__ y,
-                                                                const float *__restrict__ z,
-                                                                const float *__restrict__ inten,
-                                                                const uint32_t *__restrict__ perm,
-                                                                uint32_t n, float4 *__restrict__ spos,
-                                                                unsigned long long *flags) {
-    const uint32_t i = blockIdx.x * kThreads + threadIdx.x;
-    if (i >= n) return;
-    const uint32_t v = perm[i];
-    const float4 p = make_float4(x[v], y[v], z[v], inten[v]);
-    if (!isfinite(p.x) || !isfinite(p.y) || !isfinite(p.z) || !isfinite(p.w)) atomicOr(flags, HRR_FLAG_NONFINITE);
-    spos[i] = p;
-}
-
 __global__ void __launch_bounds__(kThreads) links_kernel(const hrr_node *__restrict__ nodes, uint32_t n,
                                                          uint32_t *__restrict__ leaf_parent,
                                                          uint32_t *__restrict__ int_parent,
@@ -301,8 +253,10 @@ __global__ void __launch_bounds__(kThreads) links_kernel(const hrr_node *__restr
     if (last == s + 1) leaf_parent[s + 1] = code | 1u; else int_parent[s + 1] = code | 1u;
 }
 
+// The hierarchy of one light: its record, its permutation and (with `wide`) the records derived
+// from it: the leaf in slot 0 of the width-four record, the rest and the top slots empty.
 __global__ void single_leaf_kernel(const float *x, const float *y, const float *z,
-                                   const float *inten, hrr_node *node, uint32_t *perm,
+                                   const float *inten, hrr_node *node, uint32_t *perm, float4 *wide,
                                    unsigned long long *flags) {
     const float px = x[0], py = y[0], pz = z[0], w = inten[0];
     if (!isfinite(px) || !isfinite(py) || !isfinite(pz) || !isfinite(w)) {
@@ -315,121 +269,10 @@ __global__ void single_leaf_kernel(const float *x, const float *y, const float *
     node->split = 0;
     node->other_end = 0;
     perm[0] = 0;
-}
-
-// The top slots (HRR_TOP_SLOTS of them, layout in hrr_internal.cuh): thread s walks from the
-// root along the path of heap slot s (the bits of s + 1 below its leading one, high to low:
-// 0 = child 0, 1 = child 1), taking each child's box and maximum intensity from its parent's
-// record. A slot below a leaf is empty; a record whose split is outside its node's range
-// (not produced by the builder) empties the slots below it.
-__global__ void __launch_bounds__(64) top_kernel(const float4 *__restrict__ nodes, uint32_t n,
-                                                 float4 *__restrict__ top, const unsigned long long *flags) {
-    const uint32_t s = threadIdx.x;
-    if (s >= HRR_TOP_SLOTS) return;
-    if (*(volatile const unsigned long long *)flags & HRR_FLAG_NONFINITE) return;
-    float4 lo = make_float4(0.f, 0.f, 0.f, 0.f), hi = lo;
-    uint32_t first = 0, last = 0, node = 0, kind = HRR_TOP_EMPTY;
-    if (n > 1) {
-        const uint32_t path = s + 1u;
-        kind = HRR_TOP_INTERNAL;
-        last = __float_as_uint(nodes[3].w);  // the root's range is [0, its other end]
-        for (int b = 30 - __clz(path); b >= 0; --b) {
-            if (kind != HRR_TOP_INTERNAL) {
-                kind = HRR_TOP_EMPTY;
-                break;
-            }
-            const float4 *r = nodes + 4 * (size_t)node;
-            const uint32_t split = __float_as_uint(r[1].w);
-            if (last >= n || split < first || split >= last) {
-                kind = HRR_TOP_EMPTY;
-                break;
-            }
-            if (((path >> b) & 1u) == 0u) {
-                lo = r[0];
-                hi = r[1];
-                last = split;
-                node = split;
-            } else {
-                lo = r[2];
-                hi = r[3];
-                first = split + 1u;
-                node = split + 1u;
-            }
-            kind = first == last ? HRR_TOP_LEAF : HRR_TOP_INTERNAL;
-        }
-    }
-    if (kind == HRR_TOP_EMPTY) {
-        lo = hi = make_float4(0.f, 0.f, 0.f, 0.f);
-        first = last = node = 0;
-    }
-    top[3 * s] = lo;
-    top[3 * s + 1] = make_float4(hi.x, hi.y, hi.z, __uint_as_float(first));
-    top[3 * s + 2] = make_float4(__uint_as_float(last), __uint_as_float(node), __uint_as_float(kind), 0.f);
-}
-
-// Records of width four. The record of internal node g holds, in this order, the slots of
-// g's grandchildren over its leaf range [first, last] split at `split`:
-//   slot 0: [first, s0]      slot 1: [s0 + 1, split]     (the children of child 0)
-//   slot 2: [split + 1, s1]  slot 3: [s1 + 1, last]      (the children of child 1)
-// each 32 bytes: box low corner, maximum intensity, box high corner, and one index word
-// (s0, split, s1 and g's other range end, in slot order). A child that is a leaf takes its
-// first slot as itself (s0 = split, or s1 = last) and leaves the second slot empty (an
-// empty range). The internal slots are binary nodes s0, s0 + 1, s1, s1 + 1, whose own
-// records sit at those indices. Since a node's record is the first 32 bytes of its
-// children's binary records, re-labelled, the widening is a gather of the binary records.
-__global__ void __launch_bounds__(kThreads) widen_kernel(const float4 *__restrict__ nodes, uint32_t n,
-                                                         float4 *__restrict__ wide,
-                                                         const unsigned long long *flags) {
-    const uint32_t g = blockIdx.x * kThreads + threadIdx.x;
-    if (*(volatile const unsigned long long *)flags & HRR_FLAG_NONFINITE) return;
-    if (n == 1) {  // the single leaf in slot 0, the rest empty
-        if (g == 0) {
-            wide[0] = nodes[0];
-            wide[1] = nodes[1];
-            for (int k = 2; k < 8; ++k) wide[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-        return;
-    }
-    if (g >= n - 1) return;
-    const float4 *r = nodes + 4 * (size_t)g;
-    const float4 c0l = r[0], c0h = r[1], c1l = r[2], c1h = r[3];
-    const uint32_t split = __float_as_uint(c0h.w), other = __float_as_uint(c1h.w);
-    const uint32_t first = min(g, other), last = max(g, other);
-    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-    float4 *w = wide + 8 * (size_t)g;
-    if (first == split) {  // child 0 is a leaf: slot 0 is the leaf, slot 1 empty
-        w[0] = c0l;
-        w[1] = make_float4(c0h.x, c0h.y, c0h.z, __uint_as_float(split));
-        w[2] = zero;
-        w[3] = make_float4(0.f, 0.f, 0.f, __uint_as_float(split));
-    } else {  // the children of internal node `split`
-        const float4 *a = nodes + 4 * (size_t)split;
-        w[0] = a[0];
-        w[1] = a[1];  // its .w is the child's split, s0
-        w[2] = a[2];
-        const float4 h = a[3];
-        w[3] = make_float4(h.x, h.y, h.z, __uint_as_float(split));
-    }
-    if (split + 1u == last) {  // child 1 is a leaf
-        w[4] = c1l;
-        w[5] = make_float4(c1h.x, c1h.y, c1h.z, __uint_as_float(last));
-        w[6] = zero;
-        w[7] = make_float4(0.f, 0.f, 0.f, __uint_as_float(other));
-    } else {  // the children of internal node split + 1
-        const float4 *b = nodes + 4 * (size_t)(split + 1u);
-        w[4] = b[0];
-        w[5] = b[1];  // s1
-        w[6] = b[2];
-        const float4 h = b[3];
-        w[7] = make_float4(h.x, h.y, h.z, __uint_as_float(other));
-    }
-}
-
-template <typename T>
-T *carve(char *&p, size_t count) {
-    T *r = reinterpret_cast<T *>(p);
-    p += (sizeof(T) * count + 255) & ~size_t(255);
-    return r;
+    if (!wide) return;
+    const float4 *r = reinterpret_cast<const float4 *>(node);
+    for (int k = 0; k < 8; ++k) wide[k] = k < 2 ? r[k] : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (uint32_t k = 0; k < 3 * HRR_TOP_SLOTS; ++k) reinterpret_cast<float4 *>(node)[4 + k] = wide[2];
 }
 
 // ------------------------------------------------------------------------------------
@@ -445,7 +288,7 @@ T *carve(char *&p, size_t count) {
 // correctly rounded). A non-finite C never wins; ties go to the least |c_L - c_R|, then
 // the least k. Ranges deeper than the cost depth (root = 1)
 // take the radix split, which bounds the height. Node numbering and parent links are those
-// of topology_kernel, so refit_kernel finishes the hierarchy unchanged.
+// of topology_kernel, so the box pass finishes the hierarchy unchanged.
 //
 // Boxes and maxima are min / max reductions, exact in any order, so parallel scans give
 // the same prefix and suffix aggregates at every k as a serial sweep, and the same costs
@@ -1031,7 +874,7 @@ int hrr_build_impl(hrr_ctx *ctx, const hrr_lights &L, uint32_t n, hrr_tree **out
         return fail(hrr_cuda_fail(ctx, e, "flag reset"));
 
     if (n == 1) {
-        single_leaf_kernel<<<1, 1, 0, st>>>(L.x, L.y, L.z, L.intensity, tree->nodes, tree->perm, flags);
+        single_leaf_kernel<<<1, 1, 0, st>>>(L.x, L.y, L.z, L.intensity, tree->nodes, tree->perm, tree->wide, flags);
         ++ctx->launches;
         if ((e = cudaGetLastError()) != cudaSuccess) return fail(hrr_cuda_fail(ctx, e, "single_leaf_kernel"));
         tree->height = 0;
@@ -1041,10 +884,7 @@ int hrr_build_impl(hrr_ctx *ctx, const hrr_lights &L, uint32_t n, hrr_tree **out
         const size_t bytes = 2 * ((sizeof(uint64_t) * (size_t)n + 255) & ~size_t(255)) +
                              ((sizeof(uint32_t) * (size_t)n + 255) & ~size_t(255)) +
                              ((sizeof(uint32_t) * hist_n + 255) & ~size_t(255)) +
-                             ((sizeof(float4) * (size_t)n + 255) & ~size_t(255)) +
-                             2 * ((sizeof(uint32_t) * (size_t)n + 255) & ~size_t(255)) +
-                             ((sizeof(uint32_t) * (size_t)n + 255) & ~size_t(255)) +
-                             ((sizeof(uint32_t) * 2 * (size_t)n + 255) & ~size_t(255)) + 256 + 1024;
+                             ((sizeof(float4) * (size_t)n + 255) & ~size_t(255)) + box_scratch_bytes(n);
         char *scratch = nullptr;
         if ((e = cudaMallocAsync(&scratch, bytes, st)) != cudaSuccess) return fail(hrr_cuda_fail(ctx, e, "build scratch"));
         char *p = scratch;
@@ -1052,10 +892,7 @@ int hrr_build_impl(hrr_ctx *ctx, const hrr_lights &L, uint32_t n, hrr_tree **out
         uint32_t *vals1 = carve<uint32_t>(p, n);
         uint32_t *hist = carve<uint32_t>(p, hist_n);
         float4 *spos = carve<float4>(p, n);
-        uint32_t *leaf_parent = carve<uint32_t>(p, n), *int_parent = carve<uint32_t>(p, n);
-        uint32_t *arrivals = carve<uint32_t>(p, n);
-        uint32_t *child_height = carve<uint32_t>(p, 2 * (size_t)n);
-        uint32_t *root_height = carve<uint32_t>(p, 1);
+        const BoxScratch rs = carve_boxes(p, n);
         uint32_t *vals0 = tree->perm;
 
         const unsigned g = (n + kThreads - 1) / kThreads;
@@ -1075,29 +912,23 @@ int hrr_build_impl(hrr_ctx *ctx, const hrr_lights &L, uint32_t n, hrr_tree **out
                 uint32_t *tv = vin; vin = vout; vout = tv;
             }
             // eight passes: the sorted keys are back in keys0 and the permutation in vals0
-            gather_kernel<<<g, kThreads, 0, st>>>(L.x, L.y, L.z, L.intensity, vals0, n, spos);
-            if ((e = cudaMemsetAsync(arrivals, 0, sizeof(uint32_t) * (size_t)n, st)) != cudaSuccess) { rc = hrr_cuda_fail(ctx, e, "memset"); break; }
-            if ((e = cudaMemsetAsync(leaf_parent, 0xFF, 2 * ((sizeof(uint32_t) * (size_t)n + 255) & ~size_t(255)), st)) != cudaSuccess) { rc = hrr_cuda_fail(ctx, e, "memset"); break; }
+            gather_kernel<false><<<g, kThreads, 0, st>>>(L.x, L.y, L.z, L.intensity, vals0, n, spos, rs, flags);
             const unsigned gi = (n - 1 + kThreads - 1) / kThreads;
             if (topology == HRR_TOPOLOGY_COST) {
-                if ((rc = cost_topology(ctx, spos, keys0, n, cost_depth, tree->nodes, leaf_parent, int_parent, st)) != HRR_OK) break;
+                if ((rc = cost_topology(ctx, spos, keys0, n, cost_depth, tree->nodes, rs.leaf_parent, rs.int_parent, st)) != HRR_OK) break;
             } else {
-                topology_kernel<<<gi, kThreads, 0, st>>>(keys0, n, tree->nodes, leaf_parent, int_parent);
+                topology_kernel<<<gi, kThreads, 0, st>>>(keys0, n, tree->nodes, rs.leaf_parent, rs.int_parent);
                 ++ctx->launches;
             }
-            refit_kernel<<<g, kThreads, 0, st>>>(spos, n, tree->nodes, leaf_parent, int_parent, arrivals,
-                                                 child_height, root_height, flags);
-            ctx->launches += 2;
+            boxes_enqueue(PointLeaves{spos}, n, tree->nodes, tree->wide, rs, flags, st);
+            ctx->launches += 3;
             if ((e = cudaGetLastError()) != cudaSuccess) { rc = hrr_cuda_fail(ctx, e, "build kernels"); break; }
-            if ((e = cudaMemcpyAsync(&ctx->host_counters[4], root_height, sizeof(uint32_t),
+            if ((e = cudaMemcpyAsync(&ctx->host_counters[4], rs.root_height, sizeof(uint32_t),
                                      cudaMemcpyDeviceToHost, st)) != cudaSuccess) { rc = hrr_cuda_fail(ctx, e, "height copy"); break; }
         } while (0);
         cudaFreeAsync(scratch, st);
         if (rc != HRR_OK) return fail(rc);
     }
-    if ((e = hrr_derived_enqueue(tree, flags, st)) != cudaSuccess)
-        return fail(hrr_cuda_fail(ctx, e, "top and widen kernels"));
-    ctx->launches += hrr_derived_launches(tree);
     if ((e = cudaMemcpyAsync(&ctx->host_counters[2], flags, sizeof(unsigned long long), cudaMemcpyDeviceToHost, st)) != cudaSuccess)
         return fail(hrr_cuda_fail(ctx, e, "flag copy"));
     if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return fail(hrr_cuda_fail(ctx, e, "build"));
@@ -1114,50 +945,23 @@ int hrr_build_impl(hrr_ctx *ctx, const hrr_lights &L, uint32_t n, hrr_tree **out
 // Refit for moved lights
 // ------------------------------------------------------------------------------------
 
-size_t hrr_refit_scratch_bytes(uint32_t n) {
-    const size_t un = (size_t)n;
-    return ((sizeof(float4) * un + 255) & ~size_t(255)) + 2 * ((sizeof(uint32_t) * un + 255) & ~size_t(255)) +
-           ((sizeof(uint32_t) * un + 255) & ~size_t(255)) + ((sizeof(uint32_t) * 2 * un + 255) & ~size_t(255)) +
-           256 + 1024;
-}
+size_t hrr_refit_scratch_bytes(uint32_t n) { return pad256(sizeof(float4) * (size_t)n) + box_scratch_bytes(n); }
 
 cudaError_t hrr_refit_enqueue(hrr_tree *tree, const hrr_lights &L, void *scratch_mem, unsigned long long *flags,
                               cudaStream_t st) {
     const uint32_t n = tree->n;
+    // one leaf: rewrite the single record unless the light is not finite (checked there)
     if (n == 1) {
-        // one leaf: rewrite the single record unless the light is not finite (checked there)
-        single_leaf_kernel<<<1, 1, 0, st>>>(L.x, L.y, L.z, L.intensity, tree->nodes, tree->perm, flags);
-        const cudaError_t e = cudaGetLastError();
-        return e == cudaSuccess ? hrr_derived_enqueue(tree, flags, st) : e;
+        single_leaf_kernel<<<1, 1, 0, st>>>(L.x, L.y, L.z, L.intensity, tree->nodes, tree->perm, tree->wide, flags);
+        return cudaGetLastError();
     }
     char *p = static_cast<char *>(scratch_mem);
     float4 *spos = carve<float4>(p, n);
-    uint32_t *leaf_parent = carve<uint32_t>(p, n), *int_parent = carve<uint32_t>(p, n);
-    uint32_t *arrivals = carve<uint32_t>(p, n);
-    uint32_t *child_height = carve<uint32_t>(p, 2 * (size_t)n);
-    uint32_t *root_height = carve<uint32_t>(p, 1);
+    const BoxScratch rs = carve_boxes(p, n);
     const unsigned g = (n + kThreads - 1) / kThreads, gi = (n - 1 + kThreads - 1) / kThreads;
-    gather_check_kernel<<<g, kThreads, 0, st>>>(L.x, L.y, L.z, L.intensity, tree->perm, n, spos, flags);
-    cudaError_t e = cudaMemsetAsync(arrivals, 0, sizeof(uint32_t) * (size_t)n, st);
-    if (e == cudaSuccess)
-        e = cudaMemsetAsync(leaf_parent, 0xFF, 2 * ((sizeof(uint32_t) * (size_t)n + 255) & ~size_t(255)), st);
-    if (e != cudaSuccess) return e;
-    links_kernel<<<gi, kThreads, 0, st>>>(tree->nodes, n, leaf_parent, int_parent, flags);
-    refit_kernel<<<g, kThreads, 0, st>>>(spos, n, tree->nodes, leaf_parent, int_parent, arrivals, child_height,
-                                         root_height, flags);
-    e = cudaGetLastError();
-    return e == cudaSuccess ? hrr_derived_enqueue(tree, flags, st) : e;
-}
-
-cudaError_t hrr_derived_enqueue(hrr_tree *tree, const unsigned long long *flags, cudaStream_t st) {
-    const uint32_t n = tree->n;
-    const float4 *nodes = reinterpret_cast<const float4 *>(tree->nodes);
-    const size_t n_rec = n > 1 ? n - 1 : 1;
-    top_kernel<<<1, 64, 0, st>>>(nodes, n, reinterpret_cast<float4 *>(tree->nodes) + 4 * n_rec, flags);
-    if (!tree->wide) return cudaGetLastError();
-    const unsigned g = n > 1 ? (n - 1 + kThreads - 1) / kThreads : 1;
-    widen_kernel<<<g, kThreads, 0, st>>>(nodes, n, tree->wide, flags);
-    return cudaGetLastError();
+    gather_kernel<true><<<g, kThreads, 0, st>>>(L.x, L.y, L.z, L.intensity, tree->perm, n, spos, rs, flags);
+    links_kernel<<<gi, kThreads, 0, st>>>(tree->nodes, n, rs.leaf_parent, rs.int_parent, flags);
+    return boxes_enqueue(PointLeaves{spos}, n, tree->nodes, tree->wide, rs, flags, st);
 }
 
 // ------------------------------------------------------------------------------------
@@ -1177,17 +981,12 @@ namespace {
 
 constexpr uint32_t kStaticMaxLights = HRR_STATIC_BUILD_MAX_LIGHTS;
 
-constexpr size_t pad256(size_t b) { return (b + 255) & ~size_t(255); }
-
 constexpr size_t static_scratch_bytes(size_t n) {
     return 2 * pad256(sizeof(uint64_t) * n)                               // keys, ping-pong
            + pad256(sizeof(uint32_t) * n)                                 // second value buffer
            + pad256(sizeof(uint32_t) * 256 * ((n + kTile - 1) / kTile + 1)) // digit histograms, totals
            + pad256(sizeof(float4) * n)                                   // sorted lights
-           + 2 * pad256(sizeof(uint32_t) * n)                             // parent links
-           + pad256(sizeof(uint32_t) * n)                                 // arrival counters
-           + pad256(sizeof(uint32_t) * 2 * n)                             // child heights
-           + pad256(sizeof(uint32_t))                                     // root height
+           + box_scratch_bytes((uint32_t)n)                               // box pass
            + pad256(sizeof(unsigned long long));                          // error flags
 }
 
@@ -1245,25 +1044,19 @@ extern "C" int hrr_build_light_tree_static(hrr_lights L, uint32_t n, hrr_node *d
     uint32_t *vals1 = carve<uint32_t>(p, kStaticMaxLights);
     uint32_t *hist = carve<uint32_t>(p, 256 * ((kStaticMaxLights + kTile - 1) / kTile + 1));
     float4 *spos = carve<float4>(p, kStaticMaxLights);
-    uint32_t *leaf_parent = carve<uint32_t>(p, kStaticMaxLights), *int_parent = carve<uint32_t>(p, kStaticMaxLights);
-    uint32_t *arrivals = carve<uint32_t>(p, kStaticMaxLights);
-    uint32_t *child_height = carve<uint32_t>(p, 2 * (size_t)kStaticMaxLights);
-    uint32_t *root_height = carve<uint32_t>(p, 1);
+    const BoxScratch rs = carve_boxes(p, kStaticMaxLights);
     unsigned long long *flags = carve<unsigned long long>(p, 1);
 
     // Every call reuses the array: clear what the kernels expect to start cleared.
     e = cudaMemsetAsync(flags, 0, sizeof(unsigned long long), st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(root_height, 0, sizeof(uint32_t), st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(rs.root_height, 0, sizeof(uint32_t), st);
     if (n == 1) {
         if (e == cudaSuccess) {
-            single_leaf_kernel<<<1, 1, 0, st>>>(L.x, L.y, L.z, L.intensity, dev_nodes, dev_perm, flags);
+            single_leaf_kernel<<<1, 1, 0, st>>>(L.x, L.y, L.z, L.intensity, dev_nodes, dev_perm, nullptr, flags);
             e = cudaGetLastError();
         }
     } else {
         const uint32_t nblocks = (n + kTile - 1) / kTile;
-        if (e == cudaSuccess) e = cudaMemsetAsync(arrivals, 0, sizeof(uint32_t) * (size_t)n, st);
-        if (e == cudaSuccess) e = cudaMemsetAsync(leaf_parent, 0xFF, sizeof(uint32_t) * (size_t)n, st);
-        if (e == cudaSuccess) e = cudaMemsetAsync(int_parent, 0xFF, sizeof(uint32_t) * (size_t)n, st);
         if (e == cudaSuccess) {
             const unsigned g = (n + kThreads - 1) / kThreads;
             morton_kernel<<<g, kThreads, 0, st>>>(L.x, L.y, L.z, L.intensity, n, keys0, dev_perm, flags);
@@ -1277,17 +1070,16 @@ extern "C" int hrr_build_light_tree_static(hrr_lights L, uint32_t n, hrr_node *d
                 uint64_t *tk = kin; kin = kout; kout = tk;
                 uint32_t *tv = vin; vin = vout; vout = tv;
             }
-            gather_kernel<<<g, kThreads, 0, st>>>(L.x, L.y, L.z, L.intensity, dev_perm, n, spos);
+            gather_kernel<false><<<g, kThreads, 0, st>>>(L.x, L.y, L.z, L.intensity, dev_perm, n, spos, rs, flags);
             const unsigned gi = (n - 1 + kThreads - 1) / kThreads;
-            topology_kernel<<<gi, kThreads, 0, st>>>(keys0, n, dev_nodes, leaf_parent, int_parent);
-            refit_kernel<<<g, kThreads, 0, st>>>(spos, n, dev_nodes, leaf_parent, int_parent, arrivals,
-                                                 child_height, root_height, flags);
+            topology_kernel<<<gi, kThreads, 0, st>>>(keys0, n, dev_nodes, rs.leaf_parent, rs.int_parent);
+            boxes_enqueue(PointLeaves{spos}, n, dev_nodes, nullptr, rs, flags, st);
             e = cudaGetLastError();
         }
     }
     uint32_t height = 0;
     unsigned long long host_flags = 0;
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&height, root_height, sizeof height, cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&height, rs.root_height, sizeof height, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&host_flags, flags, sizeof host_flags, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) {

@@ -100,20 +100,14 @@ struct hrr_tree {
     hrr_node *nodes = nullptr;
     uint32_t *perm = nullptr;   // n
     // The same hierarchy read with nodes of width four: for every internal node g a
-    // 128-byte record of its four grandchild slots (hrr_derived_enqueue), at index g; a
+    // 128-byte record of its four grandchild slots (hrr_build.cu), at index g; a
     // traversal of width four reads the even-depth ones only. One record (the leaf in
     // slot 0) when n == 1.
     float4 *wide = nullptr;
 };
 
-// Fill the records derived from the binary ones: the top slots after tree->nodes, and
-// tree->wide if the tree has it (one thread per internal node); skipped when *flags holds
-// HRR_FLAG_NONFINITE (a failed refit leaves the hierarchy as it was).
-cudaError_t hrr_derived_enqueue(hrr_tree *tree, const unsigned long long *flags, cudaStream_t st);
-// Kernels hrr_derived_enqueue launches for the tree.
-inline int hrr_derived_launches(const hrr_tree *tree) { return tree->wide ? 2 : 1; }
 // Kernels a refit launches (hrr_refit_enqueue).
-inline int hrr_refit_launches(const hrr_tree *tree) { return (tree->n > 1 ? 3 : 1) + hrr_derived_launches(tree); }
+inline int hrr_refit_launches(const hrr_tree *tree) { return tree->n > 1 ? 4 : 1; }
 
 // Layer (sample mod d) of a w x h x d tile: the shifts one culling pass uses.
 inline const uint32_t *hrr_tile_layer(const uint32_t *tile, uint32_t w, uint32_t h, uint32_t d,
