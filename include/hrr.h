@@ -154,7 +154,9 @@ int hrr_default_tuning(hrr_tuning *out);
 
 /* Create a context on CUDA device `device`. cuda_stream is a cudaStream_t on that device
  * (for example torch.cuda.current_stream().cuda_stream) or NULL for a stream owned by the
- * context. Allocates a few bytes of device counters and pinned host memory. */
+ * context. Allocates a few bytes of device counters and pinned host memory. Hierarchies,
+ * scenes and the working memory of builds and refits come from a memory pool of the context,
+ * which keeps up to 2 GiB of what was freed for the next ones, until hrr_destroy. */
 int hrr_create(hrr_ctx **out, int device, void *cuda_stream);
 /* Waits for the context stream, then releases the context (not trees built with it). */
 int hrr_destroy(hrr_ctx *ctx);

@@ -18,6 +18,31 @@ int hrr_cuda_fail(hrr_ctx *ctx, cudaError_t e, const char *what) {
     return hrr_fail(ctx, st, m);
 }
 
+cudaError_t hrr_alloc_bytes(hrr_ctx *ctx, void **p, size_t bytes) {
+    *p = nullptr;
+    cudaError_t e = cudaSuccess;
+    if (!ctx->pool) {
+        cudaMemPoolProps props = {};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = ctx->device;
+        if ((e = cudaMemPoolCreate(&ctx->pool, &props)) != cudaSuccess) {
+            ctx->pool = nullptr;
+            return e;
+        }
+        uint64_t keep = HRR_POOL_KEEP;
+        if ((e = cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &keep)) != cudaSuccess) return e;
+    }
+    e = cudaMallocFromPoolAsync(p, bytes, ctx->pool, ctx->stream);
+    if (e == cudaErrorMemoryAllocation) {  // idle memory of the wrong sizes: give it back and try once more
+        cudaGetLastError();
+        *p = nullptr;
+        if ((e = cudaStreamSynchronize(ctx->stream)) == cudaSuccess && (e = cudaMemPoolTrimTo(ctx->pool, 0)) == cudaSuccess)
+            e = cudaMallocFromPoolAsync(p, bytes, ctx->pool, ctx->stream);
+    }
+    return e;
+}
+
 void hrr_timing_begin(hrr_ctx *ctx) {
     if (!ctx->timing) return;
     cudaEvent_t a, b;
@@ -129,6 +154,7 @@ int hrr_destroy(hrr_ctx *ctx) {
     if (ctx->host_slices) cudaFreeHost(ctx->host_slices);
     if (ctx->copy_stream) cudaStreamDestroy(ctx->copy_stream);
     if (ctx->stream2) cudaStreamDestroy(ctx->stream2);
+    if (ctx->pool) cudaMemPoolDestroy(ctx->pool);
     if (ctx->own_stream && ctx->stream) cudaStreamDestroy(ctx->stream);
     delete ctx;
     return HRR_OK;
@@ -201,7 +227,7 @@ int hrr_build_light_tree_host(hrr_ctx *ctx, hrr_lights H, uint32_t n_lights, con
         if (ctx->host_lights_dev) cudaFree(ctx->host_lights_dev);
         ctx->host_lights_dev = nullptr;
         ctx->host_lights_cap = 0;
-        if (cudaMalloc(&ctx->host_lights_dev, 4 * sizeof(float) * stride) != cudaSuccess) {
+        if (hrr_malloc(ctx, &ctx->host_lights_dev, 4 * sizeof(float) * stride) != cudaSuccess) {
             cudaGetLastError();
             return hrr_fail(ctx, HRR_ERR_OOM, "device staging area of the lights");
         }
@@ -266,7 +292,7 @@ int hrr_refit_light_tree(hrr_ctx *ctx, hrr_tree *tree, hrr_lights lights) {
     unsigned long long *flags = ctx->counters + 2;
     HRR_CUDA(ctx, cudaMemsetAsync(flags, 0, sizeof(unsigned long long), st));
     void *scratch = nullptr;
-    HRR_CUDA(ctx, cudaMallocAsync(&scratch, hrr_refit_scratch_bytes(tree->n), st));
+    HRR_CUDA(ctx, hrr_alloc(ctx, &scratch, hrr_refit_scratch_bytes(tree->n)));
     const cudaError_t e = hrr_refit_enqueue(tree, lights, scratch, flags, st);
     ctx->launches += hrr_refit_launches(tree);
     cudaFreeAsync(scratch, st);
@@ -287,7 +313,7 @@ int hrr_set_shift_tile_3d(hrr_ctx *ctx, const uint32_t *host_tile, uint32_t w, u
     DeviceGuard g(ctx->device);
     const size_t bytes = sizeof(uint32_t) * (size_t)w * h * d;
     uint32_t *dev = nullptr;
-    HRR_CUDA(ctx, cudaMallocAsync(&dev, bytes, ctx->stream));
+    HRR_CUDA(ctx, hrr_alloc(ctx, &dev, bytes));
     cudaError_t e = cudaMemcpyAsync(dev, host_tile, bytes, cudaMemcpyHostToDevice, ctx->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
     if (e != cudaSuccess) {

@@ -181,8 +181,8 @@ int hrr_batch_create(hrr_ctx *ctx, const hrr_frame *frames, uint32_t n_frames, c
     }
     b->spill_cap = hrr_cull_spill_cap(height, b->tuning.node_width);
     const size_t spill_bytes = hrr_cull_spill_entries(grid_max, height, b->tuning) * sizeof(uint2);
-    cudaError_t e = cudaMalloc(&b->spill[0], spill_bytes);
-    if (e == cudaSuccess && b->parts.size() > 1) e = cudaMalloc(&b->spill[1], spill_bytes);
+    cudaError_t e = hrr_malloc(ctx, &b->spill[0], spill_bytes);
+    if (e == cudaSuccess && b->parts.size() > 1) e = hrr_malloc(ctx, &b->spill[1], spill_bytes);
     if (e == cudaSuccess && b->parts.size() > 1) e = cudaStreamCreateWithFlags(&b->side, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->join, cudaEventDisableTiming);

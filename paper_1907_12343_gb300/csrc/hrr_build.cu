@@ -769,7 +769,7 @@ int cost_topology(hrr_ctx *ctx, const float4 *spos, const uint64_t *keys, uint32
                          3 * rup(sizeof(AggRec) * cap_t) + rup(sizeof(Best) * cap_t) + rup(sizeof(uint32_t) * cap_b) +
                          256;
     char *scratch = nullptr;
-    cudaError_t e = cudaMallocAsync(&scratch, bytes, st);
+    cudaError_t e = hrr_alloc(ctx, &scratch, bytes);
     if (e != cudaSuccess) return hrr_cuda_fail(ctx, e, "topology scratch");
     struct Lists {
         Seg *small, *radix_end, *mid, *big;
@@ -865,9 +865,9 @@ int hrr_build_impl(hrr_ctx *ctx, const hrr_lights &L, uint32_t n, hrr_tree **out
         return status;
     };
     const uint32_t n_rec = n > 1 ? n - 1 : 1;
-    cudaError_t e = cudaMallocAsync(&tree->nodes, sizeof(hrr_node) * (size_t)n_rec + HRR_TOP_BYTES, st);
-    if (e == cudaSuccess) e = cudaMallocAsync(&tree->perm, sizeof(uint32_t) * (size_t)n, st);
-    if (e == cudaSuccess) e = cudaMallocAsync(&tree->wide, 8 * sizeof(float4) * (size_t)n_rec, st);
+    cudaError_t e = hrr_alloc(ctx, &tree->nodes, sizeof(hrr_node) * (size_t)n_rec + HRR_TOP_BYTES);
+    if (e == cudaSuccess) e = hrr_alloc(ctx, &tree->perm, sizeof(uint32_t) * (size_t)n);
+    if (e == cudaSuccess) e = hrr_alloc(ctx, &tree->wide, 8 * sizeof(float4) * (size_t)n_rec);
     if (e != cudaSuccess) return fail(hrr_cuda_fail(ctx, e, "tree allocation"));
     unsigned long long *flags = ctx->counters + 2;
     if ((e = cudaMemsetAsync(flags, 0, sizeof(unsigned long long), st)) != cudaSuccess)
@@ -886,7 +886,7 @@ int hrr_build_impl(hrr_ctx *ctx, const hrr_lights &L, uint32_t n, hrr_tree **out
                              ((sizeof(uint32_t) * hist_n + 255) & ~size_t(255)) +
                              ((sizeof(float4) * (size_t)n + 255) & ~size_t(255)) + box_scratch_bytes(n);
         char *scratch = nullptr;
-        if ((e = cudaMallocAsync(&scratch, bytes, st)) != cudaSuccess) return fail(hrr_cuda_fail(ctx, e, "build scratch"));
+        if ((e = hrr_alloc(ctx, &scratch, bytes)) != cudaSuccess) return fail(hrr_cuda_fail(ctx, e, "build scratch"));
         char *p = scratch;
         uint64_t *keys0 = carve<uint64_t>(p, n), *keys1 = carve<uint64_t>(p, n);
         uint32_t *vals1 = carve<uint32_t>(p, n);

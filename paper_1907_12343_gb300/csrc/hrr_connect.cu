@@ -348,7 +348,7 @@ int hrr_build_scene(hrr_ctx *ctx, const float *dev_tris, uint32_t n_tris, hrr_sc
     unsigned long long *flags = ctx->counters + 2;
     const size_t n = n_tris;
     float *cen = nullptr;
-    HRR_CUDA(ctx, cudaMallocAsync(&cen, sizeof(float) * 4 * n, st));
+    HRR_CUDA(ctx, hrr_alloc(ctx, &cen, sizeof(float) * 4 * n));
     const unsigned gr = (unsigned)((n + kThreads - 1) / kThreads);
     HRR_CUDA(ctx, cudaMemsetAsync(flags, 0, sizeof(unsigned long long), st));
     centroid_kernel<<<gr, kThreads, 0, st>>>(dev_tris, n_tris, cen, cen + n, cen + 2 * n, cen + 3 * n, flags);
@@ -377,8 +377,8 @@ int hrr_build_scene(hrr_ctx *ctx, const float *dev_tris, uint32_t n_tris, hrr_sc
     sc->n = n_tris;
     sc->tree = tree;
     uint32_t *links = nullptr;
-    cudaError_t e = cudaMallocAsync(&sc->tris, sizeof(float) * kTriFloats * n, st);
-    if (e == cudaSuccess) e = cudaMallocAsync(&links, sizeof(uint32_t) * 3 * n, st);
+    cudaError_t e = hrr_alloc(ctx, &sc->tris, sizeof(float) * kTriFloats * n);
+    if (e == cudaSuccess) e = hrr_alloc(ctx, &links, sizeof(uint32_t) * 3 * n);
     if (e == cudaSuccess) e = cudaMemsetAsync(links, 0xFF, sizeof(uint32_t) * 2 * n, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(links + 2 * n, 0, sizeof(uint32_t) * n, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(flags, 0, sizeof(unsigned long long), st);

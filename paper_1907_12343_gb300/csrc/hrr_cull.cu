@@ -139,7 +139,7 @@ int ensure_spill(hrr_ctx *ctx, size_t need) {
     if (ctx->spill) cudaFree(ctx->spill);
     ctx->spill = nullptr;
     ctx->spill_entries = 0;
-    if (cudaMalloc(&ctx->spill, need * sizeof(uint2)) != cudaSuccess) {
+    if (hrr_malloc(ctx, &ctx->spill, need * sizeof(uint2)) != cudaSuccess) {
         cudaGetLastError();
         return hrr_fail(ctx, HRR_ERR_OOM, "traversal stack spill area");
     }
@@ -246,7 +246,7 @@ int hrr_cull_host_impl(hrr_ctx *ctx, const hrr_eyes &H, uint32_t n_eyes, const h
         if (buf) cudaFree(buf);
         buf = nullptr;
         have = 0;
-        if (cudaMalloc(&buf, want * unit + 1024) != cudaSuccess) {
+        if (hrr_malloc(ctx, &buf, want * unit + 1024) != cudaSuccess) {
             cudaGetLastError();
             return hrr_fail(ctx, HRR_ERR_OOM, what);
         }

@@ -294,7 +294,7 @@ int hrr_cull_samples_impl(hrr_ctx *ctx, const hrr_eyes &E, uint32_t n_eyes, cons
             if (ctx->spill) cudaFree(ctx->spill);
             ctx->spill = nullptr;
             ctx->spill_entries = 0;
-            if (cudaMalloc(&ctx->spill, need * sizeof(uint2)) != cudaSuccess) {
+            if (hrr_malloc(ctx, &ctx->spill, need * sizeof(uint2)) != cudaSuccess) {
                 cudaGetLastError();
                 return hrr_fail(ctx, HRR_ERR_OOM, "traversal stack spill area");
             }
