@@ -227,7 +227,7 @@ __global__ void __launch_bounds__(kBoxBlock, 3) box_kernel(LEAVES leaf, uint32_t
     __shared__ float4 sa[2][kBoxBlock], sb[2][kBoxBlock];  // child: (low, imax), (high, height)
     __shared__ uint32_t arrived[kBoxBlock], up[kBoxBlock], cut[kBoxBlock];
     __shared__ bool inside[kBoxBlock];
-    if (*(volatile unsigned long long *)flags & HRR_FLAG_NONFINITE) return;  // set before the launch: block-uniform
+    if (*(volatile unsigned long long *)flags & (HRR_FLAG_NONFINITE | HRR_FLAG_RUNS)) return;  // set before the launch
     const uint32_t t = threadIdx.x, base = blockIdx.x * kBoxBlock, g = base + t;
     uint32_t split = 0, other = 0, first = 0, last = 0;
     bool whole = false;  // node g exists and lies inside the block
@@ -329,7 +329,7 @@ template <bool DERIVED, typename LEAVES>
 __global__ void __launch_bounds__(kSpanThreads) span_kernel(LEAVES leaf, uint32_t n, hrr_node *nodes, float4 *wide,
                                                             BoxScratch s, uint32_t box_blocks,
                                                             unsigned long long *flags) {
-    if (*(volatile unsigned long long *)flags & HRR_FLAG_NONFINITE) return;
+    if (*(volatile unsigned long long *)flags & (HRR_FLAG_NONFINITE | HRR_FLAG_RUNS)) return;
     const uint32_t count = *s.span_count;
     if (blockIdx.x >= box_blocks) {
         uint32_t h = 0;

@@ -5,8 +5,8 @@
 // sequence index inherit the radical inverse's stratification. This file builds such a
 // hierarchy on the device:
 //   1. morton_kernel     63-bit Morton keys (21 bits per axis) and finiteness checks;
-//   2. radix_* kernels   stable LSD radix sort of (key, original index), 8 bits per pass;
-//   3. gather_kernel     sorted (x, y, z, intensity) as float4;
+//   2. sort passes       stable radix sort of (key, original index), 8 bits each (hrr_sort.cuh);
+//   3. gather_sorted     short runs put in order; sorted (x, y, z, intensity) as float4;
 //   4. topology_kernel   binary radix tree over (key, sorted position) in parallel: every
 //                        internal node finds its range and split from its neighbours'
 //                        common-prefix lengths (Karras, HPG 2012);
@@ -15,12 +15,11 @@
 
 #include "hrr_boxes.cuh"
 #include "hrr_internal.cuh"
+#include "hrr_sort.cuh"
 
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kItems = 16;
-constexpr int kTile = kThreads * kItems;  // keys per sort block
 
 // Spread the low 21 bits of v so that bit k moves to bit 3k.
 __device__ __forceinline__ uint64_t spread3(uint64_t v) {
@@ -41,133 +40,77 @@ __device__ __forceinline__ uint32_t grid_cell(float x) {
     return f >= 2097151.0f ? 2097151u : (uint32_t)f;
 }
 
+// Keys, finiteness checks, and the digit counts of the sort's passes. Blocks stride over the
+// lights, so that few add their counts to the totals.
 __global__ void __launch_bounds__(kThreads) morton_kernel(const float *__restrict__ x,
                                                           const float *__restrict__ y,
                                                           const float *__restrict__ z,
                                                           const float *__restrict__ inten,
                                                           uint32_t n, uint64_t *__restrict__ keys,
-                                                          uint32_t *__restrict__ vals,
+                                                          int shift, int passes, uint32_t *hist,
                                                           unsigned long long *flags) {
+    __shared__ uint32_t cnt[kSortPasses * 256];
+    for (int k = threadIdx.x; k < 256 * passes; k += kThreads) cnt[k] = 0;
+    __syncthreads();
+    for (uint32_t i = blockIdx.x * kThreads + threadIdx.x; i < n; i += gridDim.x * kThreads) {
+        const float px = x[i], py = y[i], pz = z[i], w = inten[i];
+        if (!isfinite(px) || !isfinite(py) || !isfinite(pz) || !isfinite(w))
+            atomicOr(flags, HRR_FLAG_NONFINITE);
+        const uint64_t key = (spread3(grid_cell(px)) << 2) | (spread3(grid_cell(py)) << 1) | spread3(grid_cell(pz));
+        keys[i] = key;
+        count_digits(cnt, key, shift, passes);
+    }
+    __syncthreads();
+    for (int k = threadIdx.x; k < 256 * passes; k += kThreads)
+        if (cnt[k]) atomicAdd(&hist[k], cnt[k]);
+}
+inline unsigned morton_grid(uint32_t n) { return std::min(608u, (n + 4 * kThreads - 1) / (4 * kThreads)); }
+
+// After the sort: sorted keys, permutation and lights, and the box pass's scratch reset. With
+// RUNS the keys are sorted by their upper halves only, and light i's place among the lights that
+// share its upper half is counted from their lower ones (ties by the order they are in); a run
+// of more than kRunMax lights raises HRR_FLAG_RUNS and stays as it is.
+template <bool RUNS>
+__global__ void __launch_bounds__(kThreads) gather_sorted_kernel(const float *__restrict__ x,
+                                                                 const float *__restrict__ y,
+                                                                 const float *__restrict__ z,
+                                                                 const float *__restrict__ inten,
+                                                                 const uint64_t *__restrict__ keys_in,
+                                                                 const uint32_t *__restrict__ vals_in, uint32_t n,
+                                                                 uint64_t *__restrict__ keys, uint32_t *__restrict__ perm,
+                                                                 float4 *__restrict__ spos, BoxScratch s,
+                                                                 unsigned long long *flags) {
     const uint32_t i = blockIdx.x * kThreads + threadIdx.x;
     if (i >= n) return;
-    const float px = x[i], py = y[i], pz = z[i], w = inten[i];
-    if (!isfinite(px) || !isfinite(py) || !isfinite(pz) || !isfinite(w))
-        atomicOr(flags, HRR_FLAG_NONFINITE);
-    keys[i] = (spread3(grid_cell(px)) << 2) | (spread3(grid_cell(py)) << 1) | spread3(grid_cell(pz));
-    vals[i] = i;
+    const uint32_t v = vals_in[i];
+    const float4 p = make_float4(x[v], y[v], z[v], inten[v]);
+    const uint64_t key = keys_in[i];
+    uint32_t to = i;
+    if (RUNS) {
+        uint32_t left = 0, right = 0, ahead = 0;  // neighbours of the run, and those that move ahead of i
+        while (left <= kRunMax && left < i) {
+            const uint64_t o = keys_in[i - left - 1u];
+            if ((o ^ key) >> kTopShift) break;
+            ahead += o <= key;
+            ++left;
+        }
+        while (right <= kRunMax && i + right + 1u < n) {
+            const uint64_t o = keys_in[i + right + 1u];
+            if ((o ^ key) >> kTopShift) break;
+            ahead += o < key;
+            ++right;
+        }
+        if (left + right + 1u > kRunMax) atomicOr(flags, HRR_FLAG_RUNS);
+        else to = i - left + ahead;
+    }
+    keys[to] = key;
+    perm[to] = v;
+    spos[to] = p;
+    box_reset(s, i, n);
 }
 
-__global__ void __launch_bounds__(kThreads) radix_hist_kernel(const uint64_t *__restrict__ keys,
-                                                              uint32_t n, int shift,
-                                                              uint32_t *__restrict__ hist,
-                                                              uint32_t nblocks) {
-    __shared__ uint32_t h[256];
-    h[threadIdx.x] = 0;
-    __syncthreads();
-    const uint64_t base = (uint64_t)blockIdx.x * kTile;
-#pragma unroll 4
-    for (int k = 0; k < kItems; ++k) {
-        const uint64_t i = base + (uint64_t)k * kThreads + threadIdx.x;
-        if (i < n) atomicAdd(&h[(keys[i] >> shift) & 255u], 1u);
-    }
-    __syncthreads();
-    hist[(uint64_t)threadIdx.x * nblocks + blockIdx.x] = h[threadIdx.x];
-}
-
-// Exclusive prefix sums of each digit's row of the digit-major histogram
-// hist[d * nblocks + b] (256 digits), in place, one warp per digit (8 consecutive counts per
-// lane, a running carry over chunks of 256), and each digit's total in totals[d].
-__global__ void __launch_bounds__(256) digit_scan_kernel(uint32_t *hist, uint32_t nblocks, uint32_t *totals) {
-    const int lane = threadIdx.x & 31;
-    const uint32_t d = blockIdx.x * 8u + (threadIdx.x >> 5);
-    uint32_t *row = hist + (uint64_t)d * nblocks;
-    uint32_t carry = 0;
-    for (uint32_t b0 = 0; b0 < nblocks; b0 += 256) {
-        const uint32_t base = b0 + (uint32_t)lane * 8u;
-        uint32_t v[8], s = 0;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            v[k] = base + k < nblocks ? row[base + k] : 0u;
-            s += v[k];
-        }
-        uint32_t x = s;
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
-            if (lane >= o) x += y;
-        }
-        uint32_t run = carry + x - s;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            if (base + k < nblocks) row[base + k] = run;
-            run += v[k];
-        }
-        carry += __shfl_sync(0xFFFFFFFFu, x, 31);
-    }
-    if (lane == 0) totals[d] = carry;
-}
-
-// Stable scatter of one tile: items are taken in groups of 256 in tile order; an item's
-// rank among equal digits is (earlier groups) + (earlier warps of its group) + (earlier
-// lanes of its warp, from __match_any_sync); the digit's base comes first.
-__global__ void __launch_bounds__(kThreads) radix_scatter_kernel(
-    const uint64_t *__restrict__ keys_in, const uint32_t *__restrict__ vals_in,
-    uint64_t *__restrict__ keys_out, uint32_t *__restrict__ vals_out, uint32_t n, int shift,
-    const uint32_t *__restrict__ offsets, uint32_t nblocks, const uint32_t *__restrict__ totals) {
-    static_assert(kThreads == 256, "one digit per thread");
-    __shared__ uint32_t running[256];
-    __shared__ uint32_t warp_cnt[kThreads / 32][256];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    {  // the digit's base: exclusive prefix of the digit totals (a block scan)
-        const uint32_t t = totals[threadIdx.x];
-        uint32_t x = t;
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
-            if (lane >= o) x += y;
-        }
-        if (lane == 31) running[warp] = x;
-        __syncthreads();
-        uint32_t before = 0;
-        for (int w = 0; w < warp; ++w) before += running[w];
-        __syncthreads();
-        running[threadIdx.x] = offsets[(uint64_t)threadIdx.x * nblocks + blockIdx.x] + before + x - t;
-    }
-#pragma unroll
-    for (int w = 0; w < kThreads / 32; ++w) warp_cnt[w][threadIdx.x] = 0;
-    __syncthreads();
-    const uint64_t base = (uint64_t)blockIdx.x * kTile;
-    const unsigned lt = (1u << lane) - 1u;
-    for (int k = 0; k < kItems; ++k) {
-        const uint64_t i = base + (uint64_t)k * kThreads + threadIdx.x;
-        const bool valid = i < n;
-        const uint64_t key = valid ? keys_in[i] : 0ull;
-        const uint32_t val = valid ? vals_in[i] : 0u;
-        const uint32_t d = valid ? (uint32_t)((key >> shift) & 255u) : 256u;
-        const unsigned peers = __match_any_sync(0xFFFFFFFFu, d);
-        const uint32_t rank = __popc(peers & lt);
-        if (valid && rank == 0) warp_cnt[warp][d] = __popc(peers);
-        __syncthreads();
-        if (valid) {
-            uint32_t before = 0;
-            for (int w = 0; w < warp; ++w) before += warp_cnt[w][d];
-            const uint32_t pos = running[d] + before + rank;
-            keys_out[pos] = key;
-            vals_out[pos] = val;
-        }
-        __syncthreads();
-        uint32_t tot = 0;
-#pragma unroll
-        for (int w = 0; w < kThreads / 32; ++w) {
-            tot += warp_cnt[w][threadIdx.x];
-            warp_cnt[w][threadIdx.x] = 0;
-        }
-        running[threadIdx.x] += tot;
-        __syncthreads();
-    }
-}
-
-// Positions and intensities in leaf order, and the box pass's scratch reset (leaf i's entries
-// by thread i, in place of three memory sets).
-template <bool CHECK>
+// Moved lights in leaf order, checked, and the box pass's scratch reset (leaf i's entries by
+// thread i, in place of memory sets).
 __global__ void __launch_bounds__(kThreads) gather_kernel(const float *__restrict__ x,
                                                           const float *__restrict__ y,
                                                           const float *__restrict__ z,
@@ -179,8 +122,7 @@ __global__ void __launch_bounds__(kThreads) gather_kernel(const float *__restric
     if (i >= n) return;
     const uint32_t v = perm[i];
     const float4 p = make_float4(x[v], y[v], z[v], inten[v]);
-    if (CHECK && (!isfinite(p.x) || !isfinite(p.y) || !isfinite(p.z) || !isfinite(p.w)))
-        atomicOr(flags, HRR_FLAG_NONFINITE);
+    if (!isfinite(p.x) || !isfinite(p.y) || !isfinite(p.z) || !isfinite(p.w)) atomicOr(flags, HRR_FLAG_NONFINITE);
     spos[i] = p;
     box_reset(s, i, n);
 }
@@ -198,10 +140,11 @@ __device__ __forceinline__ int prefix_len(const uint64_t *__restrict__ keys, int
 __global__ void __launch_bounds__(kThreads) topology_kernel(const uint64_t *__restrict__ keys,
                                                             uint32_t n, hrr_node *__restrict__ nodes,
                                                             uint32_t *__restrict__ leaf_parent,
-                                                            uint32_t *__restrict__ int_parent) {
+                                                            uint32_t *__restrict__ int_parent,
+                                                            const unsigned long long *flags) {
     const int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x;
     const int64_t N = n;
-    if (i >= N - 1) return;
+    if (i >= N - 1 || (*flags & HRR_FLAG_RUNS)) return;  // not sorted
     const int d = (prefix_len(keys, N, i, i + 1) - prefix_len(keys, N, i, i - 1)) >= 0 ? 1 : -1;
     const int dmin = prefix_len(keys, N, i, i - d);
     int64_t lmax = 2;
@@ -758,7 +701,8 @@ namespace {
 // The cost-driven topology for n >= 2 sorted lights: writes split / other_end of every
 // record and the parent links, level by level (one host round trip per level).
 int cost_topology(hrr_ctx *ctx, const float4 *spos, const uint64_t *keys, uint32_t n, uint32_t cost_depth,
-                  hrr_node *nodes, uint32_t *leaf_parent, uint32_t *int_parent, cudaStream_t st) {
+                  hrr_node *nodes, uint32_t *leaf_parent, uint32_t *int_parent, const unsigned long long *flags,
+                  cudaStream_t st) {
     const size_t cap_s = (size_t)n / 2 + 1;                    // ranges of >= 2 lights in a level
     const size_t cap_m = (size_t)n / (kSmallMax + 1) + 1;      // ... of > 32
     const size_t cap_b = (size_t)n / (kMidMax + 1) + 1;        // ... of > 256
@@ -835,7 +779,9 @@ int cost_topology(hrr_ctx *ctx, const float4 *spos, const uint64_t *keys, uint32
         }
         if ((e = cudaGetLastError()) != cudaSuccess) break;
         if ((e = cudaMemcpyAsync(host, counts, sizeof(uint32_t) * 6, cudaMemcpyDeviceToHost, st)) != cudaSuccess) break;
+        if ((e = cudaMemcpyAsync(&ctx->host_counters[2], flags, sizeof(*flags), cudaMemcpyDeviceToHost, st)) != cudaSuccess) break;
         if ((e = cudaStreamSynchronize(st)) != cudaSuccess) break;
+        if (ctx->host_counters[2] & (HRR_FLAG_RUNS | HRR_FLAG_NONFINITE)) break;  // the build starts over, or fails
         ns = host[0];
         nm = host[1];
         nr = host[2];
@@ -849,9 +795,9 @@ int cost_topology(hrr_ctx *ctx, const float4 *spos, const uint64_t *keys, uint32
     return rc;
 }
 
-}  // namespace
-
-int hrr_build_impl(hrr_ctx *ctx, const hrr_lights &L, uint32_t n, hrr_tree **out, int topology, uint32_t cost_depth) {
+// Sorts by the key bits from `shift` up (kTopShift, or 0 for all).
+int build_attempt(hrr_ctx *ctx, const hrr_lights &L, uint32_t n, hrr_tree **out, int topology, uint32_t cost_depth,
+                  int shift) {
     cudaStream_t st = ctx->stream;
     hrr_tree *tree = new (std::nothrow) hrr_tree();
     if (!tree) return hrr_fail(ctx, HRR_ERR_OOM, "host allocation of the tree");
@@ -879,49 +825,36 @@ int hrr_build_impl(hrr_ctx *ctx, const hrr_lights &L, uint32_t n, hrr_tree **out
         if ((e = cudaGetLastError()) != cudaSuccess) return fail(hrr_cuda_fail(ctx, e, "single_leaf_kernel"));
         tree->height = 0;
     } else {
-        const uint32_t nblocks = (n + kTile - 1) / kTile;
-        const uint64_t hist_n = 256ull * (nblocks + 1);  // digit-major counts, then the digit totals
-        const size_t bytes = 2 * ((sizeof(uint64_t) * (size_t)n + 255) & ~size_t(255)) +
-                             ((sizeof(uint32_t) * (size_t)n + 255) & ~size_t(255)) +
-                             ((sizeof(uint32_t) * hist_n + 255) & ~size_t(255)) +
-                             ((sizeof(float4) * (size_t)n + 255) & ~size_t(255)) + box_scratch_bytes(n);
+        const size_t bytes = 2 * pad256(sizeof(uint64_t) * (size_t)n) + pad256(sizeof(uint32_t) * (size_t)n) +
+                             pad256(sort_scratch_bytes(n)) + pad256(sizeof(float4) * (size_t)n) + box_scratch_bytes(n);
         char *scratch = nullptr;
         if ((e = hrr_alloc(ctx, &scratch, bytes)) != cudaSuccess) return fail(hrr_cuda_fail(ctx, e, "build scratch"));
         char *p = scratch;
         uint64_t *keys0 = carve<uint64_t>(p, n), *keys1 = carve<uint64_t>(p, n);
-        uint32_t *vals1 = carve<uint32_t>(p, n);
-        uint32_t *hist = carve<uint32_t>(p, hist_n);
+        uint32_t *vals0 = carve<uint32_t>(p, n);
+        const SortScratch ss = carve_sort(p, n);
         float4 *spos = carve<float4>(p, n);
         const BoxScratch rs = carve_boxes(p, n);
-        uint32_t *vals0 = tree->perm;
 
         const unsigned g = (n + kThreads - 1) / kThreads;
         int rc = HRR_OK;
         do {
-            morton_kernel<<<g, kThreads, 0, st>>>(L.x, L.y, L.z, L.intensity, n, keys0, vals0, flags);
-            ++ctx->launches;
-            uint64_t *kin = keys0, *kout = keys1;
-            uint32_t *vin = vals0, *vout = vals1;
-            for (int shift = 0; shift < 64; shift += 8) {
-                radix_hist_kernel<<<nblocks, kThreads, 0, st>>>(kin, n, shift, hist, nblocks);
-                digit_scan_kernel<<<32, 256, 0, st>>>(hist, nblocks, hist + 256 * (size_t)nblocks);
-                radix_scatter_kernel<<<nblocks, kThreads, 0, st>>>(kin, vin, kout, vout, n, shift, hist, nblocks,
-                                                                     hist + 256 * (size_t)nblocks);
-                ctx->launches += 3;
-                uint64_t *tk = kin; kin = kout; kout = tk;
-                uint32_t *tv = vin; vin = vout; vout = tv;
-            }
-            // eight passes: the sorted keys are back in keys0 and the permutation in vals0
-            gather_kernel<false><<<g, kThreads, 0, st>>>(L.x, L.y, L.z, L.intensity, vals0, n, spos, rs, flags);
+            if ((e = cudaMemsetAsync(ss.hist, 0, sort_scratch_bytes(n), st)) != cudaSuccess) { rc = hrr_cuda_fail(ctx, e, "memset"); break; }
+            const int passes = sort_passes(shift);
+            morton_kernel<<<morton_grid(n), kThreads, 0, st>>>(L.x, L.y, L.z, L.intensity, n, keys0, shift, passes, ss.hist, flags);
+            sort_enqueue(keys0, vals0, keys1, tree->perm, n, shift, ss, flags, st);
+            (shift ? gather_sorted_kernel<true> : gather_sorted_kernel<false>)<<<g, kThreads, 0, st>>>(
+                L.x, L.y, L.z, L.intensity, keys0, vals0, n, keys1, tree->perm, spos, rs, flags);
+            ctx->launches += 2 + passes;
             const unsigned gi = (n - 1 + kThreads - 1) / kThreads;
             if (topology == HRR_TOPOLOGY_COST) {
-                if ((rc = cost_topology(ctx, spos, keys0, n, cost_depth, tree->nodes, rs.leaf_parent, rs.int_parent, st)) != HRR_OK) break;
+                if ((rc = cost_topology(ctx, spos, keys1, n, cost_depth, tree->nodes, rs.leaf_parent, rs.int_parent, flags, st)) != HRR_OK) break;
             } else {
-                topology_kernel<<<gi, kThreads, 0, st>>>(keys0, n, tree->nodes, rs.leaf_parent, rs.int_parent);
+                topology_kernel<<<gi, kThreads, 0, st>>>(keys1, n, tree->nodes, rs.leaf_parent, rs.int_parent, flags);
                 ++ctx->launches;
             }
             boxes_enqueue(PointLeaves{spos}, n, tree->nodes, tree->wide, rs, flags, st);
-            ctx->launches += 3;
+            ctx->launches += 2;
             if ((e = cudaGetLastError()) != cudaSuccess) { rc = hrr_cuda_fail(ctx, e, "build kernels"); break; }
             if ((e = cudaMemcpyAsync(&ctx->host_counters[4], rs.root_height, sizeof(uint32_t),
                                      cudaMemcpyDeviceToHost, st)) != cudaSuccess) { rc = hrr_cuda_fail(ctx, e, "height copy"); break; }
@@ -935,10 +868,20 @@ int hrr_build_impl(hrr_ctx *ctx, const hrr_lights &L, uint32_t n, hrr_tree **out
     if (n > 1) tree->height = (uint32_t)(ctx->host_counters[4] & 0xFFFFFFFFull);
     if (ctx->host_counters[2] & HRR_FLAG_NONFINITE)
         return fail(hrr_fail(ctx, HRR_ERR_INVALID_ARG, "a light position or intensity is not finite"));
-    if (ctx->host_counters[2] & HRR_FLAG_TOPOLOGY)
+    if ((ctx->host_counters[2] & HRR_FLAG_RUNS) && shift) {  // many lights in few cells: every key bit sorted
+        fail(HRR_OK);
+        return build_attempt(ctx, L, n, out, topology, cost_depth, 0);
+    }
+    if (ctx->host_counters[2] & (HRR_FLAG_TOPOLOGY | HRR_FLAG_WAIT))
         return fail(hrr_fail(ctx, HRR_ERR_DEVICE, "inconsistent radix-tree links"));
     *out = tree;
     return HRR_OK;
+}
+
+}  // namespace
+
+int hrr_build_impl(hrr_ctx *ctx, const hrr_lights &L, uint32_t n, hrr_tree **out, int topology, uint32_t cost_depth) {
+    return build_attempt(ctx, L, n, out, topology, cost_depth, kTopShift);
 }
 
 // ------------------------------------------------------------------------------------
@@ -959,7 +902,7 @@ cudaError_t hrr_refit_enqueue(hrr_tree *tree, const hrr_lights &L, void *scratch
     float4 *spos = carve<float4>(p, n);
     const BoxScratch rs = carve_boxes(p, n);
     const unsigned g = (n + kThreads - 1) / kThreads, gi = (n - 1 + kThreads - 1) / kThreads;
-    gather_kernel<true><<<g, kThreads, 0, st>>>(L.x, L.y, L.z, L.intensity, tree->perm, n, spos, rs, flags);
+    gather_kernel<<<g, kThreads, 0, st>>>(L.x, L.y, L.z, L.intensity, tree->perm, n, spos, rs, flags);
     links_kernel<<<gi, kThreads, 0, st>>>(tree->nodes, n, rs.leaf_parent, rs.int_parent, flags);
     return boxes_enqueue(PointLeaves{spos}, n, tree->nodes, tree->wide, rs, flags, st);
 }
@@ -984,7 +927,7 @@ constexpr uint32_t kStaticMaxLights = HRR_STATIC_BUILD_MAX_LIGHTS;
 constexpr size_t static_scratch_bytes(size_t n) {
     return 2 * pad256(sizeof(uint64_t) * n)                               // keys, ping-pong
            + pad256(sizeof(uint32_t) * n)                                 // second value buffer
-           + pad256(sizeof(uint32_t) * 256 * ((n + kTile - 1) / kTile + 1)) // digit histograms, totals
+           + pad256(sort_scratch_bytes(n))                                // digit counts, tile states
            + pad256(sizeof(float4) * n)                                   // sorted lights
            + box_scratch_bytes((uint32_t)n)                               // box pass
            + pad256(sizeof(unsigned long long));                          // error flags
@@ -1041,8 +984,8 @@ extern "C" int hrr_build_light_tree_static(hrr_lights L, uint32_t n, hrr_node *d
     }
     char *p = scratch;
     uint64_t *keys0 = carve<uint64_t>(p, kStaticMaxLights), *keys1 = carve<uint64_t>(p, kStaticMaxLights);
-    uint32_t *vals1 = carve<uint32_t>(p, kStaticMaxLights);
-    uint32_t *hist = carve<uint32_t>(p, 256 * ((kStaticMaxLights + kTile - 1) / kTile + 1));
+    uint32_t *vals0 = carve<uint32_t>(p, kStaticMaxLights);
+    const SortScratch ss = carve_sort(p, kStaticMaxLights);
     float4 *spos = carve<float4>(p, kStaticMaxLights);
     const BoxScratch rs = carve_boxes(p, kStaticMaxLights);
     unsigned long long *flags = carve<unsigned long long>(p, 1);
@@ -1056,23 +999,15 @@ extern "C" int hrr_build_light_tree_static(hrr_lights L, uint32_t n, hrr_node *d
             e = cudaGetLastError();
         }
     } else {
-        const uint32_t nblocks = (n + kTile - 1) / kTile;
+        if (e == cudaSuccess) e = cudaMemsetAsync(ss.hist, 0, sort_scratch_bytes(n), st);
         if (e == cudaSuccess) {
             const unsigned g = (n + kThreads - 1) / kThreads;
-            morton_kernel<<<g, kThreads, 0, st>>>(L.x, L.y, L.z, L.intensity, n, keys0, dev_perm, flags);
-            uint64_t *kin = keys0, *kout = keys1;
-            uint32_t *vin = dev_perm, *vout = vals1;
-            for (int shift = 0; shift < 64; shift += 8) {
-                radix_hist_kernel<<<nblocks, kThreads, 0, st>>>(kin, n, shift, hist, nblocks);
-                digit_scan_kernel<<<32, 256, 0, st>>>(hist, nblocks, hist + 256 * (size_t)nblocks);
-                radix_scatter_kernel<<<nblocks, kThreads, 0, st>>>(kin, vin, kout, vout, n, shift, hist, nblocks,
-                                                                     hist + 256 * (size_t)nblocks);
-                uint64_t *tk = kin; kin = kout; kout = tk;
-                uint32_t *tv = vin; vin = vout; vout = tv;
-            }
-            gather_kernel<false><<<g, kThreads, 0, st>>>(L.x, L.y, L.z, L.intensity, dev_perm, n, spos, rs, flags);
+            morton_kernel<<<morton_grid(n), kThreads, 0, st>>>(L.x, L.y, L.z, L.intensity, n, keys0, 0, kSortPasses, ss.hist, flags);
+            sort_enqueue(keys0, vals0, keys1, dev_perm, n, 0, ss, flags, st);
+            gather_sorted_kernel<false><<<g, kThreads, 0, st>>>(L.x, L.y, L.z, L.intensity, keys0, vals0, n, keys1, dev_perm,
+                                                                spos, rs, flags);
             const unsigned gi = (n - 1 + kThreads - 1) / kThreads;
-            topology_kernel<<<gi, kThreads, 0, st>>>(keys0, n, dev_nodes, rs.leaf_parent, rs.int_parent);
+            topology_kernel<<<gi, kThreads, 0, st>>>(keys1, n, dev_nodes, rs.leaf_parent, rs.int_parent, flags);
             boxes_enqueue(PointLeaves{spos}, n, dev_nodes, nullptr, rs, flags, st);
             e = cudaGetLastError();
         }
@@ -1092,7 +1027,7 @@ extern "C" int hrr_build_light_tree_static(hrr_lights L, uint32_t n, hrr_node *d
         set_err(err, err_len, "a light position or intensity is not finite");
         return HRR_ERR_INVALID_ARG;
     }
-    if (host_flags & HRR_FLAG_TOPOLOGY) {
+    if (host_flags & (HRR_FLAG_TOPOLOGY | HRR_FLAG_WAIT)) {
         set_err(err, err_len, "inconsistent radix-tree links");
         return HRR_ERR_DEVICE;
     }

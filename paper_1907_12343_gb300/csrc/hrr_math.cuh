@@ -11,6 +11,8 @@ enum : unsigned long long {
     HRR_FLAG_NONFINITE = 2ull, // a light position or intensity is not finite
     HRR_FLAG_TOPOLOGY = 4ull,  // a node record or parent link is out of range
     HRR_FLAG_RANGE = 8ull,     // an input index (a pair's eye or light) is out of range
+    HRR_FLAG_RUNS = 16ull,     // a build's keys have long runs of equal upper halves: sort them fully
+    HRR_FLAG_WAIT = 32ull,     // a bounded wait ran out (cannot happen)
 };
 
 // ------------------------------------------------------------------------------------
