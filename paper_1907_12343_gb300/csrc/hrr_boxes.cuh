@@ -165,6 +165,31 @@ __device__ __forceinline__ void box_finish_groups(const BoxScratch &s, uint32_t 
     }
 }
 
+// The groups of 32 leaves (a warp each: `mine` is leaf g's box, empty past the last leaf).
+__device__ __forceinline__ void box_groups_of_32(const BoxScratch &s, const Box &mine, uint32_t g, uint32_t n) {
+    if (!box_level(n, 1)) return;
+    const Box w = warp_box(mine);
+    if ((g & 31u) == 0 && g < n) {
+        s.groups[2 * (size_t)(g >> 5)] = box_a(w);
+        s.groups[2 * (size_t)(g >> 5) + 1] = box_b(w, 0u);
+        __threadfence();
+    }
+}
+
+// All groups on their own, for what needs ranges' boxes before the topology is there.
+template <typename LEAVES>
+__global__ void __launch_bounds__(kBoxBlock) groups_kernel(LEAVES leaf, uint32_t n, BoxScratch s) {
+    const uint32_t base = blockIdx.x * kBoxBlock, g = base + threadIdx.x;
+    box_groups_of_32(s, g < n ? leaf(g) : box_empty(), g, n);
+    __syncthreads();
+    if (threadIdx.x < 32u) box_finish_groups(s, base, n);
+}
+template <typename LEAVES>
+cudaError_t groups_enqueue(const LEAVES &leaf, uint32_t n, const BoxScratch &s, cudaStream_t st) {
+    groups_kernel<<<(n + kBoxBlock - 1) / kBoxBlock, kBoxBlock, 0, st>>>(leaf, n, s);
+    return cudaGetLastError();
+}
+
 // The union of leaves [a, b] (a <= b), by a whole warp.
 template <typename LEAVES>
 __device__ __forceinline__ Box box_range(const LEAVES &leaf, const BoxScratch &s, uint32_t n, uint32_t a, uint32_t b) {
@@ -223,7 +248,7 @@ __device__ __forceinline__ void store_record(float4 *r, float4 a0, float4 b0, fl
 // The nodes inside blocks, the groups, the list of spanning nodes.
 template <bool DERIVED, typename LEAVES>
 __global__ void __launch_bounds__(kBoxBlock, 3) box_kernel(LEAVES leaf, uint32_t n, hrr_node *nodes, float4 *wide,
-                                                        BoxScratch s, unsigned long long *flags) {
+                                                        BoxScratch s, bool have_groups, unsigned long long *flags) {
     __shared__ float4 sa[2][kBoxBlock], sb[2][kBoxBlock];  // child: (low, imax), (high, height)
     __shared__ uint32_t arrived[kBoxBlock], up[kBoxBlock], cut[kBoxBlock];
     __shared__ bool inside[kBoxBlock];
@@ -245,16 +270,9 @@ __global__ void __launch_bounds__(kBoxBlock, 3) box_kernel(LEAVES leaf, uint32_t
     cut[t] = split;
     up[t] = whole ? s.int_parent[g] : 0xFFFFFFFFu;
     const Box mine = g < n ? leaf(g) : box_empty();
-    if (box_level(n, 1)) {
-        const Box w = warp_box(mine);
-        if ((t & 31u) == 0 && g < n) {
-            s.groups[2 * (size_t)(g >> 5)] = box_a(w);
-            s.groups[2 * (size_t)(g >> 5) + 1] = box_b(w, 0u);
-            __threadfence();
-        }
-    }
+    if (!have_groups) box_groups_of_32(s, mine, g, n);
     __syncthreads();
-    if (t < 32u) box_finish_groups(s, base, n);
+    if (!have_groups && t < 32u) box_finish_groups(s, base, n);
 
     if (g < n) {
         Box x = mine;
@@ -405,16 +423,17 @@ __global__ void __launch_bounds__(kSpanThreads) span_kernel(LEAVES leaf, uint32_
 
 // Both kernels, for n >= 2 leaves: the records of `nodes` and, with `wide`, the derived records
 // (the top slots after the records, the width-four records); *s.root_height gets the height.
+// have_groups: groups_enqueue has run on the same leaves.
 template <typename LEAVES>
 cudaError_t boxes_enqueue(const LEAVES &leaf, uint32_t n, hrr_node *nodes, float4 *wide, const BoxScratch &s,
-                          unsigned long long *flags, cudaStream_t st) {
+                          unsigned long long *flags, cudaStream_t st, bool have_groups = false) {
     const unsigned blocks = (n + kBoxBlock - 1) / kBoxBlock;
     const unsigned bb = std::min(608u, 8u + blocks), hb = std::min(152u, 1u + blocks / 16u);
     if (wide) {
-        box_kernel<true><<<blocks, kBoxBlock, 0, st>>>(leaf, n, nodes, wide, s, flags);
+        box_kernel<true><<<blocks, kBoxBlock, 0, st>>>(leaf, n, nodes, wide, s, have_groups, flags);
         span_kernel<true><<<bb + hb, kSpanThreads, 0, st>>>(leaf, n, nodes, wide, s, bb, flags);
     } else {
-        box_kernel<false><<<blocks, kBoxBlock, 0, st>>>(leaf, n, nodes, wide, s, flags);
+        box_kernel<false><<<blocks, kBoxBlock, 0, st>>>(leaf, n, nodes, wide, s, have_groups, flags);
         span_kernel<false><<<bb + hb, kSpanThreads, 0, st>>>(leaf, n, nodes, wide, s, bb, flags);
     }
     return cudaGetLastError();
