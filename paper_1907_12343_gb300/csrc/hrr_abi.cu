@@ -248,6 +248,7 @@ int hrr_free_light_tree(hrr_ctx *ctx, hrr_tree *tree) {
     DeviceGuard g(ctx->device);
     if (tree->nodes) HRR_CUDA(ctx, cudaFreeAsync(tree->nodes, ctx->stream));
     if (tree->perm) HRR_CUDA(ctx, cudaFreeAsync(tree->perm, ctx->stream));
+    if (tree->pairs) HRR_CUDA(ctx, cudaFreeAsync(tree->pairs, ctx->stream));
     if (tree->wide) HRR_CUDA(ctx, cudaFreeAsync(tree->wide, ctx->stream));
     delete tree;
     return HRR_OK;

@@ -245,9 +245,22 @@ __device__ __forceinline__ void store_record(float4 *r, float4 a0, float4 b0, fl
     store32(r + 2, a1, make_float4(b1.x, b1.y, b1.z, __uint_as_float(other)));
 }
 
+// A node's paired record (hrr_tree::pairs).
+__device__ __forceinline__ void store_pairs(float4 *r, float4 a0, float4 b0, float4 a1, float4 b1, uint32_t split,
+                                            uint32_t other) {
+    store32(r, make_float4(-a0.x, -a1.x, -a0.y, -a1.y), make_float4(-a0.z, -a1.z, -b0.x, -b1.x));
+    store32(r + 2, make_float4(-b0.y, -b1.y, -b0.z, -b1.z),
+            make_float4(a0.w, a1.w, __uint_as_float(split), __uint_as_float(other)));
+}
+
+// The records derived from the binary ones, or none (scenes, builds into caller's arrays).
+struct Derived {
+    float4 *pairs, *wide;
+};
+
 // The nodes inside blocks, the groups, the list of spanning nodes.
 template <bool DERIVED, typename LEAVES>
-__global__ void __launch_bounds__(kBoxBlock, 3) box_kernel(LEAVES leaf, uint32_t n, hrr_node *nodes, float4 *wide,
+__global__ void __launch_bounds__(kBoxBlock, 3) box_kernel(LEAVES leaf, uint32_t n, hrr_node *nodes, Derived der,
                                                         BoxScratch s, bool have_groups, unsigned long long *flags) {
     __shared__ float4 sa[2][kBoxBlock], sb[2][kBoxBlock];  // child: (low, imax), (high, height)
     __shared__ uint32_t arrived[kBoxBlock], up[kBoxBlock], cut[kBoxBlock];
@@ -311,7 +324,8 @@ __global__ void __launch_bounds__(kBoxBlock, 3) box_kernel(LEAVES leaf, uint32_t
             const uint32_t k0 = leaf0 ? t : split - base, k1 = leaf1 ? t : split + 1u - base;
             const float4 a[4] = {sa[0][k0], sa[1][k0], leaf1 ? a1 : sa[0][k1], sa[1][k1]};
             const float4 b[4] = {sb[0][k0], sb[1][k0], leaf1 ? b1 : sb[0][k1], sb[1][k1]};
-            store_wide(wide + 8 * (size_t)g, a, b, leaf0, leaf1, leaf0 ? split : cut[k0], split, leaf1 ? last : cut[k1],
+            store_pairs(der.pairs + 4 * (size_t)hrr_node_slot(g, other), a0, b0, a1, b1, split, other);
+            store_wide(der.wide + 8 * (size_t)g, a, b, leaf0, leaf1, leaf0 ? split : cut[k0], split, leaf1 ? last : cut[k1],
                        other);
         }
     }
@@ -344,7 +358,7 @@ __device__ __forceinline__ uint32_t top_walk(uint32_t s, const hrr_node *nodes, 
 // thread per spanning node: its depth by the parent links, plus the heights of its children
 // inside blocks). Blocks [0, box_blocks) do the first two, the others the last.
 template <bool DERIVED, typename LEAVES>
-__global__ void __launch_bounds__(kSpanThreads) span_kernel(LEAVES leaf, uint32_t n, hrr_node *nodes, float4 *wide,
+__global__ void __launch_bounds__(kSpanThreads) span_kernel(LEAVES leaf, uint32_t n, hrr_node *nodes, Derived der,
                                                             BoxScratch s, uint32_t box_blocks,
                                                             unsigned long long *flags) {
     if (*(volatile unsigned long long *)flags & (HRR_FLAG_NONFINITE | HRR_FLAG_RUNS)) return;
@@ -416,25 +430,27 @@ __global__ void __launch_bounds__(kSpanThreads) span_kernel(LEAVES leaf, uint32_
                          box_b(x1, 0u), split, other);
             const float4 a[4] = {box_a(q[0]), box_a(q[1]), box_a(q[2]), box_a(q[3])};
             const float4 b[4] = {box_b(q[0], 0u), box_b(q[1], 0u), box_b(q[2], 0u), box_b(q[3], 0u)};
-            store_wide(wide + 8 * (size_t)g, a, b, leaf0, leaf1, split0, split, split1, other);
+            store_pairs(der.pairs + 4 * (size_t)hrr_node_slot(g, other), box_a(x0), box_b(x0, 0u), box_a(x1),
+                        box_b(x1, 0u), split, other);
+            store_wide(der.wide + 8 * (size_t)g, a, b, leaf0, leaf1, split0, split, split1, other);
         }
     }
 }
 
-// Both kernels, for n >= 2 leaves: the records of `nodes` and, with `wide`, the derived records
-// (the top slots after the records, the width-four records); *s.root_height gets the height.
+// Both kernels, for n >= 2 leaves: the records of `nodes` and, unless `der` is empty, the derived
+// records (the top slots after the records, the paired and width-four records); *s.root_height gets the height.
 // have_groups: groups_enqueue has run on the same leaves.
 template <typename LEAVES>
-cudaError_t boxes_enqueue(const LEAVES &leaf, uint32_t n, hrr_node *nodes, float4 *wide, const BoxScratch &s,
+cudaError_t boxes_enqueue(const LEAVES &leaf, uint32_t n, hrr_node *nodes, const Derived &der, const BoxScratch &s,
                           unsigned long long *flags, cudaStream_t st, bool have_groups = false) {
     const unsigned blocks = (n + kBoxBlock - 1) / kBoxBlock;
     const unsigned bb = std::min(608u, 8u + blocks), hb = std::min(152u, 1u + blocks / 16u);
-    if (wide) {
-        box_kernel<true><<<blocks, kBoxBlock, 0, st>>>(leaf, n, nodes, wide, s, have_groups, flags);
-        span_kernel<true><<<bb + hb, kSpanThreads, 0, st>>>(leaf, n, nodes, wide, s, bb, flags);
+    if (der.wide) {
+        box_kernel<true><<<blocks, kBoxBlock, 0, st>>>(leaf, n, nodes, der, s, have_groups, flags);
+        span_kernel<true><<<bb + hb, kSpanThreads, 0, st>>>(leaf, n, nodes, der, s, bb, flags);
     } else {
-        box_kernel<false><<<blocks, kBoxBlock, 0, st>>>(leaf, n, nodes, wide, s, have_groups, flags);
-        span_kernel<false><<<bb + hb, kSpanThreads, 0, st>>>(leaf, n, nodes, wide, s, bb, flags);
+        box_kernel<false><<<blocks, kBoxBlock, 0, st>>>(leaf, n, nodes, der, s, have_groups, flags);
+        span_kernel<false><<<bb + hb, kSpanThreads, 0, st>>>(leaf, n, nodes, der, s, bb, flags);
     }
     return cudaGetLastError();
 }

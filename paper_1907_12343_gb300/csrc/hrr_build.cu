@@ -172,10 +172,11 @@ __global__ void __launch_bounds__(kThreads) links_kernel(const hrr_node *__restr
     if (last == s + 1) leaf_parent[s + 1] = code | 1u; else int_parent[s + 1] = code | 1u;
 }
 
-// The hierarchy of one light: its record, its permutation and (with `wide`) the records derived
-// from it: the leaf in slot 0 of the width-four record, the rest and the top slots empty.
+// The hierarchy of one light: its record, its permutation and (unless `der` is empty) the records
+// derived from it: the leaf in slot 0 of the width-four record and in both places of the paired
+// one, the rest and the top slots empty.
 __global__ void single_leaf_kernel(const float *x, const float *y, const float *z,
-                                   const float *inten, hrr_node *node, uint32_t *perm, float4 *wide,
+                                   const float *inten, hrr_node *node, uint32_t *perm, Derived der,
                                    unsigned long long *flags) {
     const float px = x[0], py = y[0], pz = z[0], w = inten[0];
     if (!isfinite(px) || !isfinite(py) || !isfinite(pz) || !isfinite(w)) {
@@ -188,10 +189,12 @@ __global__ void single_leaf_kernel(const float *x, const float *y, const float *
     node->split = 0;
     node->other_end = 0;
     perm[0] = 0;
-    if (!wide) return;
+    if (!der.wide) return;
     const float4 *r = reinterpret_cast<const float4 *>(node);
-    for (int k = 0; k < 8; ++k) wide[k] = k < 2 ? r[k] : make_float4(0.f, 0.f, 0.f, 0.f);
-    for (uint32_t k = 0; k < 3 * HRR_TOP_SLOTS; ++k) reinterpret_cast<float4 *>(node)[4 + k] = wide[2];
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    store_pairs(der.pairs, r[0], r[1], r[0], r[1], 0u, 0u);
+    for (int k = 0; k < 8; ++k) der.wide[k] = k < 2 ? r[k] : zero;
+    for (uint32_t k = 0; k < 3 * HRR_TOP_SLOTS; ++k) reinterpret_cast<float4 *>(node)[4 + k] = zero;
 }
 
 }  // namespace
@@ -209,6 +212,7 @@ int build_attempt(hrr_ctx *ctx, const hrr_lights &L, uint32_t n, hrr_tree **out,
     auto fail = [&](int status) {
         if (tree->nodes) cudaFreeAsync(tree->nodes, st);
         if (tree->perm) cudaFreeAsync(tree->perm, st);
+        if (tree->pairs) cudaFreeAsync(tree->pairs, st);
         if (tree->wide) cudaFreeAsync(tree->wide, st);
         delete tree;
         return status;
@@ -216,6 +220,7 @@ int build_attempt(hrr_ctx *ctx, const hrr_lights &L, uint32_t n, hrr_tree **out,
     const uint32_t n_rec = n > 1 ? n - 1 : 1;
     cudaError_t e = hrr_alloc(ctx, &tree->nodes, sizeof(hrr_node) * (size_t)n_rec + HRR_TOP_BYTES);
     if (e == cudaSuccess) e = hrr_alloc(ctx, &tree->perm, sizeof(uint32_t) * (size_t)n);
+    if (e == cudaSuccess) e = hrr_alloc(ctx, &tree->pairs, 8 * sizeof(float4) * (size_t)n_rec);
     if (e == cudaSuccess) e = hrr_alloc(ctx, &tree->wide, 8 * sizeof(float4) * (size_t)n_rec);
     if (e != cudaSuccess) return fail(hrr_cuda_fail(ctx, e, "tree allocation"));
     unsigned long long *flags = ctx->counters + 2;
@@ -223,7 +228,8 @@ int build_attempt(hrr_ctx *ctx, const hrr_lights &L, uint32_t n, hrr_tree **out,
         return fail(hrr_cuda_fail(ctx, e, "flag reset"));
 
     if (n == 1) {
-        single_leaf_kernel<<<1, 1, 0, st>>>(L.x, L.y, L.z, L.intensity, tree->nodes, tree->perm, tree->wide, flags);
+        single_leaf_kernel<<<1, 1, 0, st>>>(L.x, L.y, L.z, L.intensity, tree->nodes, tree->perm,
+                                              Derived{tree->pairs, tree->wide}, flags);
         ++ctx->launches;
         if ((e = cudaGetLastError()) != cudaSuccess) return fail(hrr_cuda_fail(ctx, e, "single_leaf_kernel"));
         tree->height = 0;
@@ -261,7 +267,7 @@ int build_attempt(hrr_ctx *ctx, const hrr_lights &L, uint32_t n, hrr_tree **out,
                 topology_kernel<<<gi, kThreads, 0, st>>>(keys1, n, tree->nodes, rs.leaf_parent, rs.int_parent, flags);
                 ++ctx->launches;
             }
-            boxes_enqueue(PointLeaves{spos}, n, tree->nodes, tree->wide, rs, flags, st, groups);
+            boxes_enqueue(PointLeaves{spos}, n, tree->nodes, {tree->pairs, tree->wide}, rs, flags, st, groups);
             ctx->launches += 2;
             if ((e = cudaGetLastError()) != cudaSuccess) { rc = hrr_cuda_fail(ctx, e, "build kernels"); break; }
             if ((e = cudaMemcpyAsync(&ctx->host_counters[4], rs.root_height, sizeof(uint32_t),
@@ -303,7 +309,8 @@ cudaError_t hrr_refit_enqueue(hrr_tree *tree, const hrr_lights &L, void *scratch
     const uint32_t n = tree->n;
     // one leaf: rewrite the single record unless the light is not finite (checked there)
     if (n == 1) {
-        single_leaf_kernel<<<1, 1, 0, st>>>(L.x, L.y, L.z, L.intensity, tree->nodes, tree->perm, tree->wide, flags);
+        single_leaf_kernel<<<1, 1, 0, st>>>(L.x, L.y, L.z, L.intensity, tree->nodes, tree->perm,
+                                              Derived{tree->pairs, tree->wide}, flags);
         return cudaGetLastError();
     }
     char *p = static_cast<char *>(scratch_mem);
@@ -312,7 +319,7 @@ cudaError_t hrr_refit_enqueue(hrr_tree *tree, const hrr_lights &L, void *scratch
     const unsigned g = (n + kThreads - 1) / kThreads, gi = (n - 1 + kThreads - 1) / kThreads;
     gather_kernel<<<g, kThreads, 0, st>>>(L.x, L.y, L.z, L.intensity, tree->perm, n, spos, rs, flags);
     links_kernel<<<gi, kThreads, 0, st>>>(tree->nodes, n, rs.leaf_parent, rs.int_parent, flags);
-    return boxes_enqueue(PointLeaves{spos}, n, tree->nodes, tree->wide, rs, flags, st);
+    return boxes_enqueue(PointLeaves{spos}, n, tree->nodes, {tree->pairs, tree->wide}, rs, flags, st);
 }
 
 // ------------------------------------------------------------------------------------
@@ -403,7 +410,7 @@ extern "C" int hrr_build_light_tree_static(hrr_lights L, uint32_t n, hrr_node *d
     if (e == cudaSuccess) e = cudaMemsetAsync(rs.root_height, 0, sizeof(uint32_t), st);
     if (n == 1) {
         if (e == cudaSuccess) {
-            single_leaf_kernel<<<1, 1, 0, st>>>(L.x, L.y, L.z, L.intensity, dev_nodes, dev_perm, nullptr, flags);
+            single_leaf_kernel<<<1, 1, 0, st>>>(L.x, L.y, L.z, L.intensity, dev_nodes, dev_perm, Derived{nullptr, nullptr}, flags);
             e = cudaGetLastError();
         }
     } else {
@@ -416,7 +423,7 @@ extern "C" int hrr_build_light_tree_static(hrr_lights L, uint32_t n, hrr_node *d
                                                                 spos, rs, flags);
             const unsigned gi = (n - 1 + kThreads - 1) / kThreads;
             topology_kernel<<<gi, kThreads, 0, st>>>(keys1, n, dev_nodes, rs.leaf_parent, rs.int_parent, flags);
-            boxes_enqueue(PointLeaves{spos}, n, dev_nodes, nullptr, rs, flags, st);
+            boxes_enqueue(PointLeaves{spos}, n, dev_nodes, {nullptr, nullptr}, rs, flags, st);
             e = cudaGetLastError();
         }
     }

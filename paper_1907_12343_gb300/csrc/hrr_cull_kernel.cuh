@@ -71,14 +71,15 @@ namespace {
 constexpr uint32_t kMaxFrames = HRR_CULL_MAX_FRAMES;  // frames of one batched launch
 
 // Resident threads per SM each instantiation is compiled for (the register budget):
-// 40 registers for binary records (6 blocks of 256 threads), 64 for width four.
+// 48 registers for binary records (5 blocks of 256 threads), 64 for width four. With 40
+// registers and 6 blocks the binary form spills, and the frame takes 4% longer.
 template <int W>
 constexpr int min_blocks(int threads) {
-    return (W == 2 ? 1536 : 1024) / threads;
+    return (W == 2 ? 1280 : 1024) / threads;
 }
 
 using Frame = hrr_cull_frame_t;
-static_assert(sizeof(Frame) == 128, "frame descriptor layout");
+static_assert(sizeof(Frame) == 136, "frame descriptor layout");
 
 struct Launch {
     uint32_t n_frames;
@@ -103,13 +104,16 @@ __device__ __forceinline__ const Frame &frame_at(const Frame *F, uint32_t f) {
     else return F[f];
 }
 
-// 32 bytes (two float4) as one 256-bit read-only load that does not allocate in L1: the
-// records are scattered and rarely reused from L1, and filling it with them would take
-// L1 data-pipe cycles the kernel is bound by (they come from L2 either way).
+// 32 bytes (two float4, or four pairs of floats) as one 256-bit read-only load that does not
+// allocate in L1: the records are scattered and rarely reused from L1, and filling it with
+// them would take L1 data-pipe cycles (they come from L2 either way).
 __device__ __forceinline__ void load32(const float4 *p, float4 &a, float4 &b) {
     asm("ld.global.nc.L1::no_allocate.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
         : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w)
         : "l"(p));
+}
+__device__ __forceinline__ void load32(const float4 *p, hrr_f2 &a, hrr_f2 &b, hrr_f2 &c, hrr_f2 &d) {
+    asm("ld.global.nc.L1::no_allocate.v4.b64 {%0,%1,%2,%3}, [%4];" : "=l"(a), "=l"(b), "=l"(c), "=l"(d) : "l"(p));
 }
 
 // Range minimum of (brev(i) + r) over the L >= 1 indices from a; c = brev(2^32 - r).
@@ -135,7 +139,7 @@ struct Eye {
 template <int W>
 struct Visit {
     bool go[W], leaf[W];
-    uint32_t node[W], vmin[W], light[W];
+    uint32_t node[W], vmin[W], light[W];  // node: the child's record (slot of pairs, index of wide)
 };
 
 // Test one child slot: it survives unless its range minimum v culls it; the box is (lo, imax,
@@ -146,34 +150,36 @@ __device__ __forceinline__ bool survives(const Eye &E, const float4 &lo, const f
     return !hrr_node_culls(v, den, rhs);
 }
 
-// A visit of binary node `node`: its 64-byte record holds both children (box low corner
-// with the maximum intensity, box high corner with `split` / the range's other end).
+// A visit of the binary node at slot `slot` of hrr_tree::pairs: its 64-byte record holds both
+// children, paired axis by axis.
 template <int VARIANT>
-__device__ __forceinline__ void visit(const float4 *nodes, uint32_t n_lights, uint32_t node, uint32_t vmin,
+__device__ __forceinline__ void visit(const float4 *pairs, uint32_t n_lights, uint32_t slot, uint32_t vmin,
                                       const Eye &E, unsigned long long *flags, Visit<2> &V) {
-    float4 q0, q1, q2, q3;
-    load32(&nodes[4 * (size_t)node], q0, q1);
-    load32(&nodes[4 * (size_t)node + 2], q2, q3);
-    const uint32_t split = __float_as_uint(q1.w);
-    const uint32_t other = __float_as_uint(q3.w);
+    hrr_f2 nlox, nloy, nloz, nhix, nhiy, nhiz, imax, links;
+    load32(&pairs[4 * (size_t)slot], nlox, nloy, nloz, nhix);
+    load32(&pairs[4 * (size_t)slot + 2], nhiy, nhiz, imax, links);
+    const uint32_t node = hrr_slot_node(slot);
+    const uint32_t split = (uint32_t)links, other = (uint32_t)(links >> 32);
     const uint32_t first = min(node, other), last = max(node, other);
     if (last >= n_lights || split - first >= last - first) {  // needs first <= split < last
         atomicOr(flags, HRR_FLAG_TOPOLOGY);                    // corrupt record
         return;
     }
-    const bool int0 = first != split, int1 = split + 1u != last;
     const bool in0 = index_of(vmin, E.r) <= split;
     // the other child's minimum (of a leaf: its own value)
     const uint32_t vnew = range_min<VARIANT>(in0 ? split + 1u : first, in0 ? last - split : split - first + 1u, E.r, E.c);
     V.vmin[0] = in0 ? vmin : vnew;
     V.vmin[1] = in0 ? vnew : vmin;
-    V.node[0] = split;
-    V.node[1] = split + 1u;
-    const bool s0 = survives(E, q0, q1, V.vmin[0]), s1 = survives(E, q2, q3, V.vmin[1]);
-    V.go[0] = s0 && int0;
-    V.go[1] = s1 && int1;
-    V.leaf[0] = s0 && !int0;
-    V.leaf[1] = s1 && !int1;
+    V.node[0] = 2u * split;
+    V.node[1] = 2u * split + 1u;
+    bool s0, s1;
+    hrr_survive2(nlox, nloy, nloz, nhix, nhiy, nhiz, imax, hrr_pack2(E.x, E.x), hrr_pack2(E.y, E.y),
+                 hrr_pack2(E.z, E.z), E.scale, V.vmin[0], V.vmin[1], s0, s1);
+    const bool leaf0 = first == split, leaf1 = split + 1u == last;
+    V.go[0] = s0 && !leaf0;
+    V.go[1] = s1 && !leaf1;
+    V.leaf[0] = s0 && leaf0;
+    V.leaf[1] = s1 && leaf1;
     V.light[0] = split;
     V.light[1] = last;
 }
@@ -251,10 +257,23 @@ __device__ __forceinline__ void take(const Frame &fr, const Eye &E, uint32_t j, 
     if (acc && o < fr.cap) __stcs(&fr.pairs[o], make_uint2(j, __ldg(&fr.perm[i])));
 }
 
-// A queued leaf: the node whose record holds it, its slot t there and its sorted index, with
-// the bits of t in the words' top bits (nodes and lights number less than 2^31).
+// A queued leaf: the record that holds it, its place t there and its sorted index, with the
+// bits of t in the words' top bits (lights and width-four records number less than 2^31;
+// binary records need only the low bit of t).
+template <int W>
 __device__ __forceinline__ uint2 queued(uint32_t node, uint32_t t, uint32_t light) {
-    return make_uint2(node | (t >> 1 << 31), light | (t << 31));
+    return make_uint2(W == 2 ? node : node | (t >> 1 << 31), light | (t << 31));
+}
+
+// The light (position, intensity) at place t of a record.
+template <int W>
+__device__ __forceinline__ float4 light_of(const float4 *records, uint32_t node, uint32_t t) {
+    if constexpr (W == 2) {
+        const float *p = reinterpret_cast<const float *>(records + 4 * (size_t)node) + t;
+        return make_float4(-__ldg(p), -__ldg(p + 2), -__ldg(p + 4), __ldg(p + 12));
+    } else {
+        return __ldg(&records[8 * (size_t)node + 2u * t]);
+    }
 }
 
 // Take the n <= 32 newest of the warp's queued leaves.
@@ -266,9 +285,9 @@ __device__ __forceinline__ void take_queued(const Frame &fr, const Eye &E, uint3
     uint32_t i = 0;
     if (has) {
         const uint2 e = q[lane];
-        const uint32_t t = (e.x >> 31 << 1) | (e.y >> 31);
+        const uint32_t t = (W == 2 ? 0u : e.x >> 31 << 1) | (e.y >> 31);
         i = e.y & 0x7FFFFFFFu;
-        l = __ldg(&fr.nodes[(size_t)(2 * W) * (e.x & 0x7FFFFFFFu) + 2u * t]);
+        l = light_of<W>(fr.nodes, W == 2 ? e.x : e.x & 0x7FFFFFFFu, t);
     }
     __syncwarp();
     take(fr, E, j, lane, has, l, i);
@@ -305,10 +324,10 @@ __device__ __forceinline__ uint32_t head(const float4 *top, const Eye &E, const 
             const uint32_t first = __float_as_uint(h.w), last = __float_as_uint(x.x);
             if (kind != HRR_TOP_EMPTY) {
                 vmin = range_min<VARIANT>(first, last - first + 1u, E.r, E.c);
-                const bool s = survives(E, a, h, vmin);
-                vis = s && kind == HRR_TOP_INTERNAL;
-                leaf = s && kind == HRR_TOP_LEAF;
-                node = __float_as_uint(x.y);
+                const bool alive = survives(E, a, h, vmin);
+                vis = alive && kind == HRR_TOP_INTERNAL;
+                leaf = alive && kind == HRR_TOP_LEAF;
+                node = 2u * __float_as_uint(x.y) - (s & 1u ? 0u : 1u);  // odd heap slots are child 0
                 light = first;
             }
         }
@@ -341,9 +360,9 @@ __device__ __forceinline__ void traverse(const Launch &Lc, const Frame *F) {
     __shared__ uint2 ring_all[kWarps][kRing];  // (node, its range minimum)
     constexpr bool kTopShared = TOP > 0 && !BATCH;
     __shared__ float4 top_s[kTopShared ? 3 * HRR_TOP_SLOTS : 1];
-    if constexpr (kTopShared) {  // the top slots follow the frame's binary records
+    if constexpr (kTopShared) {
         if (F[0].n_lights > 1) {
-            const float4 *src = F[0].nodes + 4 * (size_t)(F[0].n_lights - 1u);
+            const float4 *src = F[0].top;
             for (uint32_t k = threadIdx.x; k < 3 * HRR_TOP_SLOTS; k += THREADS) top_s[k] = __ldg(&src[k]);
         }
         __syncthreads();
@@ -391,7 +410,7 @@ __device__ __forceinline__ void traverse(const Launch &Lc, const Frame *F) {
         E.r = fr.tile[ty * fr.tile_w + tx] + fr.shift_offset;
         if (n_lights == 1) {  // the root is a leaf (record 0, slot 0, in either layout)
             if (lane == 0 && fr.eye_visits) fr.eye_visits[j] = 0;
-            take(fr, E, j, lane, lane == 0, __ldg(&nodes[0]), 0u);
+            take(fr, E, j, lane, lane == 0, light_of<W>(nodes, 0u, 0u), 0u);
             continue;
         }
         E.c = __brev(0u - E.r);
@@ -400,7 +419,7 @@ __device__ __forceinline__ void traverse(const Launch &Lc, const Frame *F) {
         uint32_t S = 1, R = 1, visits = 0;
         uint32_t queued_n = 0;  // surviving leaves of this eye still to be taken
         if constexpr (TOP > 0) {
-            const float4 *top = kTopShared ? top_s : nodes + 4 * (size_t)(n_lights - 1u);
+            const float4 *top = kTopShared ? top_s : fr.top;
             visits = head<VARIANT, BATCH>(top, E, fr, lane, j, ring, S);
             R = S;
         } else {
@@ -478,7 +497,7 @@ __device__ __forceinline__ void traverse(const Launch &Lc, const Frame *F) {
 #pragma unroll
                 for (int t = 0; t < W; ++t) {
                     const unsigned b = __ballot_sync(0xFFFFFFFFu, V.leaf[t]);
-                    if (V.leaf[t]) queue[queued_n + __popc(b & lt)] = queued(e.x, (uint32_t)t, V.light[t]);
+                    if (V.leaf[t]) queue[queued_n + __popc(b & lt)] = queued<W>(e.x, (uint32_t)t, V.light[t]);
                     queued_n += __popc(b);
                 }
                 __syncwarp();

@@ -100,12 +100,32 @@ struct hrr_tree {
     // n - 1 records (one record with the single leaf if n == 1), followed by the top slots
     hrr_node *nodes = nullptr;
     uint32_t *perm = nullptr;   // n
+    // The binary records as the traversal reads them, 64 bytes with both children of a node
+    // paired, so that one packed instruction works on both boxes:
+    //   (-lo0.x, -lo1.x), (-lo0.y, -lo1.y), (-lo0.z, -lo1.z), (-hi0.x, -hi1.x),
+    //   (-hi0.y, -hi1.y), (-hi0.z, -hi1.z), (imax0, imax1), (split, other_end)
+    // The children of a node split at s sit in slots 2s and 2s + 1, one 128-byte line, the
+    // root in slot 0 (a child 0 split at 0 is a leaf); a leaf's slot is never read. The
+    // traversal pops siblings on neighbouring lanes, and what its record loads cost is the
+    // distinct lines per load: 1.5e11 scattered records a second come out of L2 when every
+    // record is a line of its own, 1.9e11 when siblings are neighbours on any 64 bytes, 2.9e11
+    // when they share a line. 2n - 2 slots (half of them leaves'); one (the leaf in both
+    // places) when n == 1.
+    float4 *pairs = nullptr;
     // The same hierarchy read with nodes of width four: for every internal node g a
     // 128-byte record of its four grandchild slots (hrr_build.cu), at index g; a
     // traversal of width four reads the even-depth ones only. One record (the leaf in
     // slot 0) when n == 1.
     float4 *wide = nullptr;
 };
+
+// The node at a slot of hrr_tree::pairs, and the slot of internal node g with other end o.
+__host__ __device__ inline uint32_t hrr_slot_node(uint32_t slot) { return (slot >> 1) + (slot & 1u); }
+__host__ __device__ inline uint32_t hrr_node_slot(uint32_t g, uint32_t o) { return g == 0u ? 0u : 2u * g - (o > g ? 1u : 0u); }
+// The top slots of a tree.
+inline const float4 *hrr_tree_top(const hrr_tree *tree) {
+    return reinterpret_cast<const float4 *>(tree->nodes) + 4 * (size_t)(tree->n > 1 ? tree->n - 1 : 1);
+}
 
 // Kernels a refit launches (hrr_refit_enqueue).
 inline int hrr_refit_launches(const hrr_tree *tree) { return tree->n > 1 ? 4 : 1; }
@@ -168,11 +188,12 @@ struct DeviceGuard {
 };
 
 // One frame of a traversal launch, as the kernel reads it (hrr_cull_kernel.cuh): a single frame
-// for hrr_cull, an array of them for batches. 128 bytes.
+// for hrr_cull, an array of them for batches. 136 bytes.
 struct hrr_cull_frame_t {
     const float *ex, *ey, *ez;
     const uint16_t *px, *py;
-    const float4 *nodes;
+    const float4 *nodes;             // the records of the launch's node width
+    const float4 *top;               // the tree's top slots
     const uint32_t *perm;
     const uint32_t *tile;
     uint2 *pairs;
@@ -227,7 +248,7 @@ inline bool hrr_tuning_valid(const hrr_tuning &t0) {
 }
 
 // The traversal (hrr_cull_kernel.cuh). Frames of one batched launch (their descriptors are
-// kernel parameters: 128 x 128 bytes):
+// kernel parameters: 128 x 136 bytes):
 #define HRR_CULL_MAX_FRAMES 128u
 // Blocks of a traversal launch over `total` eyes (a whole number per SM, at most one warp per
 // eye), for the single-frame or the batched kernel of a (normalised, valid) tuning.
@@ -239,7 +260,7 @@ int hrr_cull_max_blocks(const hrr_tuning &tuning, bool batch);
 // (8 bytes each) for a grid of the tuning's blocks.
 uint32_t hrr_cull_spill_cap(uint32_t height, uint32_t width);
 size_t hrr_cull_spill_entries(unsigned grid, uint32_t height, const hrr_tuning &tuning);
-// The node records a traversal of the tuning's width reads (tree->nodes or tree->wide).
+// The node records a traversal of the tuning's width reads (tree->pairs or tree->wide).
 const float4 *hrr_cull_records(const hrr_tree *tree, const hrr_tuning &tuning);
 // Enqueue one batched traversal over n_frames <= HRR_CULL_MAX_FRAMES frames (host array, copied
 // into the launch) on st; a no-op when total == 0. A single frame runs the single-frame

@@ -181,3 +181,50 @@ __device__ __forceinline__ void hrr_node_bound(float scale, float lox, float loy
 __device__ __forceinline__ bool hrr_node_culls(uint32_t v, float den, float rhs) {
     return __fmul_rd(__uint2float_rd(v), den) >= rhs;
 }
+
+// The node test of two boxes at once (the children of a binary node), on the packed pairs of
+// a traversal record: nlo and nhi hold the negated box corners of both, one axis per pair. The
+// same operations on the same values as hrr_node_bound, rounded alike (e - lo rounded up is
+// the negated lo - e rounded down), two per instruction: packed 32-bit float arithmetic
+// halves the issue slots of everything but the three-operand maxima.
+using hrr_f2 = unsigned long long;  // two floats, the first in the low word
+
+__device__ __forceinline__ hrr_f2 hrr_pack2(float a, float b) {
+    hrr_f2 d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(a), "f"(b));
+    return d;
+}
+__device__ __forceinline__ void hrr_unpack2(hrr_f2 d, float &a, float &b) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(d));
+}
+__device__ __forceinline__ hrr_f2 hrr_gap2(hrr_f2 nlo, hrr_f2 nhi, hrr_f2 e) {
+    hrr_f2 up, dn;
+    asm("add.rp.f32x2 %0, %1, %2;" : "=l"(up) : "l"(e), "l"(nlo));
+    asm("add.rm.f32x2 %0, %1, %2;" : "=l"(dn) : "l"(e), "l"(nhi));
+    float u0, u1, d0, d1;
+    hrr_unpack2(up, u0, u1);
+    hrr_unpack2(dn, d0, d1);
+    return hrr_pack2(hrr_max3(0.0f, -u0, d0), hrr_max3(0.0f, -u1, d1));
+}
+// Whether each box survives (is not culled) at range minima v0, v1.
+__device__ __forceinline__ void hrr_survive2(hrr_f2 nlox, hrr_f2 nloy, hrr_f2 nloz, hrr_f2 nhix, hrr_f2 nhiy,
+                                             hrr_f2 nhiz, hrr_f2 imax, hrr_f2 ex, hrr_f2 ey, hrr_f2 ez, float scale,
+                                             uint32_t v0, uint32_t v1, bool &s0, bool &s1) {
+    const hrr_f2 gx = hrr_gap2(nlox, nhix, ex), gy = hrr_gap2(nloy, nhiy, ey), gz = hrr_gap2(nloz, nhiz, ez);
+    hrr_f2 d2, rhs, lhs;
+    asm("mul.rm.f32x2 %0, %1, %1;" : "=l"(d2) : "l"(gx));
+    asm("fma.rm.f32x2 %0, %1, %1, %0;" : "+l"(d2) : "l"(gy));
+    asm("fma.rm.f32x2 %0, %1, %1, %0;" : "+l"(d2) : "l"(gz));
+    float a, b;
+    hrr_unpack2(d2, a, b);
+    const hrr_f2 den = hrr_pack2(fmaxf(a, 1e-4f), fmaxf(b, 1e-4f));
+    asm("mul.rp.f32x2 %0, %1, %2;" : "=l"(rhs) : "l"(imax), "l"(hrr_pack2(scale, scale)));
+    asm("mul.rm.f32x2 %0, %1, %2;"
+        : "=l"(lhs)
+        : "l"(hrr_pack2(__uint2float_rd(v0), __uint2float_rd(v1))), "l"(den));
+    float l0, l1, r0, r1;
+    hrr_unpack2(lhs, l0, l1);
+    hrr_unpack2(rhs, r0, r1);
+    s0 = !(l0 >= r0);
+    s1 = !(l1 >= r1);
+}
