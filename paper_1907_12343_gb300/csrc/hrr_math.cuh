@@ -116,6 +116,19 @@ __device__ __forceinline__ uint32_t hrr_range_min_value(uint32_t a, uint32_t L, 
     return __vimin3_u32(__brev(i0) + r, __brev(j0) + r, __brev(k1) + r);
 }
 
+// The same for the leaves [a, z] of a hierarchy (a <= z < 2^31, so nothing below overflows): a
+// candidate past the end may be replaced by any index of the range, so the second index of
+// either class is clamped to z instead of tested, and both of the second class are tried.
+__device__ __forceinline__ uint32_t hrr_range_min_leaves(uint32_t a, uint32_t z, uint32_t r, uint32_t T, uint32_t c) {
+    uint32_t s;  // 31 - floor(log2(z - a + 1))
+    asm("bfind.shiftamt.u32 %0, %1;" : "=r"(s) : "r"(z - a + 1u));
+    const uint32_t mh = 0x7FFFFFFFu >> s;
+    const uint32_t c2 = __brev(T + (2u << s));
+    const uint32_t i0 = a + ((c - a) & mh), i1 = a + ((c2 - a) & mh);
+    const uint32_t j0 = min(i0 + mh + 1u, z), j1 = min(i1 + mh + 1u, z);
+    return min(__vimin3_u32(__brev(i0) + r, __brev(j0) + r, __brev(i1) + r), __brev(j1) + r);
+}
+
 // Exact per-pair test (round to nearest, canonical order, no FMA): accept iff
 // xi < ceil(p 2^32), p = min(1, (tau I) / max(d2, 1e-4)). For 0 < p < 1, p 2^32 is an
 // exact float below 2^32, so its ceiling fits in 32 bits. The traversals ask it only about
@@ -206,10 +219,10 @@ __device__ __forceinline__ hrr_f2 hrr_gap2(hrr_f2 nlo, hrr_f2 nhi, hrr_f2 e) {
     hrr_unpack2(dn, d0, d1);
     return hrr_pack2(hrr_max3(0.0f, -u0, d0), hrr_max3(0.0f, -u1, d1));
 }
-// Whether each box survives (is not culled) at range minima v0, v1.
+// Whether each box survives (is not culled) at range minima v0, v1, where `ok`.
 __device__ __forceinline__ void hrr_survive2(hrr_f2 nlox, hrr_f2 nloy, hrr_f2 nloz, hrr_f2 nhix, hrr_f2 nhiy,
                                              hrr_f2 nhiz, hrr_f2 imax, hrr_f2 ex, hrr_f2 ey, hrr_f2 ez, float scale,
-                                             uint32_t v0, uint32_t v1, bool &s0, bool &s1) {
+                                             uint32_t v0, uint32_t v1, bool ok, bool &s0, bool &s1) {
     const hrr_f2 gx = hrr_gap2(nlox, nhix, ex), gy = hrr_gap2(nloy, nhiy, ey), gz = hrr_gap2(nloz, nhiz, ez);
     hrr_f2 d2, rhs, lhs;
     asm("mul.rm.f32x2 %0, %1, %1;" : "=l"(d2) : "l"(gx));
@@ -225,6 +238,6 @@ __device__ __forceinline__ void hrr_survive2(hrr_f2 nlox, hrr_f2 nloy, hrr_f2 nl
     float l0, l1, r0, r1;
     hrr_unpack2(lhs, l0, l1);
     hrr_unpack2(rhs, r0, r1);
-    s0 = !(l0 >= r0);
-    s1 = !(l1 >= r1);
+    s0 = ok && !(l0 >= r0);
+    s1 = ok && !(l1 >= r1);
 }
