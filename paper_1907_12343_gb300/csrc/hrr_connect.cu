@@ -6,33 +6,50 @@
 // times the visibility of the open segment eye -> light against a triangle scene. The
 // per-eye sums of the weights are unbiased estimates of the eyes' unculled sums.
 //
-// The scene is a bounding-volume hierarchy over the triangles: the light-hierarchy builder
-// orders the triangles by the Morton keys of their centroids and builds the same binary
-// radix tree over them; a refit then replaces the records' point boxes with triangle
-// boxes, widened so that floating-point slab tests can never reject a box that holds a
-// crossing. Each lane of a persistent grid traces one pair's shadow segment at a time (any
-// hit ends it) and takes the next pair when it is done.
+// The scene is a bounding-volume hierarchy over the triangles: the Morton order of their
+// centroids, the binary radix tree over it and the box pass of the light hierarchies (with
+// triangle boxes, widened so that floating-point slab tests can never reject a box that holds a
+// crossing) give a binary tree, and every three levels of it become one node of eight children
+// whose boxes are stored in seven bits a side, rounded outwards (Scene nodes, below). Each lane of
+// a persistent grid traces one pair's shadow segment at a time (any hit ends it) and takes the
+// next pair when it is done.
 #include <algorithm>
 #include <new>
 
+#include "hrr_boxes.cuh"
 #include "hrr_internal.cuh"
+#include "hrr_order.cuh"
+#include "hrr_sort.cuh"
 
 struct hrr_scene {
     int device = 0;
     uint32_t n = 0;
-    hrr_tree *tree = nullptr;  // records: child boxes of the triangles; perm: sorted -> original
+    uint32_t *nodes = nullptr;  // n - 1 nodes of kNodeWords words (below); one when n == 1
     float *tris = nullptr;     // sorted triangles, 16 floats each: v0, e1 = v1 - v0, e2 = v2 - v0, pad
 };
 
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kStack = 128;  // >= height of the radix tree (at most 96) + 2
 constexpr int kTriFloats = 16;  // a sorted triangle's stride (64 bytes: aligned 256-bit loads)
 
+// Scene nodes. Node g holds the up to eight nodes or triangles three levels below binary node g
+// (a leaf met on the way stands for itself), in one 128-byte line of which 96 bytes are read:
+//   words 0-2   origin o of the node's box grid
+//   word 3      bytes: exponents of S = 2^(k-127) per axis (x, y, z), mask of the children there are
+//   words 4-15  per axis: 8 low sides, 8 high sides, a byte 0x80 | q each; the side lies at
+//               o + q S / 128, so 1 + q / 128 is one byte permutation away from a float
+//   words 16-23 children: a triangle (bit 31 set) or a node
+// A binary walk over 64-byte nodes was bound by its scattered loads (93% of the L1 data pipe, 87 loads
+// a segment); this one is bound by instructions (70% of the issue slots at 32 warps per SM, L1 at
+// 55%). 8.3e6 segments against 2^18 triangles, scene build included: 6.35 -> 4.54 ms.
+constexpr uint32_t kNodeWords = 32;
+constexpr uint32_t kTriangle = 0x80000000u;
+constexpr int kSharedStack = 24;   // entries of a segment's stack in shared memory
+constexpr int kLocalStack = 232;   // ... and below them: 7 per level of at most 33, and a margin
+
 __global__ void __launch_bounds__(kThreads) centroid_kernel(const float *__restrict__ tri, uint32_t n,
-                                                             float *cx, float *cy, float *cz, float *zero,
-                                                             unsigned long long *flags) {
+                                                             float *cx, float *cy, float *cz, unsigned long long *flags) {
     const uint32_t i = blockIdx.x * kThreads + threadIdx.x;
     if (i >= n) return;
     const float *t = tri + 9 * (size_t)i;
@@ -42,10 +59,10 @@ __global__ void __launch_bounds__(kThreads) centroid_kernel(const float *__restr
         if (!isfinite(a) || !isfinite(b) || !isfinite(d)) atomicOr(flags, HRR_FLAG_NONFINITE);
         s[c] = (a + b + d) * (1.0f / 3.0f);
     }
+    if (!isfinite(s[0]) || !isfinite(s[1]) || !isfinite(s[2])) atomicOr(flags, HRR_FLAG_NONFINITE);
     cx[i] = s[0];
     cy[i] = s[1];
     cz[i] = s[2];
-    zero[i] = 0.0f;
 }
 
 // A box that surely holds a triangle: its vertices' bounds widened by 2^-16 of the
@@ -61,72 +78,120 @@ __device__ __forceinline__ void tri_box(const float *t, float lo[3], float hi[3]
     }
 }
 
-__device__ __forceinline__ void store_box(hrr_node *node, uint32_t slot, const float lo[3], const float hi[3]) {
-    float *f = reinterpret_cast<float *>(node) + (slot ? 8 : 0);
-    f[0] = lo[0]; f[1] = lo[1]; f[2] = lo[2]; f[3] = 0.0f;
-    f[4] = hi[0]; f[5] = hi[1]; f[6] = hi[2];
-}
-
-// Sorted triangles, and the bottom-up refit of the records with triangle boxes (the same
-// arrival scheme as the light refit: the second child to arrive finishes its parent).
-__global__ void __launch_bounds__(kThreads) tri_refit_kernel(const float *__restrict__ tri, const uint32_t *perm,
-                                                             uint32_t n, hrr_node *nodes, float *sorted,
-                                                             const uint32_t *__restrict__ leaf_parent,
-                                                             const uint32_t *__restrict__ int_parent,
-                                                             uint32_t *arrivals, unsigned long long *flags) {
-    const uint32_t leaf = blockIdx.x * kThreads + threadIdx.x;
-    if (leaf >= n) return;
-    const float *t = tri + 9 * (size_t)perm[leaf];
-    // v0 and the edges e1, e2 (the segment test's first six roundings, done once here), so
-    // that one 256-bit load and one 32-bit load fetch a triangle
-    float *o = sorted + kTriFloats * (size_t)leaf;
-    o[0] = t[0]; o[1] = t[1]; o[2] = t[2];
-    o[3] = __fsub_rn(t[3], t[0]); o[4] = __fsub_rn(t[4], t[1]); o[5] = __fsub_rn(t[5], t[2]);
-    o[6] = __fsub_rn(t[6], t[0]); o[7] = __fsub_rn(t[7], t[1]); o[8] = __fsub_rn(t[8], t[2]);
-    for (int c = 9; c < kTriFloats; ++c) o[c] = 0.0f;
-    float lo[3], hi[3];
-    tri_box(t, lo, hi);
-    if (n == 1) {
-        store_box(nodes, 0, lo, hi);
-        store_box(nodes, 1, lo, hi);
-        return;
-    }
-    uint32_t code = leaf_parent[leaf];
-    for (;;) {
-        const uint32_t node = code >> 1, slot = code & 1u;
-        if (code == 0xFFFFFFFFu || node >= n - 1) {
-            atomicOr(flags, HRR_FLAG_TOPOLOGY);
-            return;
-        }
-        store_box(&nodes[node], slot, lo, hi);
-        __threadfence();
-        if (atomicAdd(&arrivals[node], 1u) == 0u) return;
-        __threadfence();
-        const float *f = reinterpret_cast<const float *>(&nodes[node]);
-        for (int c = 0; c < 3; ++c) {
-            lo[c] = fminf(__ldcg(f + c), __ldcg(f + 8 + c));
-            hi[c] = fmaxf(__ldcg(f + 4 + c), __ldcg(f + 12 + c));
-        }
-        if (node == 0) return;
-        code = int_parent[node];
-    }
-}
-
-__global__ void __launch_bounds__(kThreads) scene_links_kernel(const hrr_node *__restrict__ nodes, uint32_t n,
-                                                               uint32_t *__restrict__ leaf_parent,
-                                                               uint32_t *__restrict__ int_parent,
-                                                               unsigned long long *flags) {
+// Sorted triangles (v0 and the edges e1, e2, the segment test's first six roundings, done once
+// here, so that one 256-bit load and one 32-bit load fetch a triangle) and their boxes.
+__global__ void __launch_bounds__(kThreads) triangles_kernel(const float *__restrict__ tri, const uint32_t *__restrict__ perm,
+                                                             uint32_t n, float *__restrict__ sorted,
+                                                             float4 *__restrict__ box) {
     const uint32_t i = blockIdx.x * kThreads + threadIdx.x;
-    if (i >= n - 1) return;
-    const uint32_t s = nodes[i].split, j = nodes[i].other_end;
-    const uint32_t first = min(i, j), last = max(i, j);
-    if (last >= n || s < first || s >= last) {
-        atomicOr(flags, HRR_FLAG_TOPOLOGY);
-        return;
+    if (i >= n) return;
+    const float *t = tri + 9 * (size_t)(perm ? perm[i] : i);
+    float v[9];
+    for (int c = 0; c < 9; ++c) v[c] = t[c];
+    float4 *o = reinterpret_cast<float4 *>(sorted + kTriFloats * (size_t)i);
+    store32(o, make_float4(v[0], v[1], v[2], __fsub_rn(v[3], v[0])),
+            make_float4(__fsub_rn(v[4], v[1]), __fsub_rn(v[5], v[2]), __fsub_rn(v[6], v[0]), __fsub_rn(v[7], v[1])));
+    store32(o + 2, make_float4(__fsub_rn(v[8], v[2]), 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f));
+    float lo[3], hi[3];
+    tri_box(v, lo, hi);
+    if (box) store32(box + 2 * (size_t)i, make_float4(lo[0], lo[1], lo[2], 0.f), make_float4(hi[0], hi[1], hi[2], 0.f));
+}
+
+// Leaves that are boxes.
+struct BoxLeaves {
+    const float4 *box;
+    __device__ __forceinline__ Box operator()(uint32_t i) const { return box_of(box[2 * (size_t)i], box[2 * (size_t)i + 1]); }
+};
+
+// One node of eight children per binary node (those that no traversal reaches as well: they are
+// cheaper made than told apart). The grid's step s = S / 128 leaves the box 124 steps, its origin
+// lies a 64th of a step below the box, and every side moves outwards by a 128th of a step before
+// it is rounded outwards: more than the rounding of the segment's slab arithmetic on a grid near
+// the eye (2^-16 of the grid; far from it the slab test's own widening covers it).
+__global__ void __launch_bounds__(kThreads) collapse_kernel(const float4 *__restrict__ nodes, uint32_t n,
+                                                            uint32_t *__restrict__ out, const unsigned long long *flags) {
+    const uint32_t g = blockIdx.x * kThreads + threadIdx.x;
+    if (g >= n - 1 || (*flags & (HRR_FLAG_NONFINITE | HRR_FLAG_RUNS | HRR_FLAG_TOPOLOGY))) return;
+    float4 lo[8], hi[8];
+    uint32_t f[8], l[8], id[8];  // ranges and node numbers; an empty place has f > l
+    for (int k = 0; k < 8; ++k) {
+        f[k] = 1;
+        l[k] = 0;
+        id[k] = 0;
+        lo[k] = hi[k] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    const uint32_t code = i << 1;
-    if (first == s) leaf_parent[s] = code; else int_parent[s] = code;
-    if (last == s + 1) leaf_parent[s + 1] = code | 1u; else int_parent[s + 1] = code | 1u;
+    {
+        const uint32_t other = __float_as_uint(nodes[4 * (size_t)g + 3].w);
+        f[0] = min(g, other);
+        l[0] = max(g, other);
+        id[0] = g;
+    }
+#pragma unroll
+    for (int step = 4; step >= 1; step >>= 1) {  // places 0, 2 step, 4 step, ... split into two
+#pragma unroll
+        for (int k = 0; k < 8; k += 2 * step) {
+            if (f[k] >= l[k]) continue;  // empty, or a leaf: it keeps its place
+            const float4 *r = nodes + 4 * (size_t)id[k];
+            const float4 r1 = r[1];
+            const uint32_t split = __float_as_uint(r1.w);
+            lo[k + step] = r[2];
+            hi[k + step] = r[3];
+            f[k + step] = split + 1u;
+            l[k + step] = l[k];
+            id[k + step] = split + 1u;
+            lo[k] = r[0];
+            hi[k] = r1;
+            l[k] = split;
+            id[k] = split;
+        }
+    }
+    float a[3] = {1e38f, 1e38f, 1e38f}, b[3] = {-1e38f, -1e38f, -1e38f};
+    for (int k = 0; k < 8; ++k)
+        if (f[k] <= l[k]) {
+            a[0] = fminf(a[0], lo[k].x); a[1] = fminf(a[1], lo[k].y); a[2] = fminf(a[2], lo[k].z);
+            b[0] = fmaxf(b[0], hi[k].x); b[1] = fmaxf(b[1], hi[k].y); b[2] = fmaxf(b[2], hi[k].z);
+        }
+    uint32_t w[24];
+    w[3] = 0;
+    for (int c = 0; c < 3; ++c) {
+        // s = 2^m, the least with 124 s >= the extent, at least 2^-112; past 2^119 (and for a box
+        // that is not finite) the axis gets S = infinity, whose sides are no numbers, and the slab
+        // test goes by the other axes
+        int m = min((int)((__float_as_uint(fmaxf((b[c] - a[c]) * (1.0f / 124.0f), 0x1p-113f)) >> 23) & 255u) - 126, 119);
+        float s, o;
+        for (;; ++m) {
+            s = __uint_as_float((uint32_t)(m + 127) << 23);
+            o = __fsub_rd(a[c], s * 0.015625f);
+            if (__fsub_ru(b[c], o) <= 126.0f * s || m >= 119) break;
+        }
+        const bool covered = __fsub_ru(b[c], o) <= 126.0f * s;
+        w[c] = covered ? __float_as_uint(o) : 0u;
+        w[3] |= (covered ? (uint32_t)(m + 7 + 127) : 255u) << (8 * c);
+        const float inv = __uint_as_float((uint32_t)(127 - m) << 23);
+        uint32_t ql[2] = {0, 0}, qh[2] = {0, 0};
+        for (int k = 0; k < 8; ++k) {
+            const float x = c == 0 ? lo[k].x : c == 1 ? lo[k].y : lo[k].z, y = c == 0 ? hi[k].x : c == 1 ? hi[k].y : hi[k].z;
+            const float u = fminf(fmaxf(floorf(__fsub_rd(x, o) * inv - 0.0078125f), 0.0f), 127.0f);
+            const float v = fminf(fmaxf(ceilf(__fsub_ru(y, o) * inv + 0.0078125f), 0.0f), 127.0f);
+            ql[k >> 2] |= (0x80u | (uint32_t)u) << (8 * (k & 3));
+            qh[k >> 2] |= (0x80u | (uint32_t)v) << (8 * (k & 3));
+        }
+        w[4 + 4 * c] = ql[0];
+        w[5 + 4 * c] = ql[1];
+        w[6 + 4 * c] = qh[0];
+        w[7 + 4 * c] = qh[1];
+    }
+    for (int k = 0; k < 8; ++k) {
+        if (f[k] <= l[k]) w[3] |= 1u << (24 + k);
+        w[16 + k] = f[k] == l[k] ? kTriangle | f[k] : id[k];
+    }
+    float4 *to = reinterpret_cast<float4 *>(out + kNodeWords * (size_t)g);
+    for (int k = 0; k < 3; ++k)
+        store32(to + 2 * k,
+                make_float4(__uint_as_float(w[8 * k]), __uint_as_float(w[8 * k + 1]), __uint_as_float(w[8 * k + 2]),
+                            __uint_as_float(w[8 * k + 3])),
+                make_float4(__uint_as_float(w[8 * k + 4]), __uint_as_float(w[8 * k + 5]), __uint_as_float(w[8 * k + 6]),
+                            __uint_as_float(w[8 * k + 7])));
 }
 
 // Open segment e -> e + D, t in (1e-4, 1 - 1e-4), against the closed triangle (v0, v1, v2),
@@ -157,26 +222,60 @@ __device__ __forceinline__ bool segment_hits(const float e[3], const float D[3],
     return t > 1e-4f && t < 1.0f - 1e-4f;
 }
 
-// Slab test of the segment's [0, 1] against a box, widened by 2^-20 on both ends.
-__device__ __forceinline__ bool box_hit(const float e[3], const float inv[3], const float lo[3], const float hi[3]) {
-    float tn = 0.0f, tf = 1.0f;
-    for (int c = 0; c < 3; ++c) {
-        const float a = (lo[c] - e[c]) * inv[c], b = (hi[c] - e[c]) * inv[c];
-        tn = fmaxf(tn, fminf(a, b));
-        tf = fminf(tf, fmaxf(a, b));
-    }
-    return tn * (1.0f - 9.5367431640625e-07f) <= tf * (1.0f + 9.5367431640625e-07f);
+// 32 bytes of a node as one 256-bit read-only load that does not allocate in L1 (scattered
+// nodes are rarely reused from L1; filling it would cost L1 data-pipe cycles).
+__device__ __forceinline__ void load8(const uint32_t *p, uint32_t (&v)[8]) {
+    asm("ld.global.nc.L1::no_allocate.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+        : "l"(p));
 }
-
-// One 64-byte record as two 256-bit read-only loads that do not allocate in L1 (scattered
-// records are rarely reused from L1; filling it would cost L1 data-pipe cycles).
-__device__ __forceinline__ void load_record(const float4 *p, float4 &q0, float4 &q1, float4 &q2, float4 &q3) {
-    asm("ld.global.nc.L1::no_allocate.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-        : "=f"(q0.x), "=f"(q0.y), "=f"(q0.z), "=f"(q0.w), "=f"(q1.x), "=f"(q1.y), "=f"(q1.z), "=f"(q1.w)
-        : "l"(p));
-    asm("ld.global.nc.L1::no_allocate.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8+32];"
-        : "=f"(q2.x), "=f"(q2.y), "=f"(q2.z), "=f"(q2.w), "=f"(q3.x), "=f"(q3.y), "=f"(q3.z), "=f"(q3.w)
-        : "l"(p));
+// min(a, b, c) in one instruction; a NaN operand is ignored.
+__device__ __forceinline__ float min3(float a, float b, float c) {
+    float d;
+    asm("min.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
+}
+// Times at which the segment passes one axis' near and far sides of child k (k & 3 in the words).
+__device__ __forceinline__ void sides(uint32_t near, uint32_t far, int k, hrr_f2 slope, hrr_f2 start, float &tn, float &tf) {
+    // bytes (0, 0, 0x80 | q, 0x3f): 1 + q / 128
+    const uint32_t sel = 0x7044u | ((uint32_t)k << 8);
+    const hrr_f2 v = hrr_pack2(__uint_as_float(__byte_perm(near, 0x3F000000u, sel)),
+                               __uint_as_float(__byte_perm(far, 0x3F000000u, sel)));
+    hrr_f2 t;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(t) : "l"(v), "l"(slope), "l"(start));
+    hrr_unpack2(t, tn, tf);
+}
+// The children of a node that the segment's [0, 1] meets (slab test, widened by 2^-18).
+__device__ __forceinline__ uint32_t meets(const uint32_t (&h)[8], const uint32_t (&q)[8], const float (&e)[3],
+                                          const float (&inv)[3]) {
+    hrr_f2 slope[3], start[3];
+    uint32_t near[3][2], far[3][2];
+    const uint32_t side[3][4] = {{h[4], h[5], h[6], h[7]}, {q[0], q[1], q[2], q[3]}, {q[4], q[5], q[6], q[7]}};
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const float S = __uint_as_float(((h[3] >> (8 * c)) & 255u) << 23);
+        const float a = S * inv[c];
+        const float b = ((__uint_as_float(h[c]) - S) - e[c]) * inv[c];
+        slope[c] = hrr_pack2(a, a);
+        start[c] = hrr_pack2(b, b);
+        const bool back = inv[c] < 0.0f;
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            near[c][k] = back ? side[c][2 + k] : side[c][k];
+            far[c][k] = back ? side[c][k] : side[c][2 + k];
+        }
+    }
+    uint32_t mask = 0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        float xn, xf, yn, yf, zn, zf;
+        sides(near[0][k >> 2], far[0][k >> 2], k & 3, slope[0], start[0], xn, xf);
+        sides(near[1][k >> 2], far[1][k >> 2], k & 3, slope[1], start[1], yn, yf);
+        sides(near[2][k >> 2], far[2][k >> 2], k & 3, slope[2], start[2], zn, zf);
+        const float tn = fmaxf(hrr_max3(xn, yn, zn), 0.0f), tf = fminf(min3(xf, yf, zf), 1.0f);
+        if (tn <= tf * (1.0f + 0x1p-18f)) mask |= 1u << k;
+    }
+    return mask & (h[3] >> 24);
 }
 
 struct ConnectArgs {
@@ -187,7 +286,7 @@ struct ConnectArgs {
     float tau;
     const uint2 *pairs;
     unsigned long long n_pairs;
-    const float4 *nodes;  // scene, or NULL
+    const uint32_t *nodes;  // scene, or NULL
     const float *tris;    // sorted triangles, kTriFloats each
     uint32_t n_tris;
     float *weight;        // per pair, or NULL
@@ -287,20 +386,28 @@ __global__ void __launch_bounds__(kThreads) weights_kernel(const ConnectArgs A, 
     }
 }
 
-// Persistent segments: each lane traces one pair's segment, one hierarchy node per step,
-// and a warp refills its idle lanes from the global pair cursor (one atomic per refill), so
-// lanes do not idle behind the warp's longest segment. A segment ends at its first
-// crossing (occluded) or when its stack runs dry (visible).
+// Persistent segments: each lane traces one pair's segment, at most one node and one triangle per
+// step, and a warp refills its idle lanes from the global pair cursor (one atomic per refill), so
+// lanes do not idle behind the warp's longest segment. A segment ends at its first crossing
+// (occluded) or when its stack runs dry (visible). The stack's first entries are in shared memory,
+// interleaved by lane (no bank conflicts whatever the depths). Letting nodes and triangles take
+// turns warp by warp (triangles only when 8, 12, 16 or 20 lanes had one) left too many lanes
+// waiting: 5.1 to 6.0 ms against 4.5; refilling below 16 or 28 busy lanes 4.6 and 4.8 ms.
 __global__ void __launch_bounds__(kThreads) connect_kernel(const ConnectArgs A) {
+    __shared__ uint32_t stack_all[kSharedStack][kThreads];
+    uint32_t deep[kLocalStack];
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
     bool alive = false, more = true;
     unsigned long long k = 0;
-    uint32_t j = 0, node = 0, steps = 0;
+    uint32_t j = 0, cur = 0, steps = 0;
     int sp = 0;
     float w = 0.0f;
     float e[3] = {0.f, 0.f, 0.f}, D[3] = {0.f, 0.f, 0.f}, inv[3] = {0.f, 0.f, 0.f};
-    uint32_t stack[kStack];
+    auto pop = [&]() {
+        --sp;
+        return sp < kSharedStack ? stack_all[sp][threadIdx.x] : deep[sp - kSharedStack];
+    };
     for (;;) {
         unsigned alive_mask = __ballot_sync(0xFFFFFFFFu, alive);
         if (more && (uint32_t)__popc(alive_mask) < kRefillBelow) {
@@ -328,17 +435,13 @@ __global__ void __launch_bounds__(kThreads) connect_kernel(const ConnectArgs A) 
                         const float den = fmaxf(d2, 1e-4f);
                         const float p = fminf(1.0f, __fdiv_rn(__fmul_rn(A.tau, inten), den));
                         w = __fdiv_rn(__fdiv_rn(inten, den), p);
-                        if (A.n_tris == 1) {
-                            finish(A, k, j, w, !segment_hits(e, D, A.tris));
-                        } else {
-                            // a zero component is taken as 1e-30: its slab then admits exactly
-                            // the boxes whose range holds e (up to 1e-30, a conservative margin)
-                            for (int c = 0; c < 3; ++c) inv[c] = __frcp_rn(D[c] == 0.0f ? 1e-30f : D[c]);
-                            node = 0;
-                            sp = 0;
-                            steps = 0;
-                            alive = true;
-                        }
+                        // a zero component is taken as 1e-30: its slab then admits exactly
+                        // the boxes whose range holds e (up to 1e-30, a conservative margin)
+                        for (int c = 0; c < 3; ++c) inv[c] = __frcp_rn(D[c] == 0.0f ? 1e-30f : D[c]);
+                        cur = A.n_tris == 1 ? kTriangle : 0u;
+                        sp = 0;
+                        steps = 0;
+                        alive = true;
                     }
                 }
             }
@@ -346,46 +449,129 @@ __global__ void __launch_bounds__(kThreads) connect_kernel(const ConnectArgs A) 
         }
         if (alive_mask == 0u && !more) break;
         if (!alive) continue;
-        float4 q0, q1, q2, q3;
-        load_record(&A.nodes[4 * (size_t)node], q0, q1, q2, q3);
-        const uint32_t split = __float_as_uint(q1.w), other = __float_as_uint(q3.w);
-        const uint32_t first = min(node, other), last = max(node, other);
-        if (last >= A.n_tris || split < first || split >= last || sp >= kStack || ++steps >= A.n_tris) {
-            // corrupt records: out-of-range links, an impossible depth, or more steps than
-            // the hierarchy has internal nodes
-            atomicOr(A.flags, HRR_FLAG_TOPOLOGY);
-            alive = false;
-            continue;
+        bool have = true, hit = false;  // cur is still to be looked at; the segment is blocked
+        if (!(cur & kTriangle)) {
+            // corrupt nodes: out-of-range links, an impossible depth, or more steps than there
+            // are nodes
+            if (cur >= A.n_tris - 1u || ++steps >= A.n_tris || sp > kSharedStack + kLocalStack - 8) {
+                atomicOr(A.flags, HRR_FLAG_TOPOLOGY);
+                alive = false;
+                continue;
+            }
+            uint32_t h[8], q[8], ref[8];
+            const uint32_t *node = A.nodes + kNodeWords * (size_t)cur;
+            load8(node, h);
+            load8(node + 8, q);
+            load8(node + 16, ref);
+            const uint32_t mask = meets(h, q, e, inv);
+            if (sp <= kSharedStack - 8) {
+                uint32_t *at = &stack_all[sp][threadIdx.x];
+#pragma unroll
+                for (int c = 0; c < 8; ++c)
+                    if ((mask >> c) & 1u) {
+                        *at = ref[c];
+                        at += kThreads;
+                    }
+            } else {
+                int s = sp;
+#pragma unroll
+                for (int c = 0; c < 8; ++c)
+                    if ((mask >> c) & 1u) {
+                        if (s < kSharedStack) stack_all[s][threadIdx.x] = ref[c];
+                        else deep[s - kSharedStack] = ref[c];
+                        ++s;
+                    }
+            }
+            sp += __popc(mask);
+            have = sp > 0;
+            if (have) cur = pop();
         }
-        const float lo0[3] = {q0.x, q0.y, q0.z}, hi0[3] = {q1.x, q1.y, q1.z};
-        const float lo1[3] = {q2.x, q2.y, q2.z}, hi1[3] = {q3.x, q3.y, q3.z};
-        const bool h0 = box_hit(e, inv, lo0, hi0), h1 = box_hit(e, inv, lo1, hi1);
-        const bool leaf0 = first == split, leaf1 = split + 1 == last;
-        bool hit = false;
-        if (h0 && leaf0) {
-            hit = segment_hits(e, D, A.tris + kTriFloats * (size_t)split);
+        if (have && (cur & kTriangle)) {
+            const uint32_t i = cur & ~kTriangle;
+            if (i >= A.n_tris) {
+                atomicOr(A.flags, HRR_FLAG_TOPOLOGY);
+                alive = false;
+                continue;
+            }
+            hit = segment_hits(e, D, A.tris + kTriFloats * (size_t)i);
+            have = sp > 0;
+            if (have && !hit) cur = pop();
         }
-        if (!hit && h1 && leaf1) {
-            hit = segment_hits(e, D, A.tris + kTriFloats * (size_t)(split + 1));
-        }
-        const bool go0 = h0 && !leaf0, go1 = h1 && !leaf1;
-        if (hit) {
-            finish(A, k, j, w, false);
-            alive = false;
-        } else if (go0 && go1) {
-            stack[sp++] = split + 1;
-            node = split;
-        } else if (go0) {
-            node = split;
-        } else if (go1) {
-            node = split + 1;
-        } else if (sp > 0) {
-            node = stack[--sp];
-        } else {
-            finish(A, k, j, w, true);
+        if (hit || !have) {
+            finish(A, k, j, w, !hit);
             alive = false;
         }
     }
+}
+
+// Sorts by the key bits from `shift` up, as the light builder does.
+int scene_attempt(hrr_ctx *ctx, const float *tris, uint32_t n, hrr_scene *sc, int shift) {
+    cudaStream_t st = ctx->stream;
+    const size_t un = n;
+    unsigned long long *flags = ctx->counters + 2;
+    const size_t bytes = 3 * pad256(sizeof(float) * un) + 2 * pad256(sizeof(uint64_t) * un) + 2 * pad256(sizeof(uint32_t) * un) +
+                         pad256(sort_scratch_bytes(un)) + pad256(sizeof(float4) * un) + pad256(2 * sizeof(float4) * un) +
+                         pad256(sizeof(hrr_node) * un) + box_scratch_bytes(n);
+    char *scratch = nullptr;
+    HRR_CUDA(ctx, hrr_alloc(ctx, &scratch, bytes));
+    char *p = scratch;
+    float *cx = carve<float>(p, un), *cy = carve<float>(p, un), *cz = carve<float>(p, un);
+    uint64_t *keys0 = carve<uint64_t>(p, un), *keys1 = carve<uint64_t>(p, un);
+    uint32_t *vals0 = carve<uint32_t>(p, un), *perm = carve<uint32_t>(p, un);
+    const SortScratch ss = carve_sort(p, un);
+    float4 *spos = carve<float4>(p, un), *box = carve<float4>(p, 2 * un);
+    hrr_node *nodes = carve<hrr_node>(p, un);
+    const BoxScratch bs = carve_boxes(p, n);
+    const unsigned g = (unsigned)((un + kThreads - 1) / kThreads);
+    cudaError_t e = cudaMemsetAsync(flags, 0, sizeof(unsigned long long), st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(ss.hist, 0, sort_scratch_bytes(un), st);
+    if (e == cudaSuccess) {
+        centroid_kernel<<<g, kThreads, 0, st>>>(tris, n, cx, cy, cz, flags);
+        const int passes = sort_passes(shift);
+        morton_kernel<<<morton_grid(n), kThreads, 0, st>>>(cx, cy, cz, cx, n, keys0, shift, passes, ss.hist, flags);
+        sort_enqueue(keys0, vals0, keys1, perm, n, shift, ss, flags, st);
+        (shift ? gather_sorted_kernel<true> : gather_sorted_kernel<false>)<<<g, kThreads, 0, st>>>(
+            cx, cy, cz, cx, keys0, vals0, n, keys1, perm, spos, bs, flags);
+        topology_kernel<<<g, kThreads, 0, st>>>(keys1, n, nodes, bs.leaf_parent, bs.int_parent, flags);
+        triangles_kernel<<<g, kThreads, 0, st>>>(tris, perm, n, sc->tris, box);
+        boxes_enqueue(BoxLeaves{box}, n, nodes, {nullptr, nullptr}, bs, flags, st);
+        collapse_kernel<<<g, kThreads, 0, st>>>(reinterpret_cast<const float4 *>(nodes), n, sc->nodes, flags);
+        ctx->launches += 8 + passes;
+        e = cudaGetLastError();
+    }
+    cudaFreeAsync(scratch, st);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(&ctx->host_counters[2], flags, sizeof(unsigned long long), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return hrr_cuda_fail(ctx, e, "scene build");
+    const unsigned long long f = ctx->host_counters[2];
+    if (f & HRR_FLAG_NONFINITE) return hrr_fail(ctx, HRR_ERR_INVALID_ARG, "a triangle vertex is not finite");
+    if ((f & HRR_FLAG_RUNS) && shift) return scene_attempt(ctx, tris, n, sc, 0);
+    if (f & (HRR_FLAG_TOPOLOGY | HRR_FLAG_WAIT)) return hrr_fail(ctx, HRR_ERR_DEVICE, "scene links");
+    return HRR_OK;
+}
+
+// A scene of one triangle: no nodes, the triangle alone.
+int scene_of_one(hrr_ctx *ctx, const float *tris, hrr_scene *sc) {
+    cudaStream_t st = ctx->stream;
+    unsigned long long *flags = ctx->counters + 2;
+    float *cen = nullptr;
+    HRR_CUDA(ctx, hrr_alloc(ctx, &cen, 3 * sizeof(float)));
+    cudaError_t e = cudaMemsetAsync(flags, 0, sizeof(unsigned long long), st);
+    if (e == cudaSuccess) {
+        centroid_kernel<<<1, kThreads, 0, st>>>(tris, 1u, cen, cen + 1, cen + 2, flags);
+        triangles_kernel<<<1, kThreads, 0, st>>>(tris, nullptr, 1u, sc->tris, nullptr);
+        ctx->launches += 2;
+        e = cudaGetLastError();
+    }
+    cudaFreeAsync(cen, st);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(&ctx->host_counters[2], flags, sizeof(unsigned long long), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return hrr_cuda_fail(ctx, e, "scene build");
+    if (ctx->host_counters[2] & HRR_FLAG_NONFINITE)
+        return hrr_fail(ctx, HRR_ERR_INVALID_ARG, "a triangle vertex is not finite");
+    return HRR_OK;
 }
 
 }  // namespace
@@ -399,62 +585,20 @@ int hrr_build_scene(hrr_ctx *ctx, const float *dev_tris, uint32_t n_tris, hrr_sc
     if (!dev_tris || n_tris == 0 || n_tris > 0x7FFFFFFFu)
         return hrr_fail(ctx, HRR_ERR_INVALID_ARG, "need 1 .. 2^31 - 1 triangles");
     DeviceGuard g(ctx->device);
-    cudaStream_t st = ctx->stream;
-    unsigned long long *flags = ctx->counters + 2;
-    const size_t n = n_tris;
-    float *cen = nullptr;
-    HRR_CUDA(ctx, hrr_alloc(ctx, &cen, sizeof(float) * 4 * n));
-    const unsigned gr = (unsigned)((n + kThreads - 1) / kThreads);
-    HRR_CUDA(ctx, cudaMemsetAsync(flags, 0, sizeof(unsigned long long), st));
-    centroid_kernel<<<gr, kThreads, 0, st>>>(dev_tris, n_tris, cen, cen + n, cen + 2 * n, cen + 3 * n, flags);
-    ++ctx->launches;
-    HRR_CUDA(ctx, cudaMemcpyAsync(&ctx->host_counters[2], flags, sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
-    HRR_CUDA(ctx, cudaStreamSynchronize(st));
-    if (ctx->host_counters[2] & HRR_FLAG_NONFINITE) {
-        cudaFreeAsync(cen, st);
-        return hrr_fail(ctx, HRR_ERR_INVALID_ARG, "a triangle vertex is not finite");
-    }
-    hrr_tree *tree = nullptr;
-    const hrr_lights L{cen, cen + n, cen + 2 * n, cen + 3 * n};
-    int rc = hrr_build_impl(ctx, L, n_tris, &tree);  // the centroids' radix tree (synchronous)
-    cudaFreeAsync(cen, st);
-    if (rc != HRR_OK) return rc;
-    for (float4 **derived : {&tree->wide, &tree->pairs}) {  // the segment walk reads the binary records only
-        if (*derived) cudaFreeAsync(*derived, st);
-        *derived = nullptr;
-    }
     hrr_scene *sc = new (std::nothrow) hrr_scene();
-    if (!sc) {
-        hrr_free_light_tree(ctx, tree);
-        return hrr_fail(ctx, HRR_ERR_OOM, "host allocation of the scene");
-    }
+    if (!sc) return hrr_fail(ctx, HRR_ERR_OOM, "host allocation of the scene");
     sc->device = ctx->device;
     sc->n = n_tris;
-    sc->tree = tree;
-    uint32_t *links = nullptr;
-    cudaError_t e = hrr_alloc(ctx, &sc->tris, sizeof(float) * kTriFloats * n);
-    if (e == cudaSuccess) e = hrr_alloc(ctx, &links, sizeof(uint32_t) * 3 * n);
-    if (e == cudaSuccess) e = cudaMemsetAsync(links, 0xFF, sizeof(uint32_t) * 2 * n, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(links + 2 * n, 0, sizeof(uint32_t) * n, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(flags, 0, sizeof(unsigned long long), st);
-    if (e == cudaSuccess) {
-        if (n > 1) {
-            scene_links_kernel<<<(unsigned)((n - 1 + kThreads - 1) / kThreads), kThreads, 0, st>>>(
-                tree->nodes, n_tris, links, links + n, flags);
-            ++ctx->launches;
-        }
-        tri_refit_kernel<<<gr, kThreads, 0, st>>>(dev_tris, tree->perm, n_tris, tree->nodes, sc->tris, links,
-                                                  links + n, links + 2 * n, flags);
-        ++ctx->launches;
-        e = cudaGetLastError();
-    }
-    if (links) cudaFreeAsync(links, st);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(&ctx->host_counters[2], flags, sizeof(unsigned long long), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess || (ctx->host_counters[2] & HRR_FLAG_TOPOLOGY)) {
+    cudaError_t e = hrr_alloc(ctx, &sc->tris, sizeof(float) * kTriFloats * (size_t)n_tris);
+    if (e == cudaSuccess) e = hrr_alloc(ctx, &sc->nodes, sizeof(uint32_t) * kNodeWords * (size_t)std::max(n_tris - 1u, 1u));
+    const int rc = e != cudaSuccess ? hrr_cuda_fail(ctx, e, "scene allocation")
+                   : n_tris == 1    ? scene_of_one(ctx, dev_tris, sc)
+                                    : scene_attempt(ctx, dev_tris, n_tris, sc, kTopShift);
+    if (rc != HRR_OK) {
+        const std::string err = ctx->err;
         hrr_free_scene(ctx, sc);
-        return e != cudaSuccess ? hrr_cuda_fail(ctx, e, "scene build") : hrr_fail(ctx, HRR_ERR_DEVICE, "scene links");
+        ctx->err = err;
+        return rc;
     }
     *out = sc;
     return HRR_OK;
@@ -463,7 +607,7 @@ int hrr_build_scene(hrr_ctx *ctx, const float *dev_tris, uint32_t n_tris, hrr_sc
 int hrr_free_scene(hrr_ctx *ctx, hrr_scene *scene) {
     if (!ctx || !scene) return HRR_ERR_INVALID_ARG;
     DeviceGuard g(ctx->device);
-    if (scene->tree) hrr_free_light_tree(ctx, scene->tree);
+    if (scene->nodes) cudaFreeAsync(scene->nodes, ctx->stream);
     if (scene->tris) cudaFreeAsync(scene->tris, ctx->stream);
     delete scene;
     return HRR_OK;
@@ -494,7 +638,7 @@ int hrr_connect(hrr_ctx *ctx, hrr_eyes eyes, uint32_t n_eyes, hrr_lights lights,
         A.tau = tau;
         A.pairs = reinterpret_cast<const uint2 *>(dev_pairs);
         A.n_pairs = n_pairs;
-        A.nodes = scene ? reinterpret_cast<const float4 *>(scene->tree->nodes) : nullptr;
+        A.nodes = scene ? scene->nodes : nullptr;
         A.tris = scene ? scene->tris : nullptr;
         A.n_tris = scene ? scene->n : 0;
         A.weight = dev_weight;

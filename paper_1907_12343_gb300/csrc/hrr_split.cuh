@@ -33,6 +33,7 @@
 
 #include "hrr_boxes.cuh"
 #include "hrr_internal.cuh"
+#include "hrr_order.cuh"
 
 namespace {
 
@@ -208,39 +209,6 @@ __device__ __forceinline__ void run_best(const float4 (&p)[R], uint32_t cnt, uin
             }
         }
     }
-}
-
-// Common-prefix length of the ordering keys (Morton key, sorted position) of leaves i, j; -1
-// outside [f, l].
-__device__ __forceinline__ int prefix_len(const uint64_t *__restrict__ keys, int64_t f, int64_t l, int64_t i, int64_t j) {
-    if (j < f || j > l) return -1;
-    const uint64_t ki = keys[i], kj = keys[j];
-    if (ki != kj) return __clzll((long long)(ki ^ kj));
-    return 64 + __clz((uint32_t)(i ^ j));
-}
-
-// Range and split of node i of the binary radix tree over the leaves [f, l] (f <= i < l): each
-// node finds them from its neighbours' common-prefix lengths (Karras, HPG 2012).
-__device__ __forceinline__ void radix_node(const uint64_t *__restrict__ keys, uint32_t f32, uint32_t l32, uint32_t i32,
-                                           uint32_t &first, uint32_t &last, uint32_t &split) {
-    const int64_t f = f32, l = l32, i = i32;
-    const int d = (prefix_len(keys, f, l, i, i + 1) - prefix_len(keys, f, l, i, i - 1)) >= 0 ? 1 : -1;
-    const int dmin = prefix_len(keys, f, l, i, i - d);
-    int64_t most = 2;
-    while (prefix_len(keys, f, l, i, i + most * d) > dmin) most <<= 1;
-    int64_t len = 0;
-    for (int64_t t = most >> 1; t >= 1; t >>= 1)
-        if (prefix_len(keys, f, l, i, i + (len + t) * d) > dmin) len += t;
-    const int64_t j = i + len * d;
-    const int dnode = prefix_len(keys, f, l, i, j);
-    int64_t s = 0, t = len;
-    do {
-        t = (t + 1) >> 1;
-        if (prefix_len(keys, f, l, i, i + (s + t) * d) > dnode) s += t;
-    } while (t > 1);
-    split = (uint32_t)(i + s * d + (d < 0 ? -1 : 0));
-    first = (uint32_t)(i < j ? i : j);
-    last = (uint32_t)(i < j ? j : i);
 }
 
 // The best split in runs of R lights per lane of a warp (or thread of a block, SCAN giving the
