@@ -376,8 +376,10 @@ __device__ __forceinline__ uint32_t walk_pairs(const Frame &fr, const Eye &E, ui
         // the other child's minimum (of a leaf: its own value)
         const uint32_t vnew = range_min_leaves<VARIANT>(in0 ? split + 1u : first, in0 ? last : split, E);
         const uint32_t v0 = in0 ? e.y : vnew, v1 = in0 ? vnew : e.y;
+        hrr_f2 den, rhs;
+        hrr_bound2(nlox, nloy, nloz, nhix, nhiy, nhiz, imax, ex, ey, ez, E.scale, den, rhs);
         bool s0, s1;
-        hrr_survive2(nlox, nloy, nloz, nhix, nhiy, nhiz, imax, ex, ey, ez, E.scale, v0, v1, ok, s0, s1);
+        hrr_survive2(den, rhs, v0, v1, ok, s0, s1);
         const bool go0 = s0 && first != split, go1 = s1 && split + 1u != last;
         const unsigned b0 = __ballot_sync(0xFFFFFFFFu, go0), b1 = __ballot_sync(0xFFFFFFFFu, go1);
         const uint32_t n = __popc(b0) + __popc(b1);

@@ -219,19 +219,23 @@ __device__ __forceinline__ hrr_f2 hrr_gap2(hrr_f2 nlo, hrr_f2 nhi, hrr_f2 e) {
     hrr_unpack2(dn, d0, d1);
     return hrr_pack2(hrr_max3(0.0f, -u0, d0), hrr_max3(0.0f, -u1, d1));
 }
-// Whether each box survives (is not culled) at range minima v0, v1, where `ok`.
-__device__ __forceinline__ void hrr_survive2(hrr_f2 nlox, hrr_f2 nloy, hrr_f2 nloz, hrr_f2 nhix, hrr_f2 nhiy,
-                                             hrr_f2 nhiz, hrr_f2 imax, hrr_f2 ex, hrr_f2 ey, hrr_f2 ez, float scale,
-                                             uint32_t v0, uint32_t v1, bool ok, bool &s0, bool &s1) {
+// Both boxes' sides of the cull test (hrr_node_bound).
+__device__ __forceinline__ void hrr_bound2(hrr_f2 nlox, hrr_f2 nloy, hrr_f2 nloz, hrr_f2 nhix, hrr_f2 nhiy, hrr_f2 nhiz,
+                                           hrr_f2 imax, hrr_f2 ex, hrr_f2 ey, hrr_f2 ez, float scale, hrr_f2 &den,
+                                           hrr_f2 &rhs) {
     const hrr_f2 gx = hrr_gap2(nlox, nhix, ex), gy = hrr_gap2(nloy, nhiy, ey), gz = hrr_gap2(nloz, nhiz, ez);
-    hrr_f2 d2, rhs, lhs;
+    hrr_f2 d2;
     asm("mul.rm.f32x2 %0, %1, %1;" : "=l"(d2) : "l"(gx));
     asm("fma.rm.f32x2 %0, %1, %1, %0;" : "+l"(d2) : "l"(gy));
     asm("fma.rm.f32x2 %0, %1, %1, %0;" : "+l"(d2) : "l"(gz));
     float a, b;
     hrr_unpack2(d2, a, b);
-    const hrr_f2 den = hrr_pack2(fmaxf(a, 1e-4f), fmaxf(b, 1e-4f));
+    den = hrr_pack2(fmaxf(a, 1e-4f), fmaxf(b, 1e-4f));
     asm("mul.rp.f32x2 %0, %1, %2;" : "=l"(rhs) : "l"(imax), "l"(hrr_pack2(scale, scale)));
+}
+// Whether each box survives (is not culled) at range minima v0, v1, where `ok`.
+__device__ __forceinline__ void hrr_survive2(hrr_f2 den, hrr_f2 rhs, uint32_t v0, uint32_t v1, bool ok, bool &s0, bool &s1) {
+    hrr_f2 lhs;
     asm("mul.rm.f32x2 %0, %1, %2;"
         : "=l"(lhs)
         : "l"(hrr_pack2(__uint2float_rd(v0), __uint2float_rd(v1))), "l"(den));

@@ -35,7 +35,7 @@ constexpr int kMinBlocks = 5;    // resident blocks per SM the register budget i
 struct SampleLaunch {
     const float *ex, *ey, *ez;
     const uint16_t *px, *py;
-    const float4 *nodes;
+    const float4 *pairs_rec;      // the paired records (hrr_tree::pairs)
     const uint32_t *perm;
     const uint32_t *tile;         // d layers of w x h
     uint32_t tile_w, tile_h, tile_d;
@@ -53,15 +53,17 @@ struct SampleLaunch {
     uint2 *spill;
 };
 
-// One 64-byte record as two 256-bit read-only loads that do not allocate in L1 (scattered
+// One 64-byte paired record as two 256-bit read-only loads that do not allocate in L1 (scattered
 // records are rarely reused from L1; filling it would cost L1 data-pipe cycles).
-__device__ __forceinline__ void load_record(const float4 *p, float4 &q0, float4 &q1, float4 &q2, float4 &q3) {
-    asm("ld.global.nc.L1::no_allocate.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-        : "=f"(q0.x), "=f"(q0.y), "=f"(q0.z), "=f"(q0.w), "=f"(q1.x), "=f"(q1.y), "=f"(q1.z), "=f"(q1.w)
-        : "l"(p));
-    asm("ld.global.nc.L1::no_allocate.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8+32];"
-        : "=f"(q2.x), "=f"(q2.y), "=f"(q2.z), "=f"(q2.w), "=f"(q3.x), "=f"(q3.y), "=f"(q3.z), "=f"(q3.w)
-        : "l"(p));
+__device__ __forceinline__ void load_pairs(const float4 *p, hrr_f2 &a, hrr_f2 &b, hrr_f2 &c, hrr_f2 &d, hrr_f2 &e, hrr_f2 &f,
+                                           hrr_f2 &g, hrr_f2 &h) {
+    asm("ld.global.nc.L1::no_allocate.v4.b64 {%0,%1,%2,%3}, [%4];" : "=l"(a), "=l"(b), "=l"(c), "=l"(d) : "l"(p));
+    asm("ld.global.nc.L1::no_allocate.v4.b64 {%0,%1,%2,%3}, [%4+32];" : "=l"(e), "=l"(f), "=l"(g), "=l"(h) : "l"(p));
+}
+
+// The shift of sample s at tile pixel (tx, ty).
+__device__ __forceinline__ uint32_t shift_of(const SampleLaunch &P, uint32_t s, uint32_t ty, uint32_t tx) {
+    return P.tile[(size_t)(s % P.tile_d) * P.tile_w * P.tile_h + ty * P.tile_w + tx] + P.offset[s];
 }
 
 // Append the warp's cnt staged entries to their samples' outputs (warp-collective).
@@ -137,13 +139,14 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) cull_samples_kernel(cons
         const uint32_t j = (uint32_t)g;
         const float ex = P.ex[j], ey = P.ey[j], ez = P.ez[j];
         const uint32_t tx = P.px[j] % P.tile_w, ty = P.py[j] % P.tile_h;
+        const hrr_f2 ex2 = hrr_pack2(ex, ex), ey2 = hrr_pack2(ey, ey), ez2 = hrr_pack2(ez, ez);
         // lane s < n_samples: shift r of sample s and c = brev(2^32 - r)
         uint32_t rl = 0;
-        if ((uint32_t)lane < P.n_samples)
-            rl = P.tile[(size_t)((uint32_t)lane % P.tile_d) * P.tile_w * P.tile_h + ty * P.tile_w + tx] + P.offset[lane];
+        if ((uint32_t)lane < P.n_samples) rl = shift_of(P, (uint32_t)lane, ty, tx);
         const uint32_t cl = __brev(0u - rl);
         if (P.n_lights == 1) {  // the root is a leaf (record 0, slot 0)
-            const float4 q0 = __ldg(&P.nodes[0]);
+            const float *rec = reinterpret_cast<const float *>(P.pairs_rec);
+            const float4 q0 = make_float4(-rec[0], -rec[2], -rec[4], rec[12]);
             uint32_t acc = 0;
             for (uint32_t s = 0; s < P.n_samples; ++s) {
                 const uint32_t rs = __shfl_sync(0xFFFFFFFFu, rl, s);
@@ -156,7 +159,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) cull_samples_kernel(cons
         // Stack: logical entries [0, S); the newest R of them are in the ring at index & mask,
         // the others in the spill area at their logical index.
         uint32_t S = 1, R = 1, visits = 0;
-        if (lane == 0) ring[0] = make_uint2(0u, all);
+        if (lane == 0) ring[0] = make_uint2(0u, all);  // the root's slot
         __syncwarp();
         while (S > 0) {
             if (visits >= P.n_lights) {  // each internal node is visited at most once per eye
@@ -172,55 +175,55 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) cull_samples_kernel(cons
                 __syncwarp();
             }
             const bool active = (uint32_t)lane < m;
-            uint2 e = make_uint2(0u, 0u);
-            if (active) e = ring[(S - m + lane) & kRingMask];
+            const uint2 e = ring[(S - m + min((uint32_t)lane, m - 1u)) & kRingMask];
             S -= m;
             R -= m;
             visits += m;
             __syncwarp();
 
-            bool valid = false, int0 = false, int1 = false;
-            uint32_t split = 0, first = 0, last = 0;
-            float4 q0 = make_float4(0.f, 0.f, 0.f, 0.f), q2 = q0;
-            float den0 = 0.f, rhs0 = 0.f, den1 = 0.f, rhs1 = 0.f;
-            if (active) {
-                sample_visits += __popc(e.y);
-                float4 q1, q3;
-                load_record(&P.nodes[4 * (size_t)e.x], q0, q1, q2, q3);
-                split = __float_as_uint(q1.w);
-                const uint32_t other = __float_as_uint(q3.w);
-                first = min(e.x, other);
-                last = max(e.x, other);
-                if (last >= P.n_lights || split - first >= last - first) {  // needs first <= split < last
-                    atomicOr(P.flags, HRR_FLAG_TOPOLOGY);                     // corrupt record
-                } else {
-                    valid = true;
-                    int0 = first != split;
-                    int1 = split + 1u != last;
-                    hrr_node_bound(scale, q0.x, q0.y, q0.z, q1.x, q1.y, q1.z, q0.w, ex, ey, ez, den0, rhs0);
-                    hrr_node_bound(scale, q2.x, q2.y, q2.z, q3.x, q3.y, q3.z, q2.w, ex, ey, ez, den1, rhs1);
-                }
-            }
-            // per sample: the children's range minima and cull tests, or the leaf tests
+            // The record (idle lanes take the last lane's, whose line the load touches anyway), both
+            // children's box bounds, and per sample both range minima and cull tests. A leaf's
+            // minimum is its own value and its box the light; few leaves survive, and only those
+            // take the exact test.
+            if (active) sample_visits += __popc(e.y);
+            hrr_f2 nlox, nloy, nloz, nhix, nhiy, nhiz, imax, links;
+            load_pairs(&P.pairs_rec[4 * (size_t)e.x], nlox, nloy, nloz, nhix, nhiy, nhiz, imax, links);
+            const uint32_t node = hrr_slot_node(e.x);
+            const uint32_t split = (uint32_t)links, other = (uint32_t)(links >> 32);
+            const uint32_t first = min(node, other), last = max(node, other);
+            const bool ok = active && last < P.n_lights && split - first < last - first;  // first <= split < last < n
+            if (active && !ok) atomicOr(P.flags, HRR_FLAG_TOPOLOGY);                      // corrupt record
+            const uint32_t live = ok ? e.y : 0u;
+            const bool int0 = first != split, int1 = split + 1u != last;
+            hrr_f2 den, rhs;
+            hrr_bound2(nlox, nloy, nloz, nhix, nhiy, nhiz, imax, ex2, ey2, ez2, scale, den, rhs);
             uint32_t mask0 = 0, mask1 = 0, acc0 = 0, acc1 = 0;
             for (uint32_t s = 0; s < P.n_samples; ++s) {
                 const uint32_t rs = __shfl_sync(0xFFFFFFFFu, rl, s), cs = __shfl_sync(0xFFFFFFFFu, cl, s);
-                if (valid && ((e.y >> s) & 1u)) {
-                    const uint32_t bit = 1u << s;
-                    // a leaf's minimum is its own value, its box the light: few leaves
-                    // survive the node test, and only those take the exact one
-                    const uint32_t v0 = hrr_range_min_value(first, split + 1u - first, rs, 0u - rs, cs);
-                    if (!hrr_node_culls(v0, den0, rhs0)) {
-                        if (int0) mask0 |= bit;
-                        else if (hrr_pair_accepts(v0, tau, q0.x, q0.y, q0.z, q0.w, ex, ey, ez)) acc0 |= bit;
+                const uint32_t v0 = hrr_range_min_leaves(first, split, rs, 0u - rs, cs);
+                const uint32_t v1 = hrr_range_min_leaves(split + 1u, last, rs, 0u - rs, cs);
+                bool s0, s1;
+                hrr_survive2(den, rhs, v0, v1, ((live >> s) & 1u) != 0u, s0, s1);
+                const uint32_t bit = 1u << s;
+                if (s0) mask0 |= bit;
+                if (s1) mask1 |= bit;
+            }
+            if ((!int0 && mask0) || (!int1 && mask1)) {
+                const float *rec = reinterpret_cast<const float *>(P.pairs_rec + 4 * (size_t)e.x);
+                for (uint32_t c = 0; c < 2; ++c) {
+                    uint32_t m2 = c == 0 ? (int0 ? 0u : mask0) : (int1 ? 0u : mask1), acc = 0;
+                    const uint32_t i = c == 0 ? split : last;
+                    for (; m2; m2 &= m2 - 1u) {
+                        const uint32_t s = (uint32_t)__ffs((int)m2) - 1u;
+                        const uint32_t xi = __brev(i) + shift_of(P, s, ty, tx);
+                        if (hrr_pair_accepts(xi, tau, -rec[c], -rec[2 + c], -rec[4 + c], rec[12 + c], ex, ey, ez)) acc |= 1u << s;
                     }
-                    const uint32_t v1 = hrr_range_min_value(split + 1u, last - split, rs, 0u - rs, cs);
-                    if (!hrr_node_culls(v1, den1, rhs1)) {
-                        if (int1) mask1 |= bit;
-                        else if (hrr_pair_accepts(v1, tau, q2.x, q2.y, q2.z, q2.w, ex, ey, ez)) acc1 |= bit;
-                    }
+                    if (c == 0) acc0 = acc;
+                    else acc1 = acc;
                 }
             }
+            if (!int0) mask0 = 0;
+            if (!int1) mask1 = 0;
             // Push the children that are alive for some sample as one compacted run.
             const bool go0 = mask0 != 0u, go1 = mask1 != 0u;
             const unsigned b0 = __ballot_sync(0xFFFFFFFFu, go0), b1 = __ballot_sync(0xFFFFFFFFu, go1);
@@ -240,8 +243,8 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) cull_samples_kernel(cons
                 // lane by lane, siblings side by side (popped together by neighbouring lanes,
                 // whose records are neighbours in memory)
                 const uint32_t at = S + __popc(b0 & lt) + __popc(b1 & lt);
-                if (go0) ring[at & kRingMask] = make_uint2(split, mask0);
-                if (go1) ring[(at + (go0 ? 1u : 0u)) & kRingMask] = make_uint2(split + 1u, mask1);
+                if (go0) ring[at & kRingMask] = make_uint2(2u * split, mask0);
+                if (go1) ring[(at + (go0 ? 1u : 0u)) & kRingMask] = make_uint2(2u * split + 1u, mask1);
                 S += n;
                 R += n;
                 __syncwarp();
@@ -302,7 +305,7 @@ int hrr_cull_samples_impl(hrr_ctx *ctx, const hrr_eyes &E, uint32_t n_eyes, cons
         }
         SampleLaunch P{};
         P.ex = E.x; P.ey = E.y; P.ez = E.z; P.px = E.px; P.py = E.py;
-        P.nodes = reinterpret_cast<const float4 *>(tree->nodes);
+        P.pairs_rec = tree->pairs;
         P.perm = tree->perm;
         P.tile = ctx->tile;
         P.tile_w = ctx->tile_w; P.tile_h = ctx->tile_h; P.tile_d = ctx->tile_d ? ctx->tile_d : 1u;
