@@ -24,8 +24,8 @@
 //     and the rest are subtrees of a warp each.
 //   * up to 32 lights: one warp builds the whole subtree, a light per lane.
 // With one level of every size per pass, four kernels and a host round trip each, the build of
-// 2^20 lights took 1843 us, now 1064 us. What is left is instructions (the subtrees of 33 to 1024
-// lights: 176 million warp instructions, 41% of the issue slots at 28 warps per SM, 345 us) and the
+// 2^20 lights took 1843 us, now 1043 us. What is left is instructions (the subtrees of 33 to 1024
+// lights and below: 212 and 132 us) and the
 // latency of about twenty levels (8 to 20 us each).
 #pragma once
 
@@ -358,7 +358,7 @@ __device__ __forceinline__ void subtree_warp(const Seg &g0, const float4 *lights
     }
 }
 
-__global__ void __launch_bounds__(kSplitThreads) subtree_kernel(const float4 *__restrict__ spos,
+__global__ void __launch_bounds__(kSplitThreads, 5) subtree_kernel(const float4 *__restrict__ spos,
                                                                 const uint64_t *__restrict__ keys, SplitOut o) {
     const uint32_t count = o.counts[0];
     for (uint32_t w = (blockIdx.x * kSplitThreads + threadIdx.x) >> 5; w < count; w += gridDim.x * (kSplitThreads / 32)) {
@@ -367,13 +367,14 @@ __global__ void __launch_bounds__(kSplitThreads) subtree_kernel(const float4 *__
     }
 }
 
-// Ranges of 33 to kSubMax lights: a block each, the lights in shared memory.
+// Ranges of 33 to kSubMax lights: a block each, the lights in shared memory. What it leaves of up
+// to 32 lights goes to subtree_kernel's list.
 __global__ void __launch_bounds__(kSubThreads, 7) sub_kernel(const float4 *__restrict__ spos,
-                                                          const uint64_t *__restrict__ keys, SplitOut o) {
+                                                          SplitOut o) {
     constexpr uint32_t kWarps = kSubThreads / 32;
     __shared__ float4 pos[kSubMax];
     __shared__ Seg wide[2][4], mid[2][kSubMax / (kSmallMax + 1) + 1], small[kSubMax / 2];
-    __shared__ uint32_t n_wide[2], n_mid[2], n_small;
+    __shared__ uint32_t n_wide[2], n_mid[2], n_small, small_at;
     __shared__ Agg sh[kWarps];
     __shared__ Best shb[kWarps];
     const uint32_t t = threadIdx.x, warp = t >> 5, lane = t & 31u;
@@ -432,11 +433,9 @@ __global__ void __launch_bounds__(kSubThreads, 7) sub_kernel(const float4 *__res
             q ^= 1u;
             __syncthreads();
         }
-        const uint32_t ns = n_small;
-        for (uint32_t k = warp; k < ns; k += kWarps) {
-            const Seg g = small[k];
-            subtree_warp(g, pos + (g.f - root.f), keys, o);
-        }
+        if (t == 0 && n_small) small_at = atomicAdd(&o.counts[0], n_small);
+        __syncthreads();
+        for (uint32_t k = t; k < n_small; k += kSubThreads) o.small[small_at + k] = small[k];
         __syncthreads();  // before the lists and lights are refilled
     }
 }
@@ -597,8 +596,8 @@ int cost_topology(hrr_ctx *ctx, const float4 *spos, const uint64_t *keys, uint32
     }
     if (e == cudaSuccess && rc == HRR_OK) {
         const unsigned sub_grid = (unsigned)std::min<size_t>(un / 33 + 1, (size_t)ctx->sm_count * 16);
-        const unsigned small_grid = (unsigned)std::min<size_t>(un / 16 + 1, (size_t)ctx->sm_count * 8);
-        sub_kernel<<<sub_grid, kSubThreads, 0, st>>>(spos, keys, o);
+        const unsigned small_grid = (unsigned)std::min<size_t>(un / 16 + 1, (size_t)ctx->sm_count * 5);
+        sub_kernel<<<sub_grid, kSubThreads, 0, st>>>(spos, o);
         subtree_kernel<<<small_grid, kSplitThreads, 0, st>>>(spos, keys, o);
         radix_subtrees_kernel<<<(unsigned)ctx->sm_count * 4u, kSplitThreads, 0, st>>>(keys, o);
         ctx->launches += 3;
