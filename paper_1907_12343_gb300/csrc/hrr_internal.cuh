@@ -128,7 +128,7 @@ inline const float4 *hrr_tree_top(const hrr_tree *tree) {
 }
 
 // Kernels a refit launches (hrr_refit_enqueue).
-inline int hrr_refit_launches(const hrr_tree *tree) { return tree->n > 1 ? 4 : 1; }
+inline int hrr_refit_launches(const hrr_tree *tree) { return tree->n > 1 ? 3 : 1; }
 
 // Layer (sample mod d) of a w x h x d tile: the shifts one culling pass uses.
 inline const uint32_t *hrr_tile_layer(const uint32_t *tile, uint32_t w, uint32_t h, uint32_t d,
