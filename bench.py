@@ -280,12 +280,12 @@ def run_ours(args):
 
 
 # Algorithmic work of one node visit on the frame workload with the cost-driven hierarchy
-# (counted with the oracle's traversal over 3,000 evenly spaced eyes): 1.960 internal child
-# tests x 19 ops (the box gap, 9; its square, 3 with fused multiply-adds; the distance floor
-# and the scaled bound, 2; the value of the range minimum, 2; the division-free cull
-# comparison, 3) + 0.973 new range minima x 51 integer ops + 0.988 inherited minima x 2 +
-# 0.040 leaf tests x 17.
-OPS_PER_VISIT = 1.960 * 19 + 0.973 * 51 + 0.988 * 2 + 0.040 * 17
+# (counted with the oracle's traversal over 3,000 evenly spaced eyes): 2.000 child tests x 17
+# ops (the box gap, 9; its square, 3 with fused multiply-adds; the distance floor and the
+# scaled bound, 2; the division-free cull comparison, 3; leaf children take the same test) +
+# 0.973 new range minima x 27 integer ops + the index of the inherited minimum and its side, 3,
+# + 0.009 exact leaf tests x 17.
+OPS_PER_VISIT = 2.000 * 17 + 0.973 * 27 + 3 + 0.009 * 17
 PROFILE_SUMMARY = os.path.join(ROOT, "profiles", "cull_single_kernel_frame_1920x1080.md")
 PROFILE_SMALL = os.path.join(ROOT, "profiles", "cull_single_kernel_frame_480x270.md")
 TOPOLOGY = "cost"  # hierarchy shape of the benchmarked builds (set from --topology)
@@ -316,7 +316,9 @@ def kernel_source_hash(files=None) -> str:
 
 def build_source_hash() -> str:
     """The hierarchy build's source: the cull's traffic depends on the tree it walks."""
-    return kernel_source_hash([os.path.join(ROOT, "paper_1907_12343_gb300", "csrc", "hrr_build.cu")])
+    return kernel_source_hash([os.path.join(ROOT, "paper_1907_12343_gb300", "csrc", f)
+                               for f in ("hrr_build.cu", "hrr_boxes.cuh", "hrr_order.cuh", "hrr_sort.cuh",
+                                         "hrr_split.cuh")])
 
 
 def _profile_keys(path, topology=None):
@@ -382,8 +384,9 @@ def aggregate_throughput(units_per_rank: float, t_rank: float, dist=None, device
 
 
 def roofline(V, accepted, n_e, cull_ms, peaks, kind, clk, workload="", n_l=0, measured=None, tile_bytes=0):
-    """Roofline of the traversal kernel, which is bound by instruction issue: the node
-    records (64 B per visit) stay in L2 and DRAM traffic is essentially the output.
+    """Roofline of the traversal kernel: the node records (64 B per visit) stay in L2 and DRAM
+    traffic is essentially the output, so the ceiling of the algorithm is integer and FP32
+    work (the kernel itself runs into the L1 data pipe first, see the profile summaries).
     achieved = algorithmic ops per launch (node visits x OPS_PER_VISIT) / kernel time;
     peak = SMs x 4 schedulers x 32 lanes x maximum SM clock (one lane-op per lane per
     clock at full issue)."""
@@ -413,7 +416,8 @@ def roofline(V, accepted, n_e, cull_ms, peaks, kind, clk, workload="", n_l=0, me
 def other_fractions(V, accepted, n_e, n_l, sec, peaks, measured, tile_bytes):
     """The traversal's other rooflines, against denominators measured on this GPU:
     - l2: node-record bytes (64 B per visit) against an L2 streaming read, and visits
-      against scattered 64-byte record fetches (two 256-bit loads each, the same form);
+      against scattered 64-byte record fetches (two 256-bit loads each); the traversal's
+      siblings share a 128-byte line, so it can pass that scattered rate;
     - hbm: the bytes that must cross HBM once (records 64 (N_l - 1), eyes 16 N_e, the tile,
       pairs 8 |A|) against the measured copy bandwidth;
     - int32: the algorithmic ops per visit against independent 32-bit op chains."""

@@ -21,15 +21,16 @@
 // child tested, for one extra range minimum per visit.
 //
 // Execution: a persistent grid (a whole number of resident blocks per SM) in which each
-// warp traverses one eye at a time. The warp's stack of pending nodes is a ring in shared
-// memory; every step pops up to 32 nodes, one per lane, and the lanes push the children
-// that survive their tests back as one compacted run (ballot + popc). All lanes of a step
-// execute the same test on the same eye, leaf children included, so the warp stays
-// converged. A leaf child that survives (about one in a hundred visits, nearly all of them
-// accepted) is queued in shared memory, and the exact pair test runs on 32 queued leaves at
-// a time, and on the rest when the eye is done. Testing leaves in the step itself took a
-// divergent branch with one or two lanes in two of three steps. When the ring would overflow, its oldest entries move to a per-warp area in
-// global memory, and they come back when the ring runs low. The stack never exceeds
+// warp traverses one eye at a time. The newest of the warp's pending nodes are kept in shared
+// memory (binary records: a linear stack; width four: a ring); every step pops up to 32 nodes,
+// one per lane, and the lanes push the children that survive their tests back as one compacted
+// run (ballot + popc). All lanes of a step execute the same test on the same eye, leaf children
+// included, so the warp stays converged. A leaf child that survives (about one in a hundred
+// visits, nearly all of them accepted) is queued in shared memory, and the exact pair test runs
+// on 32 queued leaves at a time, and on the rest when the eye is done. Testing leaves in the step
+// itself took a divergent branch with one or two lanes in two of three steps. When the shared
+// entries would overflow, the oldest move to a per-warp area in global memory, and they come
+// back when few are left. The stack never exceeds
 // (w - 1) * 32 * L + 32 entries for node width w and L depth levels of pushed nodes (each
 // remainder of a pushed run below the top holds at most (w - 1) * 32 entries, and the
 // shallowest depth of those runs grows from the bottom of the stack to its top), and the
@@ -513,92 +514,90 @@ __device__ __forceinline__ void traverse(const Launch &Lc, const Frame *F) {
         if constexpr (W == 2) {
             visits += walk_pairs<VARIANT, kRing>(fr, E, j, lane, ring, queue, S, visits, HRR_WARP_SPILL, Lc.spill_cap,
                                                  Lc.flags);
-            S = 0;
-        }
-        while (W != 2 && S > 0) {
-            if (visits >= n_lights) {  // each internal node is visited at most once per eye
-                if (lane == 0) atomicOr(Lc.flags, HRR_FLAG_TOPOLOGY);
-                break;
-            }
-            const uint32_t m = min(32u, S);
-            if (R < m) {  // bring spilled entries back into the ring
-                const uint32_t fc = min(S - R, kRing / 2 - R);
-                const uint32_t base = S - R - fc;
-                const uint2 *spill = HRR_WARP_SPILL;
-                for (uint32_t k = lane; k < fc; k += 32) ring[(base + k) & kRingMask] = spill[base + k];
-                R += fc;
-                __syncwarp();
-            }
-            const bool active = (uint32_t)lane < m;
-            uint2 e = make_uint2(0u, 0u);
-            if (active) e = ring[(S - m + lane) & kRingMask];
-            S -= m;
-            R -= m;
-            visits += m;
-            __syncwarp();
-
-            Visit<W> V;
-#pragma unroll
-            for (int t = 0; t < W; ++t) {
-                V.go[t] = V.leaf[t] = false;
-                V.node[t] = V.vmin[t] = V.light[t] = 0;
-            }
-            if constexpr (W == 4) {
-                if (active) visit<VARIANT>(nodes, n_lights, e.x, e.y, E, Lc.flags, V);
-            }
-            // Push the surviving children as one compacted run.
-            unsigned bal[W];
-            uint32_t n = 0;
-#pragma unroll
-            for (int t = 0; t < W; ++t) {
-                bal[t] = __ballot_sync(0xFFFFFFFFu, V.go[t]);
-                n += __popc(bal[t]);
-            }
-            if (n) {
-                if (R + n > kRing) {  // move the oldest resident entries to the spill area
-                    const uint32_t s = (R + n - kRing + 31u) & ~31u;
-                    const uint32_t base = S - R;
-                    if (base + s > Lc.spill_cap) {  // cannot happen: the area holds the bound
-                        if (lane == 0) atomicOr(Lc.flags, HRR_FLAG_STACK);
-                        break;
-                    }
-                    uint2 *spill = HRR_WARP_SPILL;
-                    for (uint32_t k = lane; k < s; k += 32) spill[base + k] = ring[(base + k) & kRingMask];
-                    R -= s;
+        } else {
+            while (S > 0) {
+                if (visits >= n_lights) {  // each internal node is visited at most once per eye
+                    if (lane == 0) atomicOr(Lc.flags, HRR_FLAG_TOPOLOGY);
+                    break;
+                }
+                const uint32_t m = min(32u, S);
+                if (R < m) {  // bring spilled entries back into the ring
+                    const uint32_t fc = min(S - R, kRing / 2 - R);
+                    const uint32_t base = S - R - fc;
+                    const uint2 *spill = HRR_WARP_SPILL;
+                    for (uint32_t k = lane; k < fc; k += 32) ring[(base + k) & kRingMask] = spill[base + k];
+                    R += fc;
                     __syncwarp();
                 }
-                // Lane by lane, each lane's survivors side by side: siblings (whose records
-                // are neighbours in memory) are popped together by neighbouring lanes.
-                uint32_t pos = S;
-#pragma unroll
-                for (int t = 0; t < W; ++t) pos += __popc(bal[t] & lt);
-#pragma unroll
-                for (int t = 0; t < W; ++t) {
-                    if (V.go[t]) ring[pos & kRingMask] = make_uint2(V.node[t], V.vmin[t]);
-                    pos += V.go[t] ? 1u : 0u;
-                }
-                S += n;
-                R += n;
+                const bool active = (uint32_t)lane < m;
+                uint2 e = make_uint2(0u, 0u);
+                if (active) e = ring[(S - m + lane) & kRingMask];
+                S -= m;
+                R -= m;
+                visits += m;
                 __syncwarp();
-            }
-            bool any_leaf = false;
-#pragma unroll
-            for (int t = 0; t < W; ++t) any_leaf |= V.leaf[t];
-            if (__any_sync(0xFFFFFFFFu, any_leaf)) {
-#pragma unroll
+
+                Visit<W> V;
+    #pragma unroll
                 for (int t = 0; t < W; ++t) {
-                    const unsigned b = __ballot_sync(0xFFFFFFFFu, V.leaf[t]);
-                    if (V.leaf[t]) queue[queued_n + __popc(b & lt)] = queued<W>(e.x, (uint32_t)t, V.light[t]);
-                    queued_n += __popc(b);
+                    V.go[t] = V.leaf[t] = false;
+                    V.node[t] = V.vmin[t] = V.light[t] = 0;
                 }
-                __syncwarp();
-                while (queued_n >= 32u) {
-                    queued_n -= 32u;
-                    take_queued<W>(fr, E, j, lane, queue + queued_n, 32u);
+                if (active) visit<VARIANT>(nodes, n_lights, e.x, e.y, E, Lc.flags, V);
+                // Push the surviving children as one compacted run.
+                unsigned bal[W];
+                uint32_t n = 0;
+    #pragma unroll
+                for (int t = 0; t < W; ++t) {
+                    bal[t] = __ballot_sync(0xFFFFFFFFu, V.go[t]);
+                    n += __popc(bal[t]);
+                }
+                if (n) {
+                    if (R + n > kRing) {  // move the oldest resident entries to the spill area
+                        const uint32_t s = (R + n - kRing + 31u) & ~31u;
+                        const uint32_t base = S - R;
+                        if (base + s > Lc.spill_cap) {  // cannot happen: the area holds the bound
+                            if (lane == 0) atomicOr(Lc.flags, HRR_FLAG_STACK);
+                            break;
+                        }
+                        uint2 *spill = HRR_WARP_SPILL;
+                        for (uint32_t k = lane; k < s; k += 32) spill[base + k] = ring[(base + k) & kRingMask];
+                        R -= s;
+                        __syncwarp();
+                    }
+                    // Lane by lane, each lane's survivors side by side: siblings (whose records
+                    // are neighbours in memory) are popped together by neighbouring lanes.
+                    uint32_t pos = S;
+    #pragma unroll
+                    for (int t = 0; t < W; ++t) pos += __popc(bal[t] & lt);
+    #pragma unroll
+                    for (int t = 0; t < W; ++t) {
+                        if (V.go[t]) ring[pos & kRingMask] = make_uint2(V.node[t], V.vmin[t]);
+                        pos += V.go[t] ? 1u : 0u;
+                    }
+                    S += n;
+                    R += n;
+                    __syncwarp();
+                }
+                bool any_leaf = false;
+    #pragma unroll
+                for (int t = 0; t < W; ++t) any_leaf |= V.leaf[t];
+                if (__any_sync(0xFFFFFFFFu, any_leaf)) {
+    #pragma unroll
+                    for (int t = 0; t < W; ++t) {
+                        const unsigned b = __ballot_sync(0xFFFFFFFFu, V.leaf[t]);
+                        if (V.leaf[t]) queue[queued_n + __popc(b & lt)] = queued<W>(e.x, (uint32_t)t, V.light[t]);
+                        queued_n += __popc(b);
+                    }
+                    __syncwarp();
+                    while (queued_n >= 32u) {
+                        queued_n -= 32u;
+                        take_queued<W>(fr, E, j, lane, queue + queued_n, 32u);
+                    }
                 }
             }
+            if (queued_n) take_queued<W>(fr, E, j, lane, queue, queued_n);
         }
-        if (queued_n) take_queued<W>(fr, E, j, lane, queue, queued_n);
         if (lane == 0) {
             uint32_t *ev = frame_at<BATCH>(F, f).eye_visits;
             if (ev) ev[j] = visits;
