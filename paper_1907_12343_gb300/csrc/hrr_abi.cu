@@ -114,7 +114,9 @@ int hrr_create(hrr_ctx **out, int device, void *cuda_stream) {
             if (cudaStreamCreateWithFlags(&ctx->stream, cudaStreamNonBlocking) != cudaSuccess) { st = HRR_ERR_CUDA; break; }
             ctx->own_stream = true;
         }
-        if (cudaMalloc(&ctx->counters, 8 * sizeof(unsigned long long)) != cudaSuccess) { st = HRR_ERR_OOM; break; }
+        if (cudaMalloc(&ctx->counters, 16 * sizeof(unsigned long long)) != cudaSuccess) { st = HRR_ERR_OOM; break; }
+        ctx->cull_counters = ctx->counters + 8;
+        if (cudaMemsetAsync(ctx->cull_counters, 0, 8 * sizeof(unsigned long long), ctx->stream) != cudaSuccess) { st = HRR_ERR_CUDA; break; }
         if (cudaMallocHost(&ctx->host_counters, 8 * sizeof(unsigned long long)) != cudaSuccess) { st = HRR_ERR_OOM; break; }
         if (cudaDeviceGetAttribute(&ctx->sm_count, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) { st = HRR_ERR_CUDA; break; }
     } while (0);

@@ -292,7 +292,7 @@ struct ConnectArgs {
     float *weight;        // per pair, or NULL
     uint8_t *visible;     // per pair, or NULL
     float *eye_sum;       // per eye
-    unsigned long long *flags;
+    unsigned long long *flags;   // without a scene: a host word, written only by a bad pair
     unsigned long long *cursor;  // next pair to trace (starts at 0)
 };
 
@@ -342,7 +342,7 @@ __global__ void __launch_bounds__(kThreads) weights_kernel(const ConnectArgs A, 
 #pragma unroll
         for (int t = 0; t < kWeightItems; ++t) {
             if (ok[t] && (pr[t].x >= A.n_eyes || pr[t].y >= A.n_lights)) {
-                atomicOr(A.flags, HRR_FLAG_RANGE);
+                __stcs(A.flags, (unsigned long long)HRR_FLAG_RANGE);
                 ok[t] = false;
             }
             if (!ok[t]) continue;
@@ -626,8 +626,9 @@ int hrr_connect(hrr_ctx *ctx, hrr_eyes eyes, uint32_t n_eyes, hrr_lights lights,
     if (scene && scene->device != ctx->device) return hrr_fail(ctx, HRR_ERR_INVALID_ARG, "scene lives on another device");
     DeviceGuard g(ctx->device);
     cudaStream_t st = ctx->stream;
-    unsigned long long *flags = ctx->counters + 2;
-    HRR_CUDA(ctx, cudaMemsetAsync(flags, 0, 2 * sizeof(unsigned long long), st));  // flags, pair cursor
+    unsigned long long *flags = scene ? ctx->counters + 2 : &ctx->host_counters[2];
+    ctx->host_counters[2] = 0;
+    if (scene) HRR_CUDA(ctx, cudaMemsetAsync(flags, 0, 2 * sizeof(unsigned long long), st));  // flags, pair cursor
     if (n_eyes) HRR_CUDA(ctx, cudaMemsetAsync(dev_eye_sum, 0, sizeof(float) * (size_t)n_eyes, st));
     if (n_pairs) {
         ConnectArgs A{};
@@ -677,7 +678,8 @@ int hrr_connect(hrr_ctx *ctx, hrr_eyes eyes, uint32_t n_eyes, hrr_lights lights,
         if (packed) cudaFreeAsync(packed, st);
         HRR_CUDA(ctx, cudaGetLastError());
     }
-    HRR_CUDA(ctx, cudaMemcpyAsync(&ctx->host_counters[2], flags, sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
+    if (scene)
+        HRR_CUDA(ctx, cudaMemcpyAsync(&ctx->host_counters[2], flags, sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
     HRR_CUDA(ctx, cudaStreamSynchronize(st));
     if (ctx->host_counters[2] & HRR_FLAG_RANGE) return hrr_fail(ctx, HRR_ERR_INVALID_ARG, "a pair's eye or light index is out of range");
     if (ctx->host_counters[2] & (HRR_FLAG_STACK | HRR_FLAG_TOPOLOGY))

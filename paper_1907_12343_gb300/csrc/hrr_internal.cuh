@@ -45,10 +45,12 @@ struct hrr_ctx {
     hrr_tile_buf *tile_buf = nullptr;
     uint32_t *tile = nullptr;
     uint32_t tile_w = 0, tile_h = 0, tile_d = 1;  // d layers of w x h (a space-time tile)
-    // device counters of the last cull: [0] accepted pairs, [1] node visits, [2] flags,
-    // [3] work cursor
+    // device counters of a call: [0] accepted pairs, [1] node visits, [2] flags, [3] work cursor
     unsigned long long *counters = nullptr;
-    unsigned long long *host_counters = nullptr;  // pinned mirror
+    // the same and [4] blocks done, of hrr_cull: clear between calls (the kernel's last block
+    // reports them to host_counters and clears them)
+    unsigned long long *cull_counters = nullptr;
+    unsigned long long *host_counters = nullptr;  // pinned
     uint64_t last_visits = 0, last_accepted = 0;
     uint64_t launches = 0;
     // optional traversal-kernel timing
