@@ -183,6 +183,7 @@ __device__ __forceinline__ void box_groups_of_32(const BoxScratch &s, const Box 
 // All groups on their own, for what needs ranges' boxes before the topology is there.
 template <typename LEAVES>
 __global__ void __launch_bounds__(kBoxBlock) groups_kernel(LEAVES leaf, uint32_t n, BoxScratch s) {
+    chain_begin();
     const uint32_t base = blockIdx.x * kBoxBlock, g = base + threadIdx.x;
     box_groups_of_32(s, g < n ? leaf(g) : box_empty(), g, n);
     __syncthreads();
@@ -190,8 +191,7 @@ __global__ void __launch_bounds__(kBoxBlock) groups_kernel(LEAVES leaf, uint32_t
 }
 template <typename LEAVES>
 cudaError_t groups_enqueue(const LEAVES &leaf, uint32_t n, const BoxScratch &s, cudaStream_t st) {
-    groups_kernel<<<(n + kBoxBlock - 1) / kBoxBlock, kBoxBlock, 0, st>>>(leaf, n, s);
-    return cudaGetLastError();
+    return launch_chained(groups_kernel<LEAVES>, (n + kBoxBlock - 1) / kBoxBlock, kBoxBlock, st, leaf, n, s);
 }
 
 // The union of leaves [a, b] (a <= b), by a whole warp.
@@ -269,6 +269,7 @@ __global__ void __launch_bounds__(kBoxBlock, 3) box_kernel(LEAVES leaf, uint32_t
     __shared__ float4 sa[2][kBoxBlock], sb[2][kBoxBlock];  // child: (low, imax), (high, height)
     __shared__ uint32_t arrived[kBoxBlock], up[kBoxBlock], cut[kBoxBlock];
     __shared__ bool inside[kBoxBlock];
+    chain_begin();
     if (*(volatile unsigned long long *)flags & (HRR_FLAG_NONFINITE | HRR_FLAG_RUNS)) return;  // set before the launch
     const uint32_t t = threadIdx.x, base = blockIdx.x * kBoxBlock, g = base + t;
     uint32_t split = 0, other = 0, first = 0, last = 0;
@@ -365,6 +366,7 @@ template <bool DERIVED, typename LEAVES>
 __global__ void __launch_bounds__(kSpanThreads) span_kernel(LEAVES leaf, uint32_t n, hrr_node *nodes, Derived der,
                                                             BoxScratch s, uint32_t box_blocks,
                                                             unsigned long long *flags) {
+    chain_begin();
     if (*(volatile unsigned long long *)flags & (HRR_FLAG_NONFINITE | HRR_FLAG_RUNS)) return;
     const uint32_t count = *s.span_count;
     if (blockIdx.x >= box_blocks) {
@@ -450,11 +452,11 @@ cudaError_t boxes_enqueue(const LEAVES &leaf, uint32_t n, hrr_node *nodes, const
     const unsigned blocks = (n + kBoxBlock - 1) / kBoxBlock;
     const unsigned bb = std::min(608u, 8u + blocks), hb = std::min(152u, 1u + blocks / 16u);
     if (der.wide) {
-        box_kernel<true><<<blocks, kBoxBlock, 0, st>>>(leaf, n, nodes, der, s, have_groups, flags);
-        span_kernel<true><<<bb + hb, kSpanThreads, 0, st>>>(leaf, n, nodes, der, s, bb, flags);
+        launch_chained(box_kernel<true, LEAVES>, blocks, kBoxBlock, st, leaf, n, nodes, der, s, have_groups, flags);
+        launch_chained(span_kernel<true, LEAVES>, bb + hb, kSpanThreads, st, leaf, n, nodes, der, s, bb, flags);
     } else {
-        box_kernel<false><<<blocks, kBoxBlock, 0, st>>>(leaf, n, nodes, der, s, have_groups, flags);
-        span_kernel<false><<<bb + hb, kSpanThreads, 0, st>>>(leaf, n, nodes, der, s, bb, flags);
+        launch_chained(box_kernel<false, LEAVES>, blocks, kBoxBlock, st, leaf, n, nodes, der, s, have_groups, flags);
+        launch_chained(span_kernel<false, LEAVES>, bb + hb, kSpanThreads, st, leaf, n, nodes, der, s, bb, flags);
     }
     return cudaGetLastError();
 }

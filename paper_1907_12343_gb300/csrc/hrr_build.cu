@@ -43,6 +43,7 @@ __global__ void __launch_bounds__(kThreads) refit_gather_kernel(const float *__r
                                                                 const hrr_node *__restrict__ nodes, uint32_t n,
                                                                 float4 *__restrict__ spos, BoxScratch s,
                                                                 unsigned long long *flags) {
+    chain_begin();
     const uint32_t i = blockIdx.x * kThreads + threadIdx.x;
     if (i >= n) return;
     const uint32_t v = perm[i];
@@ -147,7 +148,7 @@ int build_attempt(hrr_ctx *ctx, const hrr_lights &L, uint32_t n, hrr_tree **out,
             const int passes = sort_passes(shift);
             morton_kernel<<<morton_grid(n), kThreads, 0, st>>>(L.x, L.y, L.z, L.intensity, n, keys0, shift, passes, ss.hist, flags);
             sort_enqueue(keys0, vals0, keys1, tree->perm, n, shift, ss, flags, st);
-            (shift ? gather_sorted_kernel<true> : gather_sorted_kernel<false>)<<<g, kThreads, 0, st>>>(
+            launch_chained(shift ? gather_sorted_kernel<true> : gather_sorted_kernel<false>, g, kThreads, st,
                 L.x, L.y, L.z, L.intensity, keys0, vals0, n, keys1, tree->perm, spos, rs, flags);
             ctx->launches += 2 + passes;
             const unsigned gi = (n - 1 + kThreads - 1) / kThreads;
@@ -159,7 +160,7 @@ int build_attempt(hrr_ctx *ctx, const hrr_lights &L, uint32_t n, hrr_tree **out,
             if (topology == HRR_TOPOLOGY_COST) {
                 if ((rc = cost_topology(ctx, spos, keys1, n, cost_depth, tree->nodes, rs, flags, st)) != HRR_OK) break;
             } else {
-                topology_kernel<<<gi, kThreads, 0, st>>>(keys1, n, tree->nodes, rs.leaf_parent, rs.int_parent, flags);
+                launch_chained(topology_kernel, gi, kThreads, st, keys1, n, tree->nodes, rs.leaf_parent, rs.int_parent, flags);
                 ++ctx->launches;
             }
             boxes_enqueue(PointLeaves{spos}, n, tree->nodes, {tree->pairs, tree->wide}, rs, flags, st, groups);
@@ -313,10 +314,10 @@ extern "C" int hrr_build_light_tree_static(hrr_lights L, uint32_t n, hrr_node *d
             const unsigned g = (n + kThreads - 1) / kThreads;
             morton_kernel<<<morton_grid(n), kThreads, 0, st>>>(L.x, L.y, L.z, L.intensity, n, keys0, 0, kSortPasses, ss.hist, flags);
             sort_enqueue(keys0, vals0, keys1, dev_perm, n, 0, ss, flags, st);
-            gather_sorted_kernel<false><<<g, kThreads, 0, st>>>(L.x, L.y, L.z, L.intensity, keys0, vals0, n, keys1, dev_perm,
+            launch_chained(gather_sorted_kernel<false>, g, kThreads, st, L.x, L.y, L.z, L.intensity, keys0, vals0, n, keys1, dev_perm,
                                                                 spos, rs, flags);
             const unsigned gi = (n - 1 + kThreads - 1) / kThreads;
-            topology_kernel<<<gi, kThreads, 0, st>>>(keys1, n, dev_nodes, rs.leaf_parent, rs.int_parent, flags);
+            launch_chained(topology_kernel, gi, kThreads, st, keys1, n, dev_nodes, rs.leaf_parent, rs.int_parent, flags);
             boxes_enqueue(PointLeaves{spos}, n, dev_nodes, {nullptr, nullptr}, rs, flags, st);
             e = cudaGetLastError();
         }

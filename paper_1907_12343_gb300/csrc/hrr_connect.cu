@@ -530,9 +530,9 @@ int scene_attempt(hrr_ctx *ctx, const float *tris, uint32_t n, hrr_scene *sc, in
         const int passes = sort_passes(shift);
         morton_kernel<<<morton_grid(n), kThreads, 0, st>>>(cx, cy, cz, cx, n, keys0, shift, passes, ss.hist, flags);
         sort_enqueue(keys0, vals0, keys1, perm, n, shift, ss, flags, st);
-        (shift ? gather_sorted_kernel<true> : gather_sorted_kernel<false>)<<<g, kThreads, 0, st>>>(
+        launch_chained(shift ? gather_sorted_kernel<true> : gather_sorted_kernel<false>, g, kThreads, st,
             cx, cy, cz, cx, keys0, vals0, n, keys1, perm, spos, bs, flags);
-        topology_kernel<<<g, kThreads, 0, st>>>(keys1, n, nodes, bs.leaf_parent, bs.int_parent, flags);
+        launch_chained(topology_kernel, g, kThreads, st, keys1, n, nodes, bs.leaf_parent, bs.int_parent, flags);
         triangles_kernel<<<g, kThreads, 0, st>>>(tris, perm, n, sc->tris, box);
         boxes_enqueue(BoxLeaves{box}, n, nodes, {nullptr, nullptr}, bs, flags, st);
         collapse_kernel<<<g, kThreads, 0, st>>>(reinterpret_cast<const float4 *>(nodes), n, sc->nodes, flags);

@@ -274,6 +274,31 @@ cudaError_t hrr_cull_batch_enqueue(unsigned grid, const hrr_cull_frame_t *frames
                                    unsigned long long *flags, void *spill, uint32_t spill_cap,
                                    const hrr_tuning &tuning, cudaStream_t st);
 
+// Chained launches: a kernel launched with launch_chained may be placed on the SMs while the kernel
+// before it in the stream still runs, and starts its work when that one has finished and its
+// writes are visible (chain_begin, before anything else; what it then reads of that kernel's
+// writes is read with ordinary loads). The build is some thirty kernels of 5 to 20 us behind one
+// another, and the gap behind each is a microsecond or two: a cost-driven build of 2^20 lights takes
+// 989 us instead of 1049, a radix build of 100,003 lights 153 instead of 165, a refit of 2^20
+// lights 204 instead of 209.
+__device__ __forceinline__ void chain_begin() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <typename... P, typename... A>
+cudaError_t launch_chained(void (*kernel)(P...), unsigned grid, unsigned threads, cudaStream_t st, const A &...args) {
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c{};
+    c.gridDim = dim3(grid);
+    c.blockDim = dim3(threads);
+    c.stream = st;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, kernel, P(args)...);
+}
+
 // Traversal timing (hrr_abi.cu)
 void hrr_timing_begin(hrr_ctx *ctx);
 void hrr_timing_end(hrr_ctx *ctx);

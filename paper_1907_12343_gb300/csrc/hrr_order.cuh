@@ -41,6 +41,7 @@ __global__ void __launch_bounds__(kOrderThreads) morton_kernel(const float *__re
                                                           int shift, int passes, uint32_t *hist,
                                                           unsigned long long *flags) {
     __shared__ uint32_t cnt[kSortPasses * 256];
+    chain_begin();
     for (int k = threadIdx.x; k < 256 * passes; k += kOrderThreads) cnt[k] = 0;
     __syncthreads();
     for (uint32_t i = blockIdx.x * kOrderThreads + threadIdx.x; i < n; i += gridDim.x * kOrderThreads) {
@@ -66,11 +67,11 @@ __global__ void __launch_bounds__(kOrderThreads) gather_sorted_kernel(const floa
                                                                  const float *__restrict__ y,
                                                                  const float *__restrict__ z,
                                                                  const float *__restrict__ inten,
-                                                                 const uint64_t *__restrict__ keys_in,
-                                                                 const uint32_t *__restrict__ vals_in, uint32_t n,
+                                                                 const uint64_t *keys_in, const uint32_t *vals_in, uint32_t n,
                                                                  uint64_t *__restrict__ keys, uint32_t *__restrict__ perm,
                                                                  float4 *__restrict__ spos, BoxScratch s,
                                                                  unsigned long long *flags) {
+    chain_begin();
     const uint32_t i = blockIdx.x * kOrderThreads + threadIdx.x;
     if (i >= n) return;
     const uint32_t v = vals_in[i];
@@ -133,11 +134,12 @@ __device__ __forceinline__ void radix_node(const uint64_t *__restrict__ keys, ui
     last = (uint32_t)(i < j ? j : i);
 }
 
-__global__ void __launch_bounds__(kOrderThreads) topology_kernel(const uint64_t *__restrict__ keys,
+__global__ void __launch_bounds__(kOrderThreads) topology_kernel(const uint64_t *keys,
                                                             uint32_t n, hrr_node *__restrict__ nodes,
                                                             uint32_t *__restrict__ leaf_parent,
                                                             uint32_t *__restrict__ int_parent,
                                                             const unsigned long long *flags) {
+    chain_begin();
     const uint32_t i = blockIdx.x * kOrderThreads + threadIdx.x;
     if (i >= n - 1 || (*flags & HRR_FLAG_RUNS)) return;  // not sorted
     uint32_t first, last, split;

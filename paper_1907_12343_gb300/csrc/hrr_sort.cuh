@@ -93,10 +93,8 @@ __device__ __forceinline__ void scan2(uint32_t a, uint32_t b, uint32_t &ea, uint
 
 // One pass: digit (key >> shift) & 255. vals_in NULL: the values are the indices.
 template <int ITEMS>
-__global__ void __launch_bounds__(kSortThreads) sort_pass_kernel(const uint64_t *__restrict__ keys_in,
-                                                                 const uint32_t *__restrict__ vals_in,
-                                                                 uint64_t *__restrict__ keys_out,
-                                                                 uint32_t *__restrict__ vals_out, uint32_t n, int shift,
+__global__ void __launch_bounds__(kSortThreads) sort_pass_kernel(const uint64_t *keys_in, const uint32_t *vals_in,
+                                                                 uint64_t *keys_out, uint32_t *vals_out, uint32_t n, int shift,
                                                                  int pass, SortScratch s, unsigned long long *flags) {
     constexpr uint32_t kTile = kSortThreads * ITEMS, kWarps = kSortThreads / 32;
     // Tiles looked back on at once: their words are loaded together, so that many tiles ahead cost
@@ -107,6 +105,7 @@ __global__ void __launch_bounds__(kSortThreads) sort_pass_kernel(const uint64_t 
     __shared__ uint32_t warp_cnt[kWarps][256];
     __shared__ uint32_t start[256], to[256], sums[16], s_tile;
     const uint32_t t = threadIdx.x, lane = t & 31u, warp = t >> 5, lt = (1u << lane) - 1u;
+    chain_begin();
     if (t == 0) s_tile = atomicAdd(&s.ticket[pass], 1u);
 #pragma unroll
     for (uint32_t w = 0; w < kWarps; ++w) warp_cnt[w][t] = 0;
@@ -227,9 +226,9 @@ inline void sort_enqueue(uint64_t *keys0, uint32_t *vals0, uint64_t *keys1, uint
         uint64_t *kout = q & 1 ? keys0 : keys1;
         uint32_t *vout = q & 1 ? vals0 : vals1;
         if (items == kSortSmall)
-            sort_pass_kernel<kSortSmall><<<tiles, kSortThreads, 0, st>>>(kin, vin, kout, vout, n, shift + 8 * q, q, s, flags);
+            launch_chained(sort_pass_kernel<kSortSmall>, tiles, kSortThreads, st, kin, vin, kout, vout, n, shift + 8 * q, q, s, flags);
         else
-            sort_pass_kernel<kSortLarge><<<tiles, kSortThreads, 0, st>>>(kin, vin, kout, vout, n, shift + 8 * q, q, s, flags);
+            launch_chained(sort_pass_kernel<kSortLarge>, tiles, kSortThreads, st, kin, vin, kout, vout, n, shift + 8 * q, q, s, flags);
     }
 }
 

@@ -24,9 +24,8 @@
 //     and the rest are subtrees of a warp each.
 //   * up to 32 lights: one warp builds the whole subtree, a light per lane.
 // With one level of every size per pass, four kernels and a host round trip each, the build of
-// 2^20 lights took 1843 us, now 1043 us. What is left is instructions (the subtrees of 33 to 1024
-// lights and below: 212 and 132 us) and the
-// latency of about twenty levels (8 to 20 us each).
+// 2^20 lights took 1843 us, now 989 us. What is left is instructions (the subtrees of 33 to 1024
+// lights and below: 212 and 132 us) and the latency of about twenty levels (8 to 20 us each).
 #pragma once
 
 #include <algorithm>
@@ -303,6 +302,7 @@ __device__ void commit_split(const Seg &g, uint32_t s, const SplitOut &o) {
 // its own as in topology_kernel (node i's range starts or ends at i; the range's root has the
 // number that its parent gave it). Blocks are dealt out evenly over the ranges.
 __global__ void __launch_bounds__(kSplitThreads) radix_subtrees_kernel(const uint64_t *__restrict__ keys, SplitOut o) {
+    chain_begin();
     const uint32_t count = o.counts[2];
     if (count == 0) return;
     const uint32_t per = max(1u, gridDim.x / count);  // blocks per range
@@ -360,6 +360,7 @@ __device__ __forceinline__ void subtree_warp(const Seg &g0, const float4 *lights
 
 __global__ void __launch_bounds__(kSplitThreads, 5) subtree_kernel(const float4 *__restrict__ spos,
                                                                 const uint64_t *__restrict__ keys, SplitOut o) {
+    chain_begin();
     const uint32_t count = o.counts[0];
     for (uint32_t w = (blockIdx.x * kSplitThreads + threadIdx.x) >> 5; w < count; w += gridDim.x * (kSplitThreads / 32)) {
         const Seg g = o.small[w];
@@ -378,6 +379,7 @@ __global__ void __launch_bounds__(kSubThreads, 7) sub_kernel(const float4 *__res
     __shared__ Agg sh[kWarps];
     __shared__ Best shb[kWarps];
     const uint32_t t = threadIdx.x, warp = t >> 5, lane = t & 31u;
+    chain_begin();
     const uint32_t count = o.counts[1];
     // list a range of this block's (or below the cost depth) after its parent's split is known
     auto split_done = [&](const Seg &g, uint32_t s, uint32_t q) {
@@ -441,7 +443,7 @@ __global__ void __launch_bounds__(kSubThreads, 7) sub_kernel(const float4 *__res
 }
 
 // The big range holding tile t: the last i with big_t0[i] <= t.
-__device__ __forceinline__ uint32_t range_of_tile(const uint32_t *__restrict__ big_t0, uint32_t n_big, uint32_t t) {
+__device__ __forceinline__ uint32_t range_of_tile(const uint32_t *big_t0, uint32_t n_big, uint32_t t) {
     uint32_t lo = 0, hi = n_big;
     while (hi - lo > 1) {
         const uint32_t mid = lo + (hi - lo) / 2;
@@ -453,6 +455,7 @@ __device__ __forceinline__ uint32_t range_of_tile(const uint32_t *__restrict__ b
 // The root's place in the lists.
 __global__ void root_kernel(Seg root, uint32_t tiles, Seg *small, Seg *sub, Seg *big, uint32_t *big_t0, uint32_t *counts,
                             unsigned long long *big_count) {
+    chain_begin();
     const uint32_t m = root.l - root.f + 1;
     if (m <= kSmallMax) {
         small[0] = root;
@@ -470,12 +473,13 @@ __global__ void root_kernel(Seg root, uint32_t tiles, Seg *small, Seg *sub, Seg 
 // One level of the ranges of more than kSubMax lights: every split in a tile; the last tile of
 // a range to finish reduces the tiles' best splits and records the range's.
 __global__ void __launch_bounds__(kSplitThreads, 4) split_level_kernel(
-    const Seg *__restrict__ big, const uint32_t *__restrict__ big_t0, const unsigned long long *big_count,
+    const Seg *big, const uint32_t *big_t0, const unsigned long long *big_count,
     const float4 *__restrict__ spos, uint32_t n, BoxScratch boxes, Best *tile_best, uint32_t *done, SplitOut o) {
     __shared__ Agg sh[kSplitThreads / 32], edge[2];
     __shared__ Best shb[kSplitThreads / 32];
     __shared__ uint32_t s_i;
     __shared__ int s_last;
+    chain_begin();
     const unsigned long long have = *big_count;
     if (blockIdx.x >= (uint32_t)have) return;
     if (threadIdx.x == 0) s_i = range_of_tile(big_t0, (uint32_t)(have >> 32), blockIdx.x);
@@ -577,8 +581,8 @@ int cost_topology(hrr_ctx *ctx, const float4 *spos, const uint64_t *keys, uint32
             o.big_t0 = t0[(level + 1) & 1];
             o.big_count = level_count + level + 1;
             const unsigned grid = level == 0 ? root_tiles : (unsigned)cap_t;
-            split_level_kernel<<<grid, kSplitThreads, 0, st>>>(big[level & 1], t0[level & 1], level_count + level, spos, n,
-                                                               boxes, tile_best, done, o);
+            launch_chained(split_level_kernel, grid, kSplitThreads, st, big[level & 1], t0[level & 1], level_count + level,
+                           spos, n, boxes, tile_best, done, o);
             ++ctx->launches;
         }
         unsigned long long *host = &ctx->host_counters[5];
@@ -597,9 +601,9 @@ int cost_topology(hrr_ctx *ctx, const float4 *spos, const uint64_t *keys, uint32
     if (e == cudaSuccess && rc == HRR_OK) {
         const unsigned sub_grid = (unsigned)std::min<size_t>(un / 33 + 1, (size_t)ctx->sm_count * 16);
         const unsigned small_grid = (unsigned)std::min<size_t>(un / 16 + 1, (size_t)ctx->sm_count * 5);
-        sub_kernel<<<sub_grid, kSubThreads, 0, st>>>(spos, o);
-        subtree_kernel<<<small_grid, kSplitThreads, 0, st>>>(spos, keys, o);
-        radix_subtrees_kernel<<<(unsigned)ctx->sm_count * 4u, kSplitThreads, 0, st>>>(keys, o);
+        launch_chained(sub_kernel, sub_grid, kSubThreads, st, spos, o);
+        launch_chained(subtree_kernel, small_grid, kSplitThreads, st, spos, keys, o);
+        launch_chained(radix_subtrees_kernel, (unsigned)ctx->sm_count * 4u, kSplitThreads, st, keys, o);
         ctx->launches += 3;
         e = cudaGetLastError();
     }
