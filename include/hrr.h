@@ -192,7 +192,7 @@ int hrr_build_light_tree(hrr_ctx *ctx, hrr_lights lights, uint32_t n_lights, hrr
  * P = dx + dy + dz of its box (float, each operation rounded separately; every split a
  * candidate; ties to the most even split, then the smaller one), and takes radix splits
  * below, which bound the height by cost_depth + 96. COST trees take fewer node visits to
- * cull (about 15% on the frame workload) and longer to build (1.0 ms for 2^20 lights). */
+ * cull (about 15% on the frame workload) and longer to build (0.9 ms for 2^20 lights). */
 typedef enum hrr_topology { HRR_TOPOLOGY_RADIX = 0, HRR_TOPOLOGY_COST = 1 } hrr_topology;
 
 typedef struct hrr_build_opts {

@@ -341,7 +341,7 @@ __device__ __forceinline__ uint32_t range_min_leaves(uint32_t a, uint32_t z, con
 // most n_lights - 1. Each step visits up to 32 nodes, one per lane. Everything rare shares a
 // test with something else that is rare: fewer than 32 entries or visits left; surviving leaves
 // or a corrupt record. That and the clamped range minimum took a step from 180 to 134 warp
-// instructions, the issue slots from 81% to 65%, and left the L1 data pipe as the limit (92% on
+// instructions, the issue slots from 81% to 65%, and left the L1 data pipe as the limit (95% on
 // 480x270 eyes and 2^20 lights: 42 wavefronts a step for the records, 8 for the stack).
 template <int VARIANT, uint32_t kRing>
 __device__ __forceinline__ uint32_t walk_pairs(const Frame &fr, const Eye &E, uint32_t j, int lane, uint2 *stack,
