@@ -242,11 +242,23 @@ __device__ __forceinline__ void store_wide(float4 *w, const float4 (&a)[4], cons
     store32(w + 4, a[2], make_float4(b[2].x, b[2].y, b[2].z, __uint_as_float(split1)));
     store32(w + 6, a3, make_float4(b3.x, b3.y, b3.z, __uint_as_float(other)));
 }
-// A node's record from its children's boxes.
+// A node's record from its children's boxes. OWN: an array of the library's, which is aligned. A
+// caller's array (a build without allocation) need not be aligned to more than a word: it takes
+// the 256-bit stores where its address allows them, else one word at a time.
+template <bool OWN>
 __device__ __forceinline__ void store_record(float4 *r, float4 a0, float4 b0, float4 a1, float4 b1, uint32_t split,
                                              uint32_t other) {
-    store32(r, a0, make_float4(b0.x, b0.y, b0.z, __uint_as_float(split)));
-    store32(r + 2, a1, make_float4(b1.x, b1.y, b1.z, __uint_as_float(other)));
+    b0.w = __uint_as_float(split);
+    b1.w = __uint_as_float(other);
+    if (OWN || ((uintptr_t)r & 31u) == 0) {
+        store32(r, a0, b0);
+        store32(r + 2, a1, b1);
+        return;
+    }
+    const float v[16] = {a0.x, a0.y, a0.z, a0.w, b0.x, b0.y, b0.z, b0.w, a1.x, a1.y, a1.z, a1.w, b1.x, b1.y, b1.z, b1.w};
+    volatile float *f = reinterpret_cast<volatile float *>(r);  // word by word: no wider store may be made of these
+#pragma unroll
+    for (int k = 0; k < 16; ++k) f[k] = v[k];
 }
 
 // A node's paired record (hrr_tree::pairs).
@@ -323,7 +335,7 @@ __global__ void __launch_bounds__(kBoxBlock, 3) box_kernel(LEAVES leaf, uint32_t
     __syncthreads();
     if (whole && arrived[t] == 2u) {
         const float4 a0 = sa[0][t], b0 = sb[0][t], a1 = sa[1][t], b1 = sb[1][t];
-        store_record(reinterpret_cast<float4 *>(nodes) + 4 * (size_t)g, a0, b0, a1, b1, split, other);
+        store_record<DERIVED>(reinterpret_cast<float4 *>(nodes) + 4 * (size_t)g, a0, b0, a1, b1, split, other);
         if (DERIVED) {  // the children's entries are in the block too
             const bool leaf0 = first == split, leaf1 = split + 1u == last;
             const uint32_t k0 = leaf0 ? t : split - base, k1 = leaf1 ? t : split + 1u - base;
@@ -414,8 +426,8 @@ __global__ void __launch_bounds__(kSpanThreads) span_kernel(LEAVES leaf, uint32_
         if (!DERIVED) {
             const Box x0 = box_range(leaf, s, n, first, split), x1 = box_range(leaf, s, n, split + 1u, last);
             if (lane == 0)
-                store_record(reinterpret_cast<float4 *>(nodes) + 4 * (size_t)g, box_a(x0), box_b(x0, 0u), box_a(x1),
-                             box_b(x1, 0u), split, other);
+                store_record<false>(reinterpret_cast<float4 *>(nodes) + 4 * (size_t)g, box_a(x0), box_b(x0, 0u), box_a(x1),
+                                    box_b(x1, 0u), split, other);
             continue;
         }
         // the grandchildren's boxes; the children's are their unions
@@ -432,8 +444,8 @@ __global__ void __launch_bounds__(kSpanThreads) span_kernel(LEAVES leaf, uint32_
             Box x0 = q[0], x1 = q[2];
             box_join(x0, q[1]);
             box_join(x1, q[3]);
-            store_record(reinterpret_cast<float4 *>(nodes) + 4 * (size_t)g, box_a(x0), box_b(x0, 0u), box_a(x1),
-                         box_b(x1, 0u), split, other);
+            store_record<true>(reinterpret_cast<float4 *>(nodes) + 4 * (size_t)g, box_a(x0), box_b(x0, 0u), box_a(x1),
+                               box_b(x1, 0u), split, other);
             const float4 a[4] = {box_a(q[0]), box_a(q[1]), box_a(q[2]), box_a(q[3])};
             const float4 b[4] = {box_b(q[0], 0u), box_b(q[1], 0u), box_b(q[2], 0u), box_b(q[3], 0u)};
             store_pairs(der.pairs + 4 * (size_t)hrr_node_slot(g, other), box_a(x0), box_b(x0, 0u), box_a(x1),
