@@ -255,7 +255,11 @@ __device__ __forceinline__ uint32_t meets(const uint32_t (&h)[8], const uint32_t
     for (int c = 0; c < 3; ++c) {
         const float S = __uint_as_float(((h[3] >> (8 * c)) & 255u) << 23);
         const float a = S * inv[c];
-        const float b = ((__uint_as_float(h[c]) - S) - e[c]) * inv[c];
+        // An axis whose start overflows (a nearly or wholly zero component on a node of some 1e8)
+        // would put both sides at the same infinity, even around an eye inside the node: 0 b + b
+        // makes it no number, which the minima and maxima below ignore, and the axis rejects nothing.
+        float b = ((__uint_as_float(h[c]) - S) - e[c]) * inv[c];
+        b = __fmaf_rn(b, 0.0f, b);
         slope[c] = hrr_pack2(a, a);
         start[c] = hrr_pack2(b, b);
         const bool back = inv[c] < 0.0f;
