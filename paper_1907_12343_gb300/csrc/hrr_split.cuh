@@ -301,10 +301,14 @@ __device__ void commit_split(const Seg &g, uint32_t s, const SplitOut &o) {
 // Ranges below the cost depth: the radix tree over each range's own keys, every node of it on
 // its own as in topology_kernel (node i's range starts or ends at i; the range's root has the
 // number that its parent gave it). Blocks are dealt out evenly over the ranges.
-__global__ void __launch_bounds__(kSplitThreads) radix_subtrees_kernel(const uint64_t *__restrict__ keys, SplitOut o) {
+// Nothing is done on keys that are not sorted (HRR_FLAG_RUNS: the build starts over), whose prefix
+// lengths can give a split outside its range; the kernels of the cost splits read no keys but in
+// searches that end inside a range.
+__global__ void __launch_bounds__(kSplitThreads) radix_subtrees_kernel(const uint64_t *__restrict__ keys, SplitOut o,
+                                                                       const unsigned long long *flags) {
     chain_begin();
     const uint32_t count = o.counts[2];
-    if (count == 0) return;
+    if (count == 0 || (*flags & HRR_FLAG_RUNS)) return;
     const uint32_t per = max(1u, gridDim.x / count);  // blocks per range
     for (uint32_t w = blockIdx.x; w < per * count; w += gridDim.x) {
         const Seg g = o.radix[w / per];
@@ -603,7 +607,7 @@ int cost_topology(hrr_ctx *ctx, const float4 *spos, const uint64_t *keys, uint32
         const unsigned small_grid = (unsigned)std::min<size_t>(un / 16 + 1, (size_t)ctx->sm_count * 5);
         launch_chained(sub_kernel, sub_grid, kSubThreads, st, spos, o);
         launch_chained(subtree_kernel, small_grid, kSplitThreads, st, spos, keys, o);
-        launch_chained(radix_subtrees_kernel, (unsigned)ctx->sm_count * 4u, kSplitThreads, st, keys, o);
+        launch_chained(radix_subtrees_kernel, (unsigned)ctx->sm_count * 4u, kSplitThreads, st, keys, o, flags);
         ctx->launches += 3;
         e = cudaGetLastError();
     }
