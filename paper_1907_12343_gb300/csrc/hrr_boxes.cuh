@@ -248,17 +248,16 @@ __device__ __forceinline__ void store_wide(float4 *w, const float4 (&a)[4], cons
 template <bool OWN>
 __device__ __forceinline__ void store_record(float4 *r, float4 a0, float4 b0, float4 a1, float4 b1, uint32_t split,
                                              uint32_t other) {
-    b0.w = __uint_as_float(split);
-    b1.w = __uint_as_float(other);
-    if (OWN || ((uintptr_t)r & 31u) == 0) {
-        store32(r, a0, b0);
-        store32(r + 2, a1, b1);
+    if (!OWN && ((uintptr_t)r & 31u) != 0) {
+        const float v[16] = {a0.x, a0.y, a0.z, a0.w, b0.x, b0.y, b0.z, __uint_as_float(split),
+                             a1.x, a1.y, a1.z, a1.w, b1.x, b1.y, b1.z, __uint_as_float(other)};
+        volatile float *f = reinterpret_cast<volatile float *>(r);  // word by word: no wider store may be made of these
+#pragma unroll
+        for (int k = 0; k < 16; ++k) f[k] = v[k];
         return;
     }
-    const float v[16] = {a0.x, a0.y, a0.z, a0.w, b0.x, b0.y, b0.z, b0.w, a1.x, a1.y, a1.z, a1.w, b1.x, b1.y, b1.z, b1.w};
-    volatile float *f = reinterpret_cast<volatile float *>(r);  // word by word: no wider store may be made of these
-#pragma unroll
-    for (int k = 0; k < 16; ++k) f[k] = v[k];
+    store32(r, a0, make_float4(b0.x, b0.y, b0.z, __uint_as_float(split)));
+    store32(r + 2, a1, make_float4(b1.x, b1.y, b1.z, __uint_as_float(other)));
 }
 
 // A node's paired record (hrr_tree::pairs).
