@@ -281,7 +281,7 @@ __global__ void __launch_bounds__(kBoxBlock, 3) box_kernel(LEAVES leaf, uint32_t
     __shared__ uint32_t arrived[kBoxBlock], up[kBoxBlock], cut[kBoxBlock];
     __shared__ bool inside[kBoxBlock];
     chain_begin();
-    if (*(volatile unsigned long long *)flags & (HRR_FLAG_NONFINITE | HRR_FLAG_RUNS)) return;  // set before the launch
+    if (*(volatile unsigned long long *)flags & (HRR_FLAG_NONFINITE | HRR_FLAG_UNSORTED)) return;  // set before the launch
     const uint32_t t = threadIdx.x, base = blockIdx.x * kBoxBlock, g = base + t;
     uint32_t split = 0, other = 0, first = 0, last = 0;
     bool whole = false;  // node g exists and lies inside the block
@@ -378,7 +378,7 @@ __global__ void __launch_bounds__(kSpanThreads) span_kernel(LEAVES leaf, uint32_
                                                             BoxScratch s, uint32_t box_blocks,
                                                             unsigned long long *flags) {
     chain_begin();
-    if (*(volatile unsigned long long *)flags & (HRR_FLAG_NONFINITE | HRR_FLAG_RUNS)) return;
+    if (*(volatile unsigned long long *)flags & (HRR_FLAG_NONFINITE | HRR_FLAG_UNSORTED)) return;
     const uint32_t count = *s.span_count;
     if (blockIdx.x >= box_blocks) {
         uint32_t h = 0;

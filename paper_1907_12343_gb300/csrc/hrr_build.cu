@@ -182,7 +182,8 @@ int build_attempt(hrr_ctx *ctx, const hrr_lights &L, uint32_t n, hrr_tree **out,
         fail(HRR_OK);
         return build_attempt(ctx, L, n, out, topology, cost_depth, 0);
     }
-    if (ctx->host_counters[2] & (HRR_FLAG_TOPOLOGY | HRR_FLAG_WAIT))
+    if (ctx->host_counters[2] & HRR_FLAG_WAIT) return fail(hrr_fail(ctx, HRR_ERR_TIMEOUT, "a wait of the sort ran out"));
+    if (ctx->host_counters[2] & HRR_FLAG_TOPOLOGY)
         return fail(hrr_fail(ctx, HRR_ERR_DEVICE, "inconsistent radix-tree links"));
     *out = tree;
     return HRR_OK;
@@ -337,7 +338,11 @@ extern "C" int hrr_build_light_tree_static(hrr_lights L, uint32_t n, hrr_node *d
         set_err(err, err_len, "a light position or intensity is not finite");
         return HRR_ERR_INVALID_ARG;
     }
-    if (host_flags & (HRR_FLAG_TOPOLOGY | HRR_FLAG_WAIT)) {
+    if (host_flags & HRR_FLAG_WAIT) {
+        set_err(err, err_len, "a wait of the sort ran out");
+        return HRR_ERR_TIMEOUT;
+    }
+    if (host_flags & HRR_FLAG_TOPOLOGY) {
         set_err(err, err_len, "inconsistent radix-tree links");
         return HRR_ERR_DEVICE;
     }

@@ -82,9 +82,9 @@ __device__ __forceinline__ void tri_box(const float *t, float lo[3], float hi[3]
 // here, so that one 256-bit load and one 32-bit load fetch a triangle) and their boxes.
 __global__ void __launch_bounds__(kThreads) triangles_kernel(const float *__restrict__ tri, const uint32_t *__restrict__ perm,
                                                              uint32_t n, float *__restrict__ sorted,
-                                                             float4 *__restrict__ box) {
+                                                             float4 *__restrict__ box, const unsigned long long *flags) {
     const uint32_t i = blockIdx.x * kThreads + threadIdx.x;
-    if (i >= n) return;
+    if (i >= n || (*flags & HRR_FLAG_WAIT)) return;  // no permutation
     const float *t = tri + 9 * (size_t)(perm ? perm[i] : i);
     float v[9];
     for (int c = 0; c < 9; ++c) v[c] = t[c];
@@ -111,7 +111,7 @@ struct BoxLeaves {
 __global__ void __launch_bounds__(kThreads) collapse_kernel(const float4 *__restrict__ nodes, uint32_t n,
                                                             uint32_t *__restrict__ out, const unsigned long long *flags) {
     const uint32_t g = blockIdx.x * kThreads + threadIdx.x;
-    if (g >= n - 1 || (*flags & (HRR_FLAG_NONFINITE | HRR_FLAG_RUNS | HRR_FLAG_TOPOLOGY))) return;
+    if (g >= n - 1 || (*flags & (HRR_FLAG_NONFINITE | HRR_FLAG_UNSORTED | HRR_FLAG_TOPOLOGY))) return;
     float4 lo[8], hi[8];
     uint32_t f[8], l[8], id[8];  // ranges and node numbers; an empty place has f > l
     for (int k = 0; k < 8; ++k) {
@@ -537,7 +537,7 @@ int scene_attempt(hrr_ctx *ctx, const float *tris, uint32_t n, hrr_scene *sc, in
         launch_chained(shift ? gather_sorted_kernel<true> : gather_sorted_kernel<false>, g, kThreads, st,
             cx, cy, cz, cx, keys0, vals0, n, keys1, perm, spos, bs, flags);
         launch_chained(topology_kernel, g, kThreads, st, keys1, n, nodes, bs.leaf_parent, bs.int_parent, flags);
-        triangles_kernel<<<g, kThreads, 0, st>>>(tris, perm, n, sc->tris, box);
+        triangles_kernel<<<g, kThreads, 0, st>>>(tris, perm, n, sc->tris, box, flags);
         boxes_enqueue(BoxLeaves{box}, n, nodes, {nullptr, nullptr}, bs, flags, st);
         collapse_kernel<<<g, kThreads, 0, st>>>(reinterpret_cast<const float4 *>(nodes), n, sc->nodes, flags);
         ctx->launches += 8 + passes;
@@ -551,7 +551,8 @@ int scene_attempt(hrr_ctx *ctx, const float *tris, uint32_t n, hrr_scene *sc, in
     const unsigned long long f = ctx->host_counters[2];
     if (f & HRR_FLAG_NONFINITE) return hrr_fail(ctx, HRR_ERR_INVALID_ARG, "a triangle vertex is not finite");
     if ((f & HRR_FLAG_RUNS) && shift) return scene_attempt(ctx, tris, n, sc, 0);
-    if (f & (HRR_FLAG_TOPOLOGY | HRR_FLAG_WAIT)) return hrr_fail(ctx, HRR_ERR_DEVICE, "scene links");
+    if (f & HRR_FLAG_WAIT) return hrr_fail(ctx, HRR_ERR_TIMEOUT, "a wait of the sort ran out");
+    if (f & HRR_FLAG_TOPOLOGY) return hrr_fail(ctx, HRR_ERR_DEVICE, "scene links");
     return HRR_OK;
 }
 
@@ -564,7 +565,7 @@ int scene_of_one(hrr_ctx *ctx, const float *tris, hrr_scene *sc) {
     cudaError_t e = cudaMemsetAsync(flags, 0, sizeof(unsigned long long), st);
     if (e == cudaSuccess) {
         centroid_kernel<<<1, kThreads, 0, st>>>(tris, 1u, cen, cen + 1, cen + 2, flags);
-        triangles_kernel<<<1, kThreads, 0, st>>>(tris, nullptr, 1u, sc->tris, nullptr);
+        triangles_kernel<<<1, kThreads, 0, st>>>(tris, nullptr, 1u, sc->tris, nullptr, flags);
         ctx->launches += 2;
         e = cudaGetLastError();
     }

@@ -12,7 +12,9 @@ enum : unsigned long long {
     HRR_FLAG_TOPOLOGY = 4ull,  // a node record or parent link is out of range
     HRR_FLAG_RANGE = 8ull,     // an input index (a pair's eye or light) is out of range
     HRR_FLAG_RUNS = 16ull,     // a build's keys have long runs of equal upper halves: sort them fully
-    HRR_FLAG_WAIT = 32ull,     // a bounded wait ran out (cannot happen)
+    HRR_FLAG_WAIT = 32ull,     // a bounded wait of the sort ran out (cannot happen)
+    // keys and values are not what the kernels after the sort take: in no order, or not written
+    HRR_FLAG_UNSORTED = HRR_FLAG_RUNS | HRR_FLAG_WAIT,
 };
 
 // ------------------------------------------------------------------------------------

@@ -61,7 +61,8 @@ inline unsigned morton_grid(uint32_t n) { return std::min(608u, (n + 4 * kOrderT
 // After the sort: sorted keys, permutation and lights, and the box pass's scratch reset. With
 // RUNS the keys are sorted by their upper halves only, and light i's place among the lights that
 // share its upper half is counted from their lower ones (ties by the order they are in); a run
-// of more than kRunMax lights raises HRR_FLAG_RUNS and stays as it is.
+// of more than kRunMax lights raises HRR_FLAG_RUNS and stays as it is. After a sort that gave up
+// nothing is done: its values index the lights.
 template <bool RUNS>
 __global__ void __launch_bounds__(kOrderThreads) gather_sorted_kernel(const float *__restrict__ x,
                                                                  const float *__restrict__ y,
@@ -73,7 +74,7 @@ __global__ void __launch_bounds__(kOrderThreads) gather_sorted_kernel(const floa
                                                                  unsigned long long *flags) {
     chain_begin();
     const uint32_t i = blockIdx.x * kOrderThreads + threadIdx.x;
-    if (i >= n) return;
+    if (i >= n || (*(volatile unsigned long long *)flags & HRR_FLAG_WAIT)) return;
     const uint32_t v = vals_in[i];
     const float4 p = make_float4(x[v], y[v], z[v], inten[v]);
     const uint64_t key = keys_in[i];
@@ -141,7 +142,7 @@ __global__ void __launch_bounds__(kOrderThreads) topology_kernel(const uint64_t 
                                                             const unsigned long long *flags) {
     chain_begin();
     const uint32_t i = blockIdx.x * kOrderThreads + threadIdx.x;
-    if (i >= n - 1 || (*flags & HRR_FLAG_RUNS)) return;  // not sorted
+    if (i >= n - 1 || (*flags & HRR_FLAG_UNSORTED)) return;
     uint32_t first, last, split;
     radix_node(keys, 0u, n - 1, i, first, last, split);
     nodes[i].split = split;

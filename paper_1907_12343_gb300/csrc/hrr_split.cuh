@@ -301,14 +301,14 @@ __device__ void commit_split(const Seg &g, uint32_t s, const SplitOut &o) {
 // Ranges below the cost depth: the radix tree over each range's own keys, every node of it on
 // its own as in topology_kernel (node i's range starts or ends at i; the range's root has the
 // number that its parent gave it). Blocks are dealt out evenly over the ranges.
-// Nothing is done on keys that are not sorted (HRR_FLAG_RUNS: the build starts over), whose prefix
+// Nothing is done on keys that are not sorted (the build starts over, or fails), whose prefix
 // lengths can give a split outside its range; the kernels of the cost splits read no keys but in
 // searches that end inside a range.
 __global__ void __launch_bounds__(kSplitThreads) radix_subtrees_kernel(const uint64_t *__restrict__ keys, SplitOut o,
                                                                        const unsigned long long *flags) {
     chain_begin();
     const uint32_t count = o.counts[2];
-    if (count == 0 || (*flags & HRR_FLAG_RUNS)) return;
+    if (count == 0 || (*flags & HRR_FLAG_UNSORTED)) return;
     const uint32_t per = max(1u, gridDim.x / count);  // blocks per range
     for (uint32_t w = blockIdx.x; w < per * count; w += gridDim.x) {
         const Seg g = o.radix[w / per];
@@ -594,7 +594,7 @@ int cost_topology(hrr_ctx *ctx, const float4 *spos, const uint64_t *keys, uint32
         if ((e = cudaMemcpyAsync(host, level_count + level, sizeof(*host), cudaMemcpyDeviceToHost, st)) != cudaSuccess) break;
         if ((e = cudaMemcpyAsync(&ctx->host_counters[2], flags, sizeof(*flags), cudaMemcpyDeviceToHost, st)) != cudaSuccess) break;
         if ((e = cudaStreamSynchronize(st)) != cudaSuccess) break;
-        if (ctx->host_counters[2] & (HRR_FLAG_RUNS | HRR_FLAG_NONFINITE)) break;  // the build starts over, or fails
+        if (ctx->host_counters[2] & (HRR_FLAG_UNSORTED | HRR_FLAG_NONFINITE)) break;  // the build starts over, or fails
         left = *host;
         if (left && level >= kLevels) {  // the radix split bounds the height
             rc = hrr_fail(ctx, HRR_ERR_DEVICE, "topology build did not terminate");
