@@ -180,7 +180,10 @@ int hrr_kernel_time(hrr_ctx *ctx, double *ms, uint64_t *launches);
  * (key, sorted position), and a bottom-up refit of boxes and maximum intensities. Leaf
  * i of the tree is the i-th light in sorted order; i is the index of the radical-inverse
  * sequence (Sec. 1: spatially sorted lights inherit the sequence's stratification).
- * 1 <= n_lights <= 2^31 - 1. Synchronises the context stream; returns
+ * 1 <= n_lights <= 2^31 - 1. Device memory: 324 bytes a light for the hierarchy, and up to 67
+ * more while it is built. Where that is not there the hierarchy does without its paired
+ * records and takes 196 bytes a light: every result stays the same, and culls of node width
+ * 2 take about a tenth longer. Synchronises the context stream; returns
  * HRR_ERR_INVALID_ARG if any position or intensity is not finite. */
 int hrr_build_light_tree(hrr_ctx *ctx, hrr_lights lights, uint32_t n_lights, hrr_tree **out);
 

@@ -39,6 +39,7 @@ cudaError_t hrr_alloc_bytes(hrr_ctx *ctx, void **p, size_t bytes) {
         *p = nullptr;
         if ((e = cudaStreamSynchronize(ctx->stream)) == cudaSuccess && (e = cudaMemPoolTrimTo(ctx->pool, 0)) == cudaSuccess)
             e = cudaMallocFromPoolAsync(p, bytes, ctx->pool, ctx->stream);
+        if (e == cudaErrorMemoryAllocation) cudaGetLastError();  // reported by the return value, not by a later launch
     }
     return e;
 }

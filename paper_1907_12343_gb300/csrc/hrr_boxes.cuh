@@ -61,18 +61,19 @@ struct BoxScratch {
     uint32_t *arrived;                   // per group: parts of it that are done
 };
 
-constexpr size_t box_scratch_bytes(uint32_t n) {
+// child_height false: the caller has 8 bytes a leaf for those itself.
+constexpr size_t box_scratch_bytes(uint32_t n, bool child_height = true) {
     const size_t un = n, g = box_groups_total(n) + 1;
-    return 3 * pad256(sizeof(uint32_t) * un) + pad256(sizeof(uint32_t) * 2 * un) + 2 * pad256(sizeof(uint32_t)) +
+    return 3 * pad256(sizeof(uint32_t) * un) + (child_height ? pad256(sizeof(uint32_t) * 2 * un) : 0) + 2 * pad256(sizeof(uint32_t)) +
            pad256(2 * sizeof(float4) * g) + pad256(sizeof(uint32_t) * g);
 }
-inline BoxScratch carve_boxes(char *&p, uint32_t n) {
+inline BoxScratch carve_boxes(char *&p, uint32_t n, bool child_height = true) {
     const size_t un = n, g = box_groups_total(n) + 1;
     BoxScratch s;
     s.leaf_parent = carve<uint32_t>(p, un);
     s.int_parent = carve<uint32_t>(p, un);
     s.span = carve<uint32_t>(p, un);
-    s.child_height = carve<uint32_t>(p, 2 * un);
+    s.child_height = child_height ? carve<uint32_t>(p, 2 * un) : nullptr;
     s.span_count = carve<uint32_t>(p, 1);
     s.root_height = carve<uint32_t>(p, 1);
     s.groups = carve<float4>(p, 2 * g);
@@ -268,13 +269,14 @@ __device__ __forceinline__ void store_pairs(float4 *r, float4 a0, float4 b0, flo
             make_float4(a0.w, a1.w, __uint_as_float(split), __uint_as_float(other)));
 }
 
-// The records derived from the binary ones, or none (scenes, builds into caller's arrays).
+// The records derived from the binary ones, or none (scenes, builds into caller's arrays); pairs
+// alone may be missing. DERIVED below: 0 none, 1 the top slots and the width-four records, 2 all.
 struct Derived {
     float4 *pairs, *wide;
 };
 
 // The nodes inside blocks, the groups, the list of spanning nodes.
-template <bool DERIVED, typename LEAVES>
+template <int DERIVED, typename LEAVES>
 __global__ void __launch_bounds__(kBoxBlock, 3) box_kernel(LEAVES leaf, uint32_t n, hrr_node *nodes, Derived der,
                                                         BoxScratch s, bool have_groups, unsigned long long *flags) {
     __shared__ float4 sa[2][kBoxBlock], sb[2][kBoxBlock];  // child: (low, imax), (high, height)
@@ -334,13 +336,13 @@ __global__ void __launch_bounds__(kBoxBlock, 3) box_kernel(LEAVES leaf, uint32_t
     __syncthreads();
     if (whole && arrived[t] == 2u) {
         const float4 a0 = sa[0][t], b0 = sb[0][t], a1 = sa[1][t], b1 = sb[1][t];
-        store_record<DERIVED>(reinterpret_cast<float4 *>(nodes) + 4 * (size_t)g, a0, b0, a1, b1, split, other);
+        store_record<(DERIVED > 0)>(reinterpret_cast<float4 *>(nodes) + 4 * (size_t)g, a0, b0, a1, b1, split, other);
         if (DERIVED) {  // the children's entries are in the block too
             const bool leaf0 = first == split, leaf1 = split + 1u == last;
             const uint32_t k0 = leaf0 ? t : split - base, k1 = leaf1 ? t : split + 1u - base;
             const float4 a[4] = {sa[0][k0], sa[1][k0], leaf1 ? a1 : sa[0][k1], sa[1][k1]};
             const float4 b[4] = {sb[0][k0], sb[1][k0], leaf1 ? b1 : sb[0][k1], sb[1][k1]};
-            store_pairs(der.pairs + 4 * (size_t)hrr_node_slot(g, other), a0, b0, a1, b1, split, other);
+            if (DERIVED > 1) store_pairs(der.pairs + 4 * (size_t)hrr_node_slot(g, other), a0, b0, a1, b1, split, other);
             store_wide(der.wide + 8 * (size_t)g, a, b, leaf0, leaf1, leaf0 ? split : cut[k0], split, leaf1 ? last : cut[k1],
                        other);
         }
@@ -373,7 +375,7 @@ __device__ __forceinline__ uint32_t top_walk(uint32_t s, const hrr_node *nodes, 
 // The nodes that span blocks (a warp each), the top slots (a warp each), and the height (a
 // thread per spanning node: its depth by the parent links, plus the heights of its children
 // inside blocks). Blocks [0, box_blocks) do the first two, the others the last.
-template <bool DERIVED, typename LEAVES>
+template <int DERIVED, typename LEAVES>
 __global__ void __launch_bounds__(kSpanThreads) span_kernel(LEAVES leaf, uint32_t n, hrr_node *nodes, Derived der,
                                                             BoxScratch s, uint32_t box_blocks,
                                                             unsigned long long *flags) {
@@ -447,8 +449,9 @@ __global__ void __launch_bounds__(kSpanThreads) span_kernel(LEAVES leaf, uint32_
                                box_b(x1, 0u), split, other);
             const float4 a[4] = {box_a(q[0]), box_a(q[1]), box_a(q[2]), box_a(q[3])};
             const float4 b[4] = {box_b(q[0], 0u), box_b(q[1], 0u), box_b(q[2], 0u), box_b(q[3], 0u)};
-            store_pairs(der.pairs + 4 * (size_t)hrr_node_slot(g, other), box_a(x0), box_b(x0, 0u), box_a(x1),
-                        box_b(x1, 0u), split, other);
+            if (DERIVED > 1)
+                store_pairs(der.pairs + 4 * (size_t)hrr_node_slot(g, other), box_a(x0), box_b(x0, 0u), box_a(x1),
+                            box_b(x1, 0u), split, other);
             store_wide(der.wide + 8 * (size_t)g, a, b, leaf0, leaf1, split0, split, split1, other);
         }
     }
@@ -462,13 +465,13 @@ cudaError_t boxes_enqueue(const LEAVES &leaf, uint32_t n, hrr_node *nodes, const
                           unsigned long long *flags, cudaStream_t st, bool have_groups = false) {
     const unsigned blocks = (n + kBoxBlock - 1) / kBoxBlock;
     const unsigned bb = std::min(608u, 8u + blocks), hb = std::min(152u, 1u + blocks / 16u);
-    if (der.wide) {
-        launch_chained(box_kernel<true, LEAVES>, blocks, kBoxBlock, st, leaf, n, nodes, der, s, have_groups, flags);
-        launch_chained(span_kernel<true, LEAVES>, bb + hb, kSpanThreads, st, leaf, n, nodes, der, s, bb, flags);
-    } else {
-        launch_chained(box_kernel<false, LEAVES>, blocks, kBoxBlock, st, leaf, n, nodes, der, s, have_groups, flags);
-        launch_chained(span_kernel<false, LEAVES>, bb + hb, kSpanThreads, st, leaf, n, nodes, der, s, bb, flags);
-    }
+    const auto run = [&](auto box, auto span) {
+        launch_chained(box, blocks, kBoxBlock, st, leaf, n, nodes, der, s, have_groups, flags);
+        launch_chained(span, bb + hb, kSpanThreads, st, leaf, n, nodes, der, s, bb, flags);
+    };
+    if (der.pairs) run(box_kernel<2, LEAVES>, span_kernel<2, LEAVES>);
+    else if (der.wide) run(box_kernel<1, LEAVES>, span_kernel<1, LEAVES>);
+    else run(box_kernel<0, LEAVES>, span_kernel<0, LEAVES>);
     return cudaGetLastError();
 }
 

@@ -88,7 +88,7 @@ __global__ void single_leaf_kernel(const float *x, const float *y, const float *
     if (!der.wide) return;
     const float4 *r = reinterpret_cast<const float4 *>(node);
     const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-    store_pairs(der.pairs, r[0], r[1], r[0], r[1], 0u, 0u);
+    if (der.pairs) store_pairs(der.pairs, r[0], r[1], r[0], r[1], 0u, 0u);
     for (int k = 0; k < 8; ++k) der.wide[k] = k < 2 ? r[k] : zero;
     for (uint32_t k = 0; k < 3 * HRR_TOP_SLOTS; ++k) reinterpret_cast<float4 *>(node)[4 + k] = zero;
 }
@@ -97,9 +97,9 @@ __global__ void single_leaf_kernel(const float *x, const float *y, const float *
 
 namespace {
 
-// Sorts by the key bits from `shift` up (kTopShift, or 0 for all).
+// Sorts by the key bits from `shift` up (kTopShift, or 0 for all); with the paired records or without.
 int build_attempt(hrr_ctx *ctx, const hrr_lights &L, uint32_t n, hrr_tree **out, int topology, uint32_t cost_depth,
-                  int shift) {
+                  int shift, bool paired) {
     cudaStream_t st = ctx->stream;
     hrr_tree *tree = new (std::nothrow) hrr_tree();
     if (!tree) return hrr_fail(ctx, HRR_ERR_OOM, "host allocation of the tree");
@@ -116,7 +116,7 @@ int build_attempt(hrr_ctx *ctx, const hrr_lights &L, uint32_t n, hrr_tree **out,
     const uint32_t n_rec = n > 1 ? n - 1 : 1;
     cudaError_t e = hrr_alloc(ctx, &tree->nodes, sizeof(hrr_node) * (size_t)n_rec + HRR_TOP_BYTES);
     if (e == cudaSuccess) e = hrr_alloc(ctx, &tree->perm, sizeof(uint32_t) * (size_t)n);
-    if (e == cudaSuccess) e = hrr_alloc(ctx, &tree->pairs, 8 * sizeof(float4) * (size_t)n_rec);
+    if (e == cudaSuccess && paired) e = hrr_alloc(ctx, &tree->pairs, 8 * sizeof(float4) * (size_t)n_rec);
     if (e == cudaSuccess) e = hrr_alloc(ctx, &tree->wide, 8 * sizeof(float4) * (size_t)n_rec);
     if (e != cudaSuccess) return fail(hrr_cuda_fail(ctx, e, "tree allocation"));
     unsigned long long *flags = ctx->counters + 2;
@@ -131,7 +131,7 @@ int build_attempt(hrr_ctx *ctx, const hrr_lights &L, uint32_t n, hrr_tree **out,
         tree->height = 0;
     } else {
         const size_t bytes = 2 * pad256(sizeof(uint64_t) * (size_t)n) + pad256(sizeof(uint32_t) * (size_t)n) +
-                             pad256(sort_scratch_bytes(n)) + pad256(sizeof(float4) * (size_t)n) + box_scratch_bytes(n);
+                             pad256(sort_scratch_bytes(n)) + pad256(sizeof(float4) * (size_t)n) + box_scratch_bytes(n, false);
         char *scratch = nullptr;
         if ((e = hrr_alloc(ctx, &scratch, bytes)) != cudaSuccess) return fail(hrr_cuda_fail(ctx, e, "build scratch"));
         char *p = scratch;
@@ -139,7 +139,8 @@ int build_attempt(hrr_ctx *ctx, const hrr_lights &L, uint32_t n, hrr_tree **out,
         uint32_t *vals0 = carve<uint32_t>(p, n);
         const SortScratch ss = carve_sort(p, n);
         float4 *spos = carve<float4>(p, n);
-        const BoxScratch rs = carve_boxes(p, n);
+        BoxScratch rs = carve_boxes(p, n, false);
+        rs.child_height = reinterpret_cast<uint32_t *>(keys0);  // the gather is the last to read those keys
 
         const unsigned g = (n + kThreads - 1) / kThreads;
         int rc = HRR_OK;
@@ -180,7 +181,7 @@ int build_attempt(hrr_ctx *ctx, const hrr_lights &L, uint32_t n, hrr_tree **out,
         return fail(hrr_fail(ctx, HRR_ERR_INVALID_ARG, "a light position or intensity is not finite"));
     if ((ctx->host_counters[2] & HRR_FLAG_RUNS) && shift) {  // many lights in few cells: every key bit sorted
         fail(HRR_OK);
-        return build_attempt(ctx, L, n, out, topology, cost_depth, 0);
+        return build_attempt(ctx, L, n, out, topology, cost_depth, 0, paired);
     }
     if (ctx->host_counters[2] & HRR_FLAG_WAIT) return fail(hrr_fail(ctx, HRR_ERR_TIMEOUT, "a wait of the sort ran out"));
     if (ctx->host_counters[2] & HRR_FLAG_TOPOLOGY)
@@ -192,7 +193,10 @@ int build_attempt(hrr_ctx *ctx, const hrr_lights &L, uint32_t n, hrr_tree **out,
 }  // namespace
 
 int hrr_build_impl(hrr_ctx *ctx, const hrr_lights &L, uint32_t n, hrr_tree **out, int topology, uint32_t cost_depth) {
-    return build_attempt(ctx, L, n, out, topology, cost_depth, kTopShift);
+    int rc = build_attempt(ctx, L, n, out, topology, cost_depth, kTopShift, true);
+    if (rc == HRR_ERR_OOM)  // the paired records are what a hierarchy can do without
+        rc = build_attempt(ctx, L, n, out, topology, cost_depth, kTopShift, false);
+    return rc;
 }
 
 // ------------------------------------------------------------------------------------

@@ -127,7 +127,8 @@ size_t hrr_cull_spill_entries(unsigned grid, uint32_t height, const hrr_tuning &
 }
 
 const float4 *hrr_cull_records(const hrr_tree *tree, const hrr_tuning &tuning) {
-    return tuning.node_width == 4 ? tree->wide : tree->pairs;
+    if (tuning.node_width == 4) return tree->wide;
+    return tree->pairs ? tree->pairs : reinterpret_cast<const float4 *>(tree->nodes);
 }
 
 namespace {
@@ -153,6 +154,7 @@ Frame single_frame(const hrr_ctx *ctx, const hrr_eyes &E, const hrr_tree *tree, 
     Frame fr{};
     fr.ex = E.x; fr.ey = E.y; fr.ez = E.z; fr.px = E.px; fr.py = E.py;
     fr.nodes = hrr_cull_records(tree, tn);
+    fr.paired = tree->pairs != nullptr;
     fr.top = hrr_tree_top(tree);
     fr.perm = tree->perm;
     fr.tile = hrr_tile_layer(ctx->tile, ctx->tile_w, ctx->tile_h, ctx->tile_d, opts.sample_index);

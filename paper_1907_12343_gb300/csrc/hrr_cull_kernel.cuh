@@ -80,7 +80,7 @@ constexpr int min_blocks(int threads) {
 }
 
 using Frame = hrr_cull_frame_t;
-static_assert(sizeof(Frame) == 136, "frame descriptor layout");
+static_assert(sizeof(Frame) == 144, "frame descriptor layout");
 
 struct Launch {
     uint32_t n_frames;
@@ -251,9 +251,11 @@ __device__ __forceinline__ uint2 queued(uint32_t node, uint32_t t, uint32_t ligh
 }
 
 // The light (position, intensity) at place t of a record.
-template <int W>
+template <int W, bool PAIRED>
 __device__ __forceinline__ float4 light_of(const float4 *records, uint32_t node, uint32_t t) {
-    if constexpr (W == 2) {
+    if constexpr (W == 2 && !PAIRED) {
+        return __ldg(&records[4 * (size_t)hrr_slot_node(node) + 2u * t]);
+    } else if constexpr (W == 2) {
         const float *p = reinterpret_cast<const float *>(records + 4 * (size_t)node) + t;
         return make_float4(-__ldg(p), -__ldg(p + 2), -__ldg(p + 4), __ldg(p + 12));
     } else {
@@ -262,7 +264,7 @@ __device__ __forceinline__ float4 light_of(const float4 *records, uint32_t node,
 }
 
 // Take the n <= 32 newest of the warp's queued leaves.
-template <int W>
+template <int W, bool PAIRED>
 __device__ __forceinline__ void take_queued(const Frame &fr, const Eye &E, uint32_t j, int lane, const uint2 *q,
                                             uint32_t n) {
     const bool has = (uint32_t)lane < n;
@@ -272,7 +274,7 @@ __device__ __forceinline__ void take_queued(const Frame &fr, const Eye &E, uint3
         const uint2 e = q[lane];
         const uint32_t t = (W == 2 ? 0u : e.x >> 31 << 1) | (e.y >> 31);
         i = e.y & 0x7FFFFFFFu;
-        l = light_of<W>(fr.nodes, W == 2 ? e.x : e.x & 0x7FFFFFFFu, t);
+        l = light_of<W, PAIRED>(fr.nodes, W == 2 ? e.x : e.x & 0x7FFFFFFFu, t);
     }
     __syncwarp();
     take(fr, E, j, lane, has, l, i);
@@ -342,14 +344,16 @@ __device__ __forceinline__ uint32_t range_min_leaves(uint32_t a, uint32_t z, con
 // test with something else that is rare: fewer than 32 entries or visits left; surviving leaves
 // or a corrupt record. That and the clamped range minimum took a step from 180 to 134 warp
 // instructions, the issue slots from 81% to 65%, and left the L1 data pipe as the limit (95% on
-// 480x270 eyes and 2^20 lights: 42 wavefronts a step for the records, 8 for the stack).
-template <int VARIANT, uint32_t kRing>
+// 480x270 eyes and 2^20 lights: 42 wavefronts a step for the records, 8 for the stack). PAIRED is
+// false for a tree without paired records: the same walk over its binary ones (5.58 ms instead of
+// 5.12 on those eyes and lights, 24.2 instead of 20.6 on 960x540).
+template <int VARIANT, uint32_t kRing, bool PAIRED>
 __device__ __forceinline__ uint32_t walk_pairs(const Frame &fr, const Eye &E, uint32_t j, int lane, uint2 *stack,
                                                uint2 *queue, uint32_t R, uint32_t before, uint2 *spill,
                                                uint32_t spill_cap, unsigned long long *flags) {
     const unsigned lt = (1u << lane) - 1u;
     const uint32_t n_lights = fr.n_lights;
-    const float4 *pairs = fr.nodes;
+    const float4 *records = fr.nodes;
     const hrr_f2 ex = hrr_pack2(E.x, E.x), ey = hrr_pack2(E.y, E.y), ez = hrr_pack2(E.z, E.z);
     uint32_t P = 0;         // older entries, in the spill area
     uint32_t queued_n = 0;  // surviving leaves still to be taken
@@ -384,9 +388,13 @@ __device__ __forceinline__ uint32_t walk_pairs(const Frame &fr, const Eye &E, ui
         __syncwarp();
 
         hrr_f2 nlox, nloy, nloz, nhix, nhiy, nhiz, imax, links;
-        load32(&pairs[4 * (size_t)e.x], nlox, nloy, nloz, nhix);
-        load32(&pairs[4 * (size_t)e.x + 2], nhiy, nhiz, imax, links);
         const uint32_t node = hrr_slot_node(e.x);
+        if constexpr (PAIRED) {
+            load32(&records[4 * (size_t)e.x], nlox, nloy, nloz, nhix);
+            load32(&records[4 * (size_t)e.x + 2], nhiy, nhiz, imax, links);
+        } else {
+            hrr_load_binary(&records[4 * (size_t)node], nlox, nloy, nloz, nhix, nhiy, nhiz, imax, links);
+        }
         const uint32_t split = (uint32_t)links, other = (uint32_t)(links >> 32);
         const uint32_t first = min(node, other), last = max(node, other);
         // needs first <= split < last < n
@@ -438,11 +446,11 @@ __device__ __forceinline__ uint32_t walk_pairs(const Frame &fr, const Eye &E, ui
             __syncwarp();
             while (queued_n >= 32u) {
                 queued_n -= 32u;
-                take_queued<2>(fr, E, j, lane, queue + queued_n, 32u);
+                take_queued<2, PAIRED>(fr, E, j, lane, queue + queued_n, 32u);
             }
         }
     }
-    if (queued_n) take_queued<2>(fr, E, j, lane, queue, queued_n);
+    if (queued_n) take_queued<2, PAIRED>(fr, E, j, lane, queue, queued_n);
     return n_lights - before - (uint32_t)left;
 }
 
@@ -513,7 +521,8 @@ __device__ __forceinline__ void traverse(const Launch &Lc, const Frame *F) {
         E.r = fr.tile[ty * fr.tile_w + tx] + fr.shift_offset;
         if (n_lights == 1) {  // the root is a leaf (record 0, slot 0, in either layout)
             if (lane == 0 && fr.eye_visits) fr.eye_visits[j] = 0;
-            take(fr, E, j, lane, lane == 0, light_of<W>(nodes, 0u, 0u), 0u);
+            const float4 l = fr.paired ? light_of<W, true>(nodes, 0u, 0u) : light_of<W, false>(nodes, 0u, 0u);
+            take(fr, E, j, lane, lane == 0, l, 0u);
             continue;
         }
         E.c = __brev(0u - E.r);
@@ -530,8 +539,10 @@ __device__ __forceinline__ void traverse(const Launch &Lc, const Frame *F) {
             __syncwarp();
         }
         if constexpr (W == 2) {
-            visits += walk_pairs<VARIANT, kRing>(fr, E, j, lane, ring, queue, S, visits, HRR_WARP_SPILL, Lc.spill_cap,
-                                                 Lc.flags);
+            visits += fr.paired ? walk_pairs<VARIANT, kRing, true>(fr, E, j, lane, ring, queue, S, visits, HRR_WARP_SPILL,
+                                                                   Lc.spill_cap, Lc.flags)
+                                : walk_pairs<VARIANT, kRing, false>(fr, E, j, lane, ring, queue, S, visits, HRR_WARP_SPILL,
+                                                                    Lc.spill_cap, Lc.flags);
         } else {
             while (S > 0) {
                 if (visits >= n_lights) {  // each internal node is visited at most once per eye
@@ -610,11 +621,11 @@ __device__ __forceinline__ void traverse(const Launch &Lc, const Frame *F) {
                     __syncwarp();
                     while (queued_n >= 32u) {
                         queued_n -= 32u;
-                        take_queued<W>(fr, E, j, lane, queue + queued_n, 32u);
+                        take_queued<W, false>(fr, E, j, lane, queue + queued_n, 32u);
                     }
                 }
             }
-            if (queued_n) take_queued<W>(fr, E, j, lane, queue, queued_n);
+            if (queued_n) take_queued<W, false>(fr, E, j, lane, queue, queued_n);
         }
         if (lane == 0) {
             uint32_t *ev = frame_at<BATCH>(F, f).eye_visits;

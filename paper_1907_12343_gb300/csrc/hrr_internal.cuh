@@ -112,7 +112,8 @@ struct hrr_tree {
     // distinct lines per load: 1.5e11 scattered records a second come out of L2 when every
     // record is a line of its own, 1.9e11 when siblings are neighbours on any 64 bytes, 2.9e11
     // when they share a line. 2n - 2 slots (half of them leaves'); one (the leaf in both
-    // places) when n == 1.
+    // places) when n == 1. They take 128 bytes a light besides the 196 of the rest, so a build that
+    // has no memory for them does without (null), and traversals read the binary records.
     float4 *pairs = nullptr;
     // The same hierarchy read with nodes of width four: for every internal node g a
     // 128-byte record of its four grandchild slots (hrr_build.cu), at index g; a
@@ -190,7 +191,7 @@ struct DeviceGuard {
 };
 
 // One frame of a traversal launch, as the kernel reads it (hrr_cull_kernel.cuh): a single frame
-// for hrr_cull, an array of them for batches. 136 bytes.
+// for hrr_cull, an array of them for batches. 144 bytes.
 struct hrr_cull_frame_t {
     const float *ex, *ey, *ez;
     const uint16_t *px, *py;
@@ -206,6 +207,7 @@ struct hrr_cull_frame_t {
     float tau;
     uint32_t eye_begin;              // first eye of the frame covered by this launch
     unsigned long long cursor_begin; // where the frame's eyes start on the launch's cursor
+    bool paired;                     // width two: the records are hrr_tree::pairs, not its nodes
 };
 
 // Traversal defaults (the fastest form on the 1920x1080-eye, 2^20-light frame): node width,
@@ -250,7 +252,7 @@ inline bool hrr_tuning_valid(const hrr_tuning &t0) {
 }
 
 // The traversal (hrr_cull_kernel.cuh). Frames of one batched launch (their descriptors are
-// kernel parameters: 128 x 136 bytes):
+// kernel parameters: 128 x 144 bytes):
 #define HRR_CULL_MAX_FRAMES 128u
 // Blocks of a traversal launch over `total` eyes (a whole number per SM, at most one warp per
 // eye), for the single-frame or the batched kernel of a (normalised, valid) tuning.
@@ -262,7 +264,8 @@ int hrr_cull_max_blocks(const hrr_tuning &tuning, bool batch);
 // (8 bytes each) for a grid of the tuning's blocks.
 uint32_t hrr_cull_spill_cap(uint32_t height, uint32_t width);
 size_t hrr_cull_spill_entries(unsigned grid, uint32_t height, const hrr_tuning &tuning);
-// The node records a traversal of the tuning's width reads (tree->pairs or tree->wide).
+// The node records a traversal of the tuning's width reads (tree->wide; tree->pairs, or the binary
+// records of a tree without).
 const float4 *hrr_cull_records(const hrr_tree *tree, const hrr_tuning &tuning);
 // Enqueue one batched traversal over n_frames <= HRR_CULL_MAX_FRAMES frames (host array, copied
 // into the launch) on st; a no-op when total == 0. A single frame runs the single-frame

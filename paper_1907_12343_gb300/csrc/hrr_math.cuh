@@ -247,3 +247,23 @@ __device__ __forceinline__ void hrr_survive2(hrr_f2 den, hrr_f2 rhs, uint32_t v0
     s0 = ok && !(l0 >= r0);
     s1 = ok && !(l1 >= r1);
 }
+
+// The paired form (hrr_tree::pairs) of a binary record, for trees without paired records.
+__device__ __forceinline__ void hrr_load_binary(const float4 *p, hrr_f2 &nlox, hrr_f2 &nloy, hrr_f2 &nloz, hrr_f2 &nhix,
+                                                hrr_f2 &nhiy, hrr_f2 &nhiz, hrr_f2 &imax, hrr_f2 &links) {
+    float4 q[4];
+#pragma unroll
+    for (int k = 0; k < 4; k += 2)
+        asm("ld.global.nc.L1::no_allocate.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+            : "=f"(q[k].x), "=f"(q[k].y), "=f"(q[k].z), "=f"(q[k].w), "=f"(q[k + 1].x), "=f"(q[k + 1].y), "=f"(q[k + 1].z),
+              "=f"(q[k + 1].w)
+            : "l"(p + k));
+    nlox = hrr_pack2(-q[0].x, -q[2].x);
+    nloy = hrr_pack2(-q[0].y, -q[2].y);
+    nloz = hrr_pack2(-q[0].z, -q[2].z);
+    nhix = hrr_pack2(-q[1].x, -q[3].x);
+    nhiy = hrr_pack2(-q[1].y, -q[3].y);
+    nhiz = hrr_pack2(-q[1].z, -q[3].z);
+    imax = hrr_pack2(q[0].w, q[2].w);
+    links = hrr_pack2(q[1].w, q[3].w);
+}

@@ -35,7 +35,7 @@ constexpr int kMinBlocks = 5;    // resident blocks per SM the register budget i
 struct SampleLaunch {
     const float *ex, *ey, *ez;
     const uint16_t *px, *py;
-    const float4 *pairs_rec;      // the paired records (hrr_tree::pairs)
+    const float4 *records;        // the paired records (hrr_tree::pairs), or the binary ones
     const uint32_t *perm;
     const uint32_t *tile;         // d layers of w x h
     uint32_t tile_w, tile_h, tile_d;
@@ -59,6 +59,14 @@ __device__ __forceinline__ void load_pairs(const float4 *p, hrr_f2 &a, hrr_f2 &b
                                            hrr_f2 &g, hrr_f2 &h) {
     asm("ld.global.nc.L1::no_allocate.v4.b64 {%0,%1,%2,%3}, [%4];" : "=l"(a), "=l"(b), "=l"(c), "=l"(d) : "l"(p));
     asm("ld.global.nc.L1::no_allocate.v4.b64 {%0,%1,%2,%3}, [%4+32];" : "=l"(e), "=l"(f), "=l"(g), "=l"(h) : "l"(p));
+}
+
+// Light c (position, intensity) of the record at a slot.
+template <bool PAIRED>
+__device__ __forceinline__ float4 light_at(const float4 *records, uint32_t slot, uint32_t c) {
+    if constexpr (!PAIRED) return __ldg(&records[4 * (size_t)hrr_slot_node(slot) + 2u * c]);
+    const float *r = reinterpret_cast<const float *>(records + 4 * (size_t)slot) + c;
+    return make_float4(-r[0], -r[2], -r[4], r[12]);
 }
 
 // The shift of sample s at tile pixel (tx, ty).
@@ -115,6 +123,7 @@ __device__ __forceinline__ void emit(const SampleLaunch &P, uint2 *wbuf, uint8_t
 
 namespace {
 
+template <bool PAIRED>
 __global__ void __launch_bounds__(kThreads, kMinBlocks) cull_samples_kernel(const __grid_constant__ SampleLaunch P) {
     __shared__ uint2 buf[kWarps][kBuf];
     __shared__ uint8_t smp[kWarps][kBuf];
@@ -145,8 +154,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) cull_samples_kernel(cons
         if ((uint32_t)lane < P.n_samples) rl = shift_of(P, (uint32_t)lane, ty, tx);
         const uint32_t cl = __brev(0u - rl);
         if (P.n_lights == 1) {  // the root is a leaf (record 0, slot 0)
-            const float *rec = reinterpret_cast<const float *>(P.pairs_rec);
-            const float4 q0 = make_float4(-rec[0], -rec[2], -rec[4], rec[12]);
+            const float4 q0 = light_at<PAIRED>(P.records, 0u, 0u);
             uint32_t acc = 0;
             for (uint32_t s = 0; s < P.n_samples; ++s) {
                 const uint32_t rs = __shfl_sync(0xFFFFFFFFu, rl, s);
@@ -187,8 +195,9 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) cull_samples_kernel(cons
             // take the exact test.
             if (active) sample_visits += __popc(e.y);
             hrr_f2 nlox, nloy, nloz, nhix, nhiy, nhiz, imax, links;
-            load_pairs(&P.pairs_rec[4 * (size_t)e.x], nlox, nloy, nloz, nhix, nhiy, nhiz, imax, links);
             const uint32_t node = hrr_slot_node(e.x);
+            if constexpr (PAIRED) load_pairs(&P.records[4 * (size_t)e.x], nlox, nloy, nloz, nhix, nhiy, nhiz, imax, links);
+            else hrr_load_binary(&P.records[4 * (size_t)node], nlox, nloy, nloz, nhix, nhiy, nhiz, imax, links);
             const uint32_t split = (uint32_t)links, other = (uint32_t)(links >> 32);
             const uint32_t first = min(node, other), last = max(node, other);
             const bool ok = active && last < P.n_lights && split - first < last - first;  // first <= split < last < n
@@ -209,14 +218,14 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) cull_samples_kernel(cons
                 if (s1) mask1 |= bit;
             }
             if ((!int0 && mask0) || (!int1 && mask1)) {
-                const float *rec = reinterpret_cast<const float *>(P.pairs_rec + 4 * (size_t)e.x);
                 for (uint32_t c = 0; c < 2; ++c) {
                     uint32_t m2 = c == 0 ? (int0 ? 0u : mask0) : (int1 ? 0u : mask1), acc = 0;
                     const uint32_t i = c == 0 ? split : last;
                     for (; m2; m2 &= m2 - 1u) {
                         const uint32_t s = (uint32_t)__ffs((int)m2) - 1u;
                         const uint32_t xi = __brev(i) + shift_of(P, s, ty, tx);
-                        if (hrr_pair_accepts(xi, tau, -rec[c], -rec[2 + c], -rec[4 + c], rec[12 + c], ex, ey, ez)) acc |= 1u << s;
+                        const float4 l = light_at<PAIRED>(P.records, e.x, c);
+                        if (hrr_pair_accepts(xi, tau, l.x, l.y, l.z, l.w, ex, ey, ez)) acc |= 1u << s;
                     }
                     if (c == 0) acc0 = acc;
                     else acc1 = acc;
@@ -279,12 +288,12 @@ int hrr_cull_samples_impl(hrr_ctx *ctx, const hrr_eyes &E, uint32_t n_eyes, cons
     HRR_CUDA(ctx, cudaMemsetAsync(counts, 0, 40 * sizeof(unsigned long long), st));
     HRR_CUDA(ctx, cudaMemsetAsync(ctx->counters + 2, 0, sizeof(unsigned long long), st));  // flags
     if (n_eyes > 0) {
-        static int per_sm = 0;  // resident blocks per SM of the kernel
+        const auto kernel = tree->pairs ? cull_samples_kernel<true> : cull_samples_kernel<false>;
+        static int occupancy[2] = {0, 0};  // resident blocks per SM of each
+        int &per_sm = occupancy[tree->pairs ? 1 : 0];
         if (!per_sm) {
             int m = 0;
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&m, cull_samples_kernel, kThreads, 0) != cudaSuccess ||
-                m < 1)
-                m = 1;
+            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&m, kernel, kThreads, 0) != cudaSuccess || m < 1) m = 1;
             per_sm = m;
         }
         const unsigned long long needed = ((unsigned long long)n_eyes + kWarps - 1) / kWarps;
@@ -305,7 +314,7 @@ int hrr_cull_samples_impl(hrr_ctx *ctx, const hrr_eyes &E, uint32_t n_eyes, cons
         }
         SampleLaunch P{};
         P.ex = E.x; P.ey = E.y; P.ez = E.z; P.px = E.px; P.py = E.py;
-        P.pairs_rec = tree->pairs;
+        P.records = tree->pairs ? tree->pairs : reinterpret_cast<const float4 *>(tree->nodes);
         P.perm = tree->perm;
         P.tile = ctx->tile;
         P.tile_w = ctx->tile_w; P.tile_h = ctx->tile_h; P.tile_d = ctx->tile_d ? ctx->tile_d : 1u;
@@ -320,7 +329,7 @@ int hrr_cull_samples_impl(hrr_ctx *ctx, const hrr_eyes &E, uint32_t n_eyes, cons
         P.counts = counts;
         P.flags = ctx->counters + 2;
         P.spill = reinterpret_cast<uint2 *>(ctx->spill);
-        cull_samples_kernel<<<grid, kThreads, 0, st>>>(P);
+        kernel<<<grid, kThreads, 0, st>>>(P);
         ++ctx->launches;
         HRR_CUDA(ctx, cudaGetLastError());
     }

@@ -11,9 +11,18 @@ ROOT = os.path.dirname(HERE)
 PACKAGE = "paper_1907_12343_gb300"
 
 
-def build(where) -> str:
-    """Copy and compile under `where`; returns the directory to import the package from."""
-    where = str(where)
+_built = None
+
+
+def build(tmp_path_factory) -> str:
+    """Copy and compile, once per process; returns the directory to import the package from."""
+    global _built
+    if _built is None:
+        _built = _build(str(tmp_path_factory.mktemp("fake")))
+    return _built
+
+
+def _build(where: str) -> str:
     shutil.copytree(os.path.join(ROOT, "include"), os.path.join(where, "include"))
     shutil.copytree(os.path.join(ROOT, PACKAGE), os.path.join(where, PACKAGE),
                     ignore=shutil.ignore_patterns("_build", "__pycache__"))

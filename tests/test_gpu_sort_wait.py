@@ -56,5 +56,5 @@ print("ok")
 """
 
 
-def test_a_wait_that_runs_out_is_a_timeout(tmp_path):
-    assert fake_lib.run(fake_lib.build(tmp_path), SCRIPT).strip().endswith("ok")
+def test_a_wait_that_runs_out_is_a_timeout(tmp_path_factory):
+    assert fake_lib.run(fake_lib.build(tmp_path_factory), SCRIPT).strip().endswith("ok")
