@@ -508,23 +508,27 @@ __global__ void __launch_bounds__(kThreads) connect_kernel(const ConnectArgs A) 
     }
 }
 
-// Sorts by the key bits from `shift` up, as the light builder does.
+// Sorts by the key bits from `shift` up, as the light builder does. All that is done with before the
+// binary nodes are collapsed is kept in the memory of the nodes they become (106 of its 128 bytes
+// a triangle), so a build takes 256 bytes a triangle at most, not 362.
 int scene_attempt(hrr_ctx *ctx, const float *tris, uint32_t n, hrr_scene *sc, int shift) {
     cudaStream_t st = ctx->stream;
     const size_t un = n;
     unsigned long long *flags = ctx->counters + 2;
-    const size_t bytes = 3 * pad256(sizeof(float) * un) + 2 * pad256(sizeof(uint64_t) * un) + 2 * pad256(sizeof(uint32_t) * un) +
-                         pad256(sort_scratch_bytes(un)) + pad256(sizeof(float4) * un) + pad256(2 * sizeof(float4) * un) +
-                         pad256(sizeof(hrr_node) * un) + box_scratch_bytes(n);
+    const size_t work = 3 * pad256(sizeof(float) * un) + 2 * pad256(sizeof(uint64_t) * un) + 2 * pad256(sizeof(uint32_t) * un) +
+                        pad256(sort_scratch_bytes(un)) + pad256(sizeof(float4) * un) + pad256(2 * sizeof(float4) * un) +
+                        box_scratch_bytes(n);
+    const bool fits = work <= sizeof(uint32_t) * kNodeWords * (un - 1);  // few triangles: the padding does not
     char *scratch = nullptr;
-    HRR_CUDA(ctx, hrr_alloc(ctx, &scratch, bytes));
+    HRR_CUDA(ctx, hrr_alloc(ctx, &scratch, pad256(sizeof(hrr_node) * un) + (fits ? 0 : work)));
     char *p = scratch;
+    hrr_node *nodes = carve<hrr_node>(p, un);
+    if (fits) p = reinterpret_cast<char *>(sc->nodes);
     float *cx = carve<float>(p, un), *cy = carve<float>(p, un), *cz = carve<float>(p, un);
     uint64_t *keys0 = carve<uint64_t>(p, un), *keys1 = carve<uint64_t>(p, un);
     uint32_t *vals0 = carve<uint32_t>(p, un), *perm = carve<uint32_t>(p, un);
     const SortScratch ss = carve_sort(p, un);
     float4 *spos = carve<float4>(p, un), *box = carve<float4>(p, 2 * un);
-    hrr_node *nodes = carve<hrr_node>(p, un);
     const BoxScratch bs = carve_boxes(p, n);
     const unsigned g = (unsigned)((un + kThreads - 1) / kThreads);
     cudaError_t e = cudaMemsetAsync(flags, 0, sizeof(unsigned long long), st);

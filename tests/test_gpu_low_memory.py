@@ -108,3 +108,44 @@ print("ok")
 
 def test_hierarchies_without_paired_records(tmp_path_factory):
     assert fake_lib.run(fake_lib.build(tmp_path_factory), LIGHTS).strip().endswith("ok")
+
+
+SCENES = HEAD + """
+rng = np.random.default_rng(4)
+n_s = 20000
+x = [torch.from_numpy(a.astype(np.float32)).to(dev()) for a in rng.random((6, n_s))] + [torch.ones(n_s, device=dev())]
+pairs = torch.arange(n_s, dtype=torch.int32, device=dev()).repeat_interleave(2).view(n_s, 2).contiguous()
+sums = torch.zeros(n_s, device=dev())
+
+def visible(scene):
+    v = torch.zeros(n_s, dtype=torch.uint8, device=dev())
+    ctx.connect(*x[:3], tuple(x[3:]), 1e-3, pairs, n_s, scene=scene, visible=v, eye_sum=sums)
+    return v.cpu().numpy()
+
+for n, spread in ((2, 1.0), (300, 1.0), (150000, 1.0), (150000, 1e-9)):
+    tris = 0.5 + spread * (rng.random((n, 1, 3)) - 0.5) + 0.5 * n ** -0.5 * rng.standard_normal((n, 3, 3))
+    if spread < 1:  # the keys of one cell: a full sort
+        tris += 0.5 - tris.mean(axis=1, keepdims=True)
+    t = torch.from_numpy(tris.reshape(n, 9).astype(np.float32)).to(dev())
+    scene = ctx.build_scene(t)
+    want, kept = visible(scene), used()
+    assert 0 < want.sum() < n_s or n == 2
+    os.environ["HRR_FAKE_MEMORY"] = str(kept + 257 * n + (1 << 16))
+    tight = ctx.build_scene(t)
+    assert np.array_equal(visible(tight), want)
+    os.environ["HRR_FAKE_MEMORY"] = str(kept + 192 * (n - 1))
+    try:
+        ctx.build_scene(t)
+        raise SystemExit("built without memory")
+    except hrr.HRRError as e:
+        assert e.status == hrr.HRR_ERR_OOM, e
+    del os.environ["HRR_FAKE_MEMORY"]
+    tight.free()
+    scene.free()
+    assert used() == 0
+print("ok")
+"""
+
+
+def test_scenes_build_in_the_memory_of_their_nodes(tmp_path_factory):
+    assert fake_lib.run(fake_lib.build(tmp_path_factory), SCENES).strip().endswith("ok")
