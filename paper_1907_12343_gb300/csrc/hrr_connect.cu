@@ -315,7 +315,7 @@ __device__ __forceinline__ void finish(const ConnectArgs &A, unsigned long long 
 
 // Lights as float4 by id, so that a pair's light is one scattered load.
 __global__ void __launch_bounds__(kThreads) pack_lights_kernel(hrr_lights l, uint32_t n, float4 *packed) {
-    for (uint32_t i = blockIdx.x * kThreads + threadIdx.x; i < n; i += gridDim.x * kThreads)
+    for (size_t i = blockIdx.x * kThreads + threadIdx.x; i < n; i += gridDim.x * kThreads)  // n may be up to 2^32 - 1
         packed[i] = make_float4(l.x[i], l.y[i], l.z[i], l.intensity[i]);
 }
 
@@ -659,7 +659,7 @@ int hrr_connect(hrr_ctx *ctx, hrr_eyes eyes, uint32_t n_eyes, hrr_lights lights,
         // packing pays from a few pairs per light on (its pass reads and writes 32 bytes a light; a
         // pair saves three requests) and where the extra launch is small beside the rest
         float4 *packed = nullptr;
-        if (!scene && n_pairs >= (1u << 20) && n_pairs / 4 >= n_lights &&
+        if (!scene && n_lights && n_pairs >= (1u << 20) && n_pairs / 4 >= n_lights &&
             hrr_alloc(ctx, &packed, sizeof(float4) * (size_t)n_lights) != cudaSuccess) {
             cudaGetLastError();
             packed = nullptr;  // no memory for it: gather from the arrays
@@ -675,7 +675,7 @@ int hrr_connect(hrr_ctx *ctx, hrr_eyes eyes, uint32_t n_eyes, hrr_lights lights,
         const unsigned grid = (unsigned)std::min<unsigned long long>(want, (unsigned long long)per_sm * ctx->sm_count);
         hrr_timing_begin(ctx);
         if (packed) {
-            pack_lights_kernel<<<(unsigned)std::min<size_t>((n_lights + kThreads - 1) / kThreads, ctx->sm_count * 8), kThreads,
+            pack_lights_kernel<<<(unsigned)std::min<size_t>(((size_t)n_lights + kThreads - 1) / kThreads, ctx->sm_count * 8), kThreads,
                                  0, st>>>(lights, n_lights, packed);
             ++ctx->launches;
         }
