@@ -154,7 +154,7 @@ int hrr_batch_create(hrr_ctx *ctx, const hrr_frame *frames, uint32_t n_frames, c
             release(b);
             return hrr_fail(ctx, HRR_ERR_INVALID_ARG, "a frame's tree has no records of the tuning's node width");
         }
-        d.paired = fr.tree->pairs != nullptr;
+        d.binary = reinterpret_cast<const float4 *>(fr.tree->nodes);
         d.top = hrr_tree_top(fr.tree);
         d.perm = fr.tree->perm;
         d.tile = fr.dev_tile ? hrr_tile_layer(fr.dev_tile, fr.tile_w, fr.tile_h, fr.tile_d, fr.sample_index)

@@ -17,15 +17,23 @@ namespace {
 // batched kernels.
 struct CullKernel {
     int variant, width, ring, threads, top;
-    const void *single, *batch;
+    const void *single[2], *batch[2];  // [1]: over the binary records of trees without paired ones
     int occ[2];  // resident blocks per SM (single, batched), 0 until first asked
 };
 
 template <int VARIANT, int W, int RING, int THREADS, int TOP>
 CullKernel cull_entry() {
-    return {VARIANT, W, RING, THREADS, TOP,
-            reinterpret_cast<const void *>(cull_single_kernel<VARIANT, W, RING, THREADS, TOP>),
-            reinterpret_cast<const void *>(cull_batch_kernel<VARIANT, W, RING, THREADS, TOP>), {0, 0}};
+    CullKernel k{VARIANT, W, RING, THREADS, TOP,
+                 {reinterpret_cast<const void *>(cull_single_kernel<VARIANT, W, RING, THREADS, TOP, true>)},
+                 {reinterpret_cast<const void *>(cull_batch_kernel<VARIANT, W, RING, THREADS, TOP, true>)}, {0, 0}};
+    if constexpr (W == 2) {
+        k.single[1] = reinterpret_cast<const void *>(cull_single_kernel<VARIANT, W, RING, THREADS, TOP, false>);
+        k.batch[1] = reinterpret_cast<const void *>(cull_batch_kernel<VARIANT, W, RING, THREADS, TOP, false>);
+    } else {
+        k.single[1] = k.single[0];
+        k.batch[1] = k.batch[0];
+    }
+    return k;
 }
 
 template <int VARIANT>
@@ -72,7 +80,7 @@ int cull_occupancy(CullKernel &k, bool batch) {
     int &n = k.occ[batch ? 1 : 0];
     if (!n) {
         int m = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&m, batch ? k.batch : k.single, k.threads, 0) !=
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&m, batch ? k.batch[0] : k.single[0], k.threads, 0) !=
                 cudaSuccess || m < 1) {
             cudaGetLastError();
             m = 1;
@@ -86,14 +94,17 @@ cudaError_t launch_single(CullKernel &k, unsigned grid, const Launch &Lc, const 
     Launch lc = Lc;
     Frame f = fr;
     void *args[] = {&lc, &f};
-    return cudaLaunchKernel(k.single, dim3(grid), dim3(k.threads), args, 0, st);
+    return cudaLaunchKernel(k.single[f.nodes == f.binary], dim3(grid), dim3(k.threads), args, 0, st);
 }
 
-cudaError_t launch_batch(CullKernel &k, unsigned grid, const Launch &Lc, const FrameArray<kMaxFrames> &fa,
-                         cudaStream_t st) {
+// One tree without paired records has the launch read all its trees' binary ones.
+cudaError_t launch_batch(CullKernel &k, unsigned grid, const Launch &Lc, FrameArray<kMaxFrames> &fa, cudaStream_t st) {
     Launch lc = Lc;
-    void *args[] = {&lc, const_cast<FrameArray<kMaxFrames> *>(&fa)};
-    return cudaLaunchKernel(k.batch, dim3(grid), dim3(k.threads), args, 0, st);
+    bool bare = false;
+    for (uint32_t i = 0; i < lc.n_frames; ++i) bare |= fa.f[i].nodes == fa.f[i].binary;
+    for (uint32_t i = 0; bare && i < lc.n_frames; ++i) fa.f[i].nodes = fa.f[i].binary;
+    void *args[] = {&lc, &fa};
+    return cudaLaunchKernel(k.batch[bare], dim3(grid), dim3(k.threads), args, 0, st);
 }
 
 }  // namespace
@@ -154,7 +165,7 @@ Frame single_frame(const hrr_ctx *ctx, const hrr_eyes &E, const hrr_tree *tree, 
     Frame fr{};
     fr.ex = E.x; fr.ey = E.y; fr.ez = E.z; fr.px = E.px; fr.py = E.py;
     fr.nodes = hrr_cull_records(tree, tn);
-    fr.paired = tree->pairs != nullptr;
+    fr.binary = reinterpret_cast<const float4 *>(tree->nodes);
     fr.top = hrr_tree_top(tree);
     fr.perm = tree->perm;
     fr.tile = hrr_tile_layer(ctx->tile, ctx->tile_w, ctx->tile_h, ctx->tile_d, opts.sample_index);

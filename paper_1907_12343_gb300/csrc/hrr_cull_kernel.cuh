@@ -455,8 +455,9 @@ __device__ __forceinline__ uint32_t walk_pairs(const Frame &fr, const Eye &E, ui
 }
 
 // The traversal over the frames F (F[0] alone for a single frame); TOP levels of the
-// hierarchy evaluated by the head (0: none, the walk starts at the root).
-template <int VARIANT, bool BATCH, int W, int RING, int THREADS, int TOP>
+// hierarchy evaluated by the head (0: none, the walk starts at the root). PAIRED: the records of
+// width two are paired ones, for every frame of the launch.
+template <int VARIANT, bool BATCH, int W, int RING, int THREADS, int TOP, bool PAIRED>
 __device__ __forceinline__ void traverse(const Launch &Lc, const Frame *F) {
     constexpr int kWarps = THREADS / 32;
     constexpr uint32_t kRing = RING;
@@ -521,8 +522,7 @@ __device__ __forceinline__ void traverse(const Launch &Lc, const Frame *F) {
         E.r = fr.tile[ty * fr.tile_w + tx] + fr.shift_offset;
         if (n_lights == 1) {  // the root is a leaf (record 0, slot 0, in either layout)
             if (lane == 0 && fr.eye_visits) fr.eye_visits[j] = 0;
-            const float4 l = fr.paired ? light_of<W, true>(nodes, 0u, 0u) : light_of<W, false>(nodes, 0u, 0u);
-            take(fr, E, j, lane, lane == 0, l, 0u);
+            take(fr, E, j, lane, lane == 0, light_of<W, PAIRED>(nodes, 0u, 0u), 0u);
             continue;
         }
         E.c = __brev(0u - E.r);
@@ -539,10 +539,8 @@ __device__ __forceinline__ void traverse(const Launch &Lc, const Frame *F) {
             __syncwarp();
         }
         if constexpr (W == 2) {
-            visits += fr.paired ? walk_pairs<VARIANT, kRing, true>(fr, E, j, lane, ring, queue, S, visits, HRR_WARP_SPILL,
-                                                                   Lc.spill_cap, Lc.flags)
-                                : walk_pairs<VARIANT, kRing, false>(fr, E, j, lane, ring, queue, S, visits, HRR_WARP_SPILL,
-                                                                    Lc.spill_cap, Lc.flags);
+            visits += walk_pairs<VARIANT, kRing, PAIRED>(fr, E, j, lane, ring, queue, S, visits, HRR_WARP_SPILL,
+                                                         Lc.spill_cap, Lc.flags);
         } else {
             while (S > 0) {
                 if (visits >= n_lights) {  // each internal node is visited at most once per eye
@@ -645,16 +643,16 @@ __device__ __forceinline__ void traverse(const Launch &Lc, const Frame *F) {
 
 // A single frame travels as a plain kernel parameter; a batch's frames as a grid-constant
 // array (indexed by the frame a warp is on).
-template <int VARIANT, int W, int RING, int THREADS, int TOP>
+template <int VARIANT, int W, int RING, int THREADS, int TOP, bool PAIRED>
 __global__ void __launch_bounds__(THREADS, min_blocks<W>(THREADS))
 cull_single_kernel(const Launch Lc, const Frame fr) {
-    traverse<VARIANT, false, W, RING, THREADS, TOP>(Lc, &fr);
+    traverse<VARIANT, false, W, RING, THREADS, TOP, PAIRED>(Lc, &fr);
 }
 
-template <int VARIANT, int W, int RING, int THREADS, int TOP>
+template <int VARIANT, int W, int RING, int THREADS, int TOP, bool PAIRED>
 __global__ void __launch_bounds__(THREADS, min_blocks<W>(THREADS))
 cull_batch_kernel(const __grid_constant__ Launch Lc, const __grid_constant__ FrameArray<kMaxFrames> FA) {
-    traverse<VARIANT, true, W, RING, THREADS, TOP>(Lc, FA.f);
+    traverse<VARIANT, true, W, RING, THREADS, TOP, PAIRED>(Lc, FA.f);
 }
 
 }  // namespace

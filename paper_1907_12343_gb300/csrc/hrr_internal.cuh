@@ -207,7 +207,7 @@ struct hrr_cull_frame_t {
     float tau;
     uint32_t eye_begin;              // first eye of the frame covered by this launch
     unsigned long long cursor_begin; // where the frame's eyes start on the launch's cursor
-    bool paired;                     // width two: the records are hrr_tree::pairs, not its nodes
+    const float4 *binary;            // the binary records, for a launch over trees without paired ones
 };
 
 // Traversal defaults (the fastest form on the 1920x1080-eye, 2^20-light frame): node width,

@@ -262,7 +262,7 @@ bool enqueue_slice(hrr_server *s, int k) {
         d.ex = j->desc.eyes.x; d.ey = j->desc.eyes.y; d.ez = j->desc.eyes.z;
         d.px = j->desc.eyes.px; d.py = j->desc.eyes.py;
         d.nodes = hrr_cull_records(j->desc.tree, s->tuning);
-        d.paired = j->desc.tree->pairs != nullptr;
+        d.binary = reinterpret_cast<const float4 *>(j->desc.tree->nodes);
         d.top = hrr_tree_top(j->desc.tree);
         d.perm = j->desc.tree->perm;
         d.tile = j->tile; d.tile_w = j->tile_w; d.tile_h = j->tile_h;
