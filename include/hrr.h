@@ -76,7 +76,8 @@ typedef struct hrr_eyes {
     const uint16_t *px, *py;
 } hrr_eyes;
 
-/* Internal node record of the light hierarchy (64 bytes, 16-byte aligned). Internal
+/* Internal node record of the light hierarchy (64 bytes, 16-byte aligned in the library's
+ * own hierarchies; an array of the caller's may start at any word). Internal
  * node n is a binary radix-tree node over the Morton-sorted leaves; its leaf range is
  * [min(n, other_end), max(n, other_end)] (inclusive) and it splits after leaf `split`:
  * child 0 covers [first, split], child 1 covers [split + 1, last]. A child whose range
@@ -183,8 +184,9 @@ int hrr_kernel_time(hrr_ctx *ctx, double *ms, uint64_t *launches);
  * 1 <= n_lights <= 2^31 - 1. Device memory: 324 bytes a light for the hierarchy, and up to 67
  * more while it is built. Where that is not there the hierarchy does without its paired
  * records and takes 196 bytes a light: every result stays the same, and culls of node width
- * 2 take about a tenth longer. Synchronises the context stream; returns
- * HRR_ERR_INVALID_ARG if any position or intensity is not finite. */
+ * 2 take 9 to 18% longer. Synchronises the context stream; returns
+ * HRR_ERR_INVALID_ARG if any position or intensity is not finite, HRR_ERR_OOM if there is
+ * not that much memory either, HRR_ERR_TIMEOUT if a wait of the sort ran out. */
 int hrr_build_light_tree(hrr_ctx *ctx, hrr_lights lights, uint32_t n_lights, hrr_tree **out);
 
 /* Hierarchy shapes over the same Morton leaf order (so the same accepted set, Sec. 1):
@@ -246,7 +248,7 @@ int hrr_tree_download(hrr_ctx *ctx, const hrr_tree *tree, hrr_node *host_nodes,
  * sorted-leaf -> original id permutation written to dev_perm (n_lights entries), both
  * device memory the caller owns. *out_height (may be NULL) receives the height.
  *   - Working memory is one library-wide static device array sized for
- *     HRR_STATIC_BUILD_MAX_LIGHTS lights (about 3.6 MiB), which every GPU that loads
+ *     HRR_STATIC_BUILD_MAX_LIGHTS lights (about 3.7 MiB), which every GPU that loads
  *     the library keeps until the process exits. Larger n_lights is rejected with
  *     HRR_ERR_INVALID_ARG.
  *   - Runs on the calling thread's current device, on cuda_stream (NULL = the legacy

@@ -249,7 +249,7 @@ constexpr size_t static_scratch_bytes(size_t n) {
 }
 
 // The shared working memory of every hrr_build_light_tree_static call on a device
-// (about 3.6 MiB for 65536 lights), held by each device that loads the library.
+// (about 3.7 MiB for 65536 lights), held by each device that loads the library.
 static __device__ __align__(256) unsigned char g_static_build_scratch[static_scratch_bytes(kStaticMaxLights)];
 
 std::mutex g_static_mutex;

@@ -40,9 +40,11 @@ constexpr int kTriFloats = 16;  // a sorted triangle's stride (64 bytes: aligned
 //   words 4-15  per axis: 8 low sides, 8 high sides, a byte 0x80 | q each; the side lies at
 //               o + q S / 128, so 1 + q / 128 is one byte permutation away from a float
 //   words 16-23 children: a triangle (bit 31 set) or a node
-// A binary walk over 64-byte nodes was bound by its scattered loads (93% of the L1 data pipe, 87 loads
-// a segment); this one is bound by instructions (70% of the issue slots at 32 warps per SM, L1 at
-// 55%). 8.3e6 segments against 2^18 triangles, scene build included: 6.35 -> 4.54 ms.
+// (Wide nodes with quantised boxes are a published method: Ylitie, Karras and Laine, "Efficient
+// Incoherent Ray Traversal on GPUs Through Compressed Wide BVHs", HPG 2017.) A binary walk over
+// 64-byte nodes was bound by its scattered loads (93% of the L1 data pipe, 87 loads a segment);
+// this one is bound by instructions (70% of the issue slots at 32 warps per SM, L1 at 53%). 8.3e6
+// segments against 2^18 triangles, scene build included: 6.35 ms, now 4.20 to 4.45.
 constexpr uint32_t kNodeWords = 32;
 constexpr uint32_t kTriangle = 0x80000000u;
 constexpr int kSharedStack = 24;   // entries of a segment's stack in shared memory

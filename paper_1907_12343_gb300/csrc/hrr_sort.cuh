@@ -8,8 +8,9 @@
 // tiles with lower tickets, whose blocks are running or done. Every wait is bounded: one that runs
 // out raises HRR_FLAG_WAIT, the tile goes on with the sum it has (so that those behind it end
 // too; no place past the arrays is written), and the kernels after the sort leave its result
-// alone, parts of which are then not written; the call reports HRR_ERR_TIMEOUT. With a histogram, a scan and a scatter kernel per digit the sort was a chain of
-// 24 launches of 3 to 29 us each (340 us for 2^20 keys, 290 us for 100,003).
+// alone, parts of which are then not written; the call reports HRR_ERR_TIMEOUT. With a histogram,
+// a scan and a scatter kernel per digit the sort was a chain of 24 launches of 3 to 29 us each
+// (340 us for 2^20 keys, 290 us for 100,003).
 //
 // Few lights share the upper 32 bits of their keys, so a build sorts by those (four passes) and
 // puts the short runs that agree in them in order afterwards (gather_sorted_kernel); keys with
@@ -101,7 +102,8 @@ __global__ void __launch_bounds__(kSortThreads) sort_pass_kernel(const uint64_t 
     constexpr uint32_t kTile = kSortThreads * ITEMS, kWarps = kSortThreads / 32;
     // Tiles looked back on at once: their words are loaded together, so that many tiles ahead cost
     // few round trips. A build of 100,003 lights (98 small tiles) takes 164 us with 32 against 186 with
-    // 8 or 16; large tiles have no registers for more than 16 (2^20 lights: 1065 us, 1073 with 8 or 32).
+    // 8 or 16; large tiles have no registers for more than 16 (a cost-driven build of 2^20 lights, when
+    // its launches were not chained yet: 1065 us, 1073 with 8 or 32).
     constexpr uint32_t kLook = ITEMS <= kSortSmall ? 32u : 16u;
     __shared__ uint64_t exchange[kTile];
     __shared__ uint32_t warp_cnt[kWarps][256];

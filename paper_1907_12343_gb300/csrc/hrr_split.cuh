@@ -24,7 +24,7 @@
 //     and the rest are subtrees of a warp each.
 //   * up to 32 lights: one warp builds the whole subtree, a light per lane.
 // With one level of every size per pass, four kernels and a host round trip each, the build of
-// 2^20 lights took 1843 us, now 989 us. What is left is instructions (the subtrees of 33 to 1024
+// 2^20 lights took 1843 us, now 980 to 1000 us (a whole call; its device time is 0.93 ms). What is left is instructions (the subtrees of 33 to 1024
 // lights and below: 212 and 132 us) and the latency of about twenty levels (8 to 20 us each).
 #pragma once
 
@@ -575,7 +575,8 @@ int cost_topology(hrr_ctx *ctx, const float4 *spos, const uint64_t *keys, uint32
     }
     uint64_t left = n > kSubMax;  // ranges of more than kSubMax lights still to split
     uint32_t level = 0;
-    // as many levels as such ranges usually have (1.5 per halving, and two), then a few at a time
+    // two levels per halving and one (21 for 2^20 lights, the last few of which seldom have any such
+    // range left), then a few at a time
     uint32_t batch = 2;
     for (size_t m = un / kSubMax; m > 1; m >>= 1) batch += batch & 1 ? 2 : 1;
     int rc = HRR_OK;
