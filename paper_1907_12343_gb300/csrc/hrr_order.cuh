@@ -74,10 +74,11 @@ __global__ void __launch_bounds__(kOrderThreads) gather_sorted_kernel(const floa
                                                                  unsigned long long *flags) {
     chain_begin();
     const uint32_t i = blockIdx.x * kOrderThreads + threadIdx.x;
-    if (i >= n || (*(volatile unsigned long long *)flags & HRR_FLAG_WAIT)) return;
+    if (i >= n) return;
     const uint32_t v = vals_in[i];
-    const float4 p = make_float4(x[v], y[v], z[v], inten[v]);
     const uint64_t key = keys_in[i];
+    if (*(volatile unsigned long long *)flags & HRR_FLAG_WAIT) return;  // read beside v and the key, not before them
+    const float4 p = make_float4(x[v], y[v], z[v], inten[v]);
     uint32_t to = i;
     if (RUNS) {
         uint32_t left = 0, right = 0, ahead = 0;  // neighbours of the run, and those that move ahead of i
