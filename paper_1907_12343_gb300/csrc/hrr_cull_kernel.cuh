@@ -343,7 +343,7 @@ __device__ __forceinline__ uint32_t range_min_leaves(uint32_t a, uint32_t z, con
 // most n_lights - 1. Each step visits up to 32 nodes, one per lane. Everything rare shares a
 // test with something else that is rare: fewer than 32 entries or visits left; surviving leaves
 // or a corrupt record. That and the clamped range minimum took a step from 180 to 134 warp
-// instructions, the issue slots from 81% to 65%, and left the L1 data pipe as the limit (94 to 95% on
+// instructions, the issue slots from 81% to 65%, and left the L1 data pipe as the limit (94 to 96% on
 // 480x270 eyes and 2^20 lights: 42 wavefronts a step for the records, 8 for the stack). PAIRED is
 // false for a tree without paired records: the same walk over its binary ones (5.58 ms instead of
 // 5.12 on those eyes and lights, 24.2 instead of 20.6 on 960x540).
