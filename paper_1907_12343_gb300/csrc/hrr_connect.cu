@@ -24,6 +24,7 @@
 struct hrr_scene {
     int device = 0;
     uint32_t n = 0;
+    bool large = false;         // a node of more than kLargeNode a side
     uint32_t *nodes = nullptr;  // n - 1 nodes of kNodeWords words (below); one when n == 1
     float *tris = nullptr;     // sorted triangles, 16 floats each: v0, e1 = v1 - v0, e2 = v2 - v0, pad
 };
@@ -47,6 +48,9 @@ constexpr int kTriFloats = 16;  // a sorted triangle's stride (64 bytes: aligned
 // segments against 2^18 triangles, scene build included: 6.35 ms, now 4.20 to 4.45.
 constexpr uint32_t kNodeWords = 32;
 constexpr uint32_t kTriangle = 0x80000000u;
+// A direction component counts as at least 1e-30 (the margin of the triangles' boxes covers the
+// difference), so an eye inside a node of S up to 2^27 has slab times up to 2 S 1e30, finite.
+constexpr uint32_t kLargeNode = 127 + 27;  // exponent of the largest such S
 constexpr int kSharedStack = 24;   // entries of a segment's stack in shared memory
 constexpr int kLocalStack = 232;   // ... and below them: 7 per level of at most 33, and a margin
 
@@ -101,6 +105,7 @@ __global__ void __launch_bounds__(kThreads) triangles_kernel(const float *__rest
 
 // Leaves that are boxes.
 struct BoxLeaves {
+    static constexpr bool kOwnNodes = true;
     const float4 *box;
     __device__ __forceinline__ Box operator()(uint32_t i) const { return box_of(box[2 * (size_t)i], box[2 * (size_t)i + 1]); }
 };
@@ -111,7 +116,7 @@ struct BoxLeaves {
 // it is rounded outwards: more than the rounding of the segment's slab arithmetic on a grid near
 // the eye (2^-16 of the grid; far from it the slab test's own widening covers it).
 __global__ void __launch_bounds__(kThreads) collapse_kernel(const float4 *__restrict__ nodes, uint32_t n,
-                                                            uint32_t *__restrict__ out, const unsigned long long *flags) {
+                                                            uint32_t *__restrict__ out, unsigned long long *flags) {
     const uint32_t g = blockIdx.x * kThreads + threadIdx.x;
     if (g >= n - 1 || (*flags & (HRR_FLAG_NONFINITE | HRR_FLAG_UNSORTED | HRR_FLAG_TOPOLOGY))) return;
     float4 lo[8], hi[8];
@@ -169,6 +174,7 @@ __global__ void __launch_bounds__(kThreads) collapse_kernel(const float4 *__rest
         const bool covered = __fsub_ru(b[c], o) <= 126.0f * s;
         w[c] = covered ? __float_as_uint(o) : 0u;
         w[3] |= (covered ? (uint32_t)(m + 7 + 127) : 255u) << (8 * c);
+        if (!covered || (uint32_t)(m + 7 + 127) > kLargeNode) atomicOr(flags, HRR_FLAG_LARGE);
         const float inv = __uint_as_float((uint32_t)(127 - m) << 23);
         uint32_t ql[2] = {0, 0}, qh[2] = {0, 0};
         for (int k = 0; k < 8; ++k) {
@@ -247,7 +253,12 @@ __device__ __forceinline__ void sides(uint32_t near, uint32_t far, int k, hrr_f2
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(t) : "l"(v), "l"(slope), "l"(start));
     hrr_unpack2(t, tn, tf);
 }
-// The children of a node that the segment's [0, 1] meets (slab test, widened by 2^-18).
+// The children of a node that the segment's [0, 1] meets (slab test, widened by 2^-18). LARGE: the
+// start of an axis may overflow (a zero or nearly zero component on a node of more than 2^27), which
+// would put both sides at the same infinity, even around an eye inside the node; 0 b + b makes such a
+// start no number, which the minima and maxima ignore, and the axis rejects nothing. The three
+// operations took 2% of the walk, so scenes without such nodes have a kernel without them.
+template <bool LARGE>
 __device__ __forceinline__ uint32_t meets(const uint32_t (&h)[8], const uint32_t (&q)[8], const float (&e)[3],
                                           const float (&inv)[3]) {
     hrr_f2 slope[3], start[3];
@@ -257,11 +268,8 @@ __device__ __forceinline__ uint32_t meets(const uint32_t (&h)[8], const uint32_t
     for (int c = 0; c < 3; ++c) {
         const float S = __uint_as_float(((h[3] >> (8 * c)) & 255u) << 23);
         const float a = S * inv[c];
-        // An axis whose start overflows (a nearly or wholly zero component on a node of some 1e8)
-        // would put both sides at the same infinity, even around an eye inside the node: 0 b + b
-        // makes it no number, which the minima and maxima below ignore, and the axis rejects nothing.
         float b = ((__uint_as_float(h[c]) - S) - e[c]) * inv[c];
-        b = __fmaf_rn(b, 0.0f, b);
+        if (LARGE) b = __fmaf_rn(b, 0.0f, b);
         slope[c] = hrr_pack2(a, a);
         start[c] = hrr_pack2(b, b);
         const bool back = inv[c] < 0.0f;
@@ -399,6 +407,7 @@ __global__ void __launch_bounds__(kThreads) weights_kernel(const ConnectArgs A, 
 // interleaved by lane (no bank conflicts whatever the depths). Letting nodes and triangles take
 // turns warp by warp (triangles only when 8, 12, 16 or 20 lanes had one) left too many lanes
 // waiting: 5.1 to 6.0 ms against 4.5; refilling below 16 or 28 busy lanes 4.6 and 4.8 ms.
+template <bool LARGE>
 __global__ void __launch_bounds__(kThreads) connect_kernel(const ConnectArgs A) {
     __shared__ uint32_t stack_all[kSharedStack][kThreads];
     uint32_t deep[kLocalStack];
@@ -441,9 +450,9 @@ __global__ void __launch_bounds__(kThreads) connect_kernel(const ConnectArgs A) 
                         const float den = fmaxf(d2, 1e-4f);
                         const float p = fminf(1.0f, __fdiv_rn(__fmul_rn(A.tau, inten), den));
                         w = __fdiv_rn(__fdiv_rn(inten, den), p);
-                        // a zero component is taken as 1e-30: its slab then admits exactly
+                        // a component below 1e-30 is taken as that: its slab then admits exactly
                         // the boxes whose range holds e (up to 1e-30, a conservative margin)
-                        for (int c = 0; c < 3; ++c) inv[c] = __frcp_rn(D[c] == 0.0f ? 1e-30f : D[c]);
+                        for (int c = 0; c < 3; ++c) inv[c] = __frcp_rn(fabsf(D[c]) < 1e-30f ? copysignf(1e-30f, D[c]) : D[c]);
                         cur = A.n_tris == 1 ? kTriangle : 0u;
                         sp = 0;
                         steps = 0;
@@ -469,7 +478,7 @@ __global__ void __launch_bounds__(kThreads) connect_kernel(const ConnectArgs A) 
             load8(node, h);
             load8(node + 8, q);
             load8(node + 16, ref);
-            const uint32_t mask = meets(h, q, e, inv);
+            const uint32_t mask = meets<LARGE>(h, q, e, inv);
             if (sp <= kSharedStack - 8) {
                 uint32_t *at = &stack_all[sp][threadIdx.x];
 #pragma unroll
@@ -559,6 +568,7 @@ int scene_attempt(hrr_ctx *ctx, const float *tris, uint32_t n, hrr_scene *sc, in
     if ((f & HRR_FLAG_RUNS) && shift) return scene_attempt(ctx, tris, n, sc, 0);
     if (f & HRR_FLAG_WAIT) return hrr_fail(ctx, HRR_ERR_TIMEOUT, "a wait of the sort ran out");
     if (f & HRR_FLAG_TOPOLOGY) return hrr_fail(ctx, HRR_ERR_DEVICE, "scene links");
+    sc->large = (f & HRR_FLAG_LARGE) != 0;
     return HRR_OK;
 }
 
@@ -666,7 +676,8 @@ int hrr_connect(hrr_ctx *ctx, hrr_eyes eyes, uint32_t n_eyes, hrr_lights lights,
             cudaGetLastError();
             packed = nullptr;  // no memory for it: gather from the arrays
         }
-        const void *fn = scene ? reinterpret_cast<const void *>(connect_kernel)
+        const auto walk = scene && scene->large ? connect_kernel<true> : connect_kernel<false>;
+        const void *fn = scene ? reinterpret_cast<const void *>(walk)
                                : packed ? reinterpret_cast<const void *>(weights_kernel<true>)
                                         : reinterpret_cast<const void *>(weights_kernel<false>);
         int per_sm = 0;
@@ -681,7 +692,7 @@ int hrr_connect(hrr_ctx *ctx, hrr_eyes eyes, uint32_t n_eyes, hrr_lights lights,
                                  0, st>>>(lights, n_lights, packed);
             ++ctx->launches;
         }
-        if (scene) connect_kernel<<<grid, kThreads, 0, st>>>(A);
+        if (scene) walk<<<grid, kThreads, 0, st>>>(A);
         else if (packed) weights_kernel<true><<<grid, kThreads, 0, st>>>(A, packed);
         else weights_kernel<false><<<grid, kThreads, 0, st>>>(A, nullptr);
         hrr_timing_end(ctx);

@@ -15,6 +15,7 @@ enum : unsigned long long {
     HRR_FLAG_WAIT = 32ull,     // a bounded wait of the sort ran out (cannot happen)
     // keys and values are not what the kernels after the sort take: in no order, or not written
     HRR_FLAG_UNSORTED = HRR_FLAG_RUNS | HRR_FLAG_WAIT,
+    HRR_FLAG_LARGE = 64ull,    // a scene has nodes on which slab times can overflow (no error)
 };
 
 // ------------------------------------------------------------------------------------
