@@ -134,6 +134,7 @@ __device__ __forceinline__ Box warp_box(const Box &x) {
 
 // Leaves that are lights: position and intensity.
 struct PointLeaves {
+    static constexpr bool kOwnNodes = false;  // without derived records the nodes are a caller's array
     const float4 *pos;
     __device__ __forceinline__ Box operator()(uint32_t i) const {
         const float4 p = pos[i];
@@ -336,7 +337,7 @@ __global__ void __launch_bounds__(kBoxBlock, 3) box_kernel(LEAVES leaf, uint32_t
     __syncthreads();
     if (whole && arrived[t] == 2u) {
         const float4 a0 = sa[0][t], b0 = sb[0][t], a1 = sa[1][t], b1 = sb[1][t];
-        store_record<(DERIVED > 0)>(reinterpret_cast<float4 *>(nodes) + 4 * (size_t)g, a0, b0, a1, b1, split, other);
+        store_record<(DERIVED > 0 || LEAVES::kOwnNodes)>(reinterpret_cast<float4 *>(nodes) + 4 * (size_t)g, a0, b0, a1, b1, split, other);
         if (DERIVED) {  // the children's entries are in the block too
             const bool leaf0 = first == split, leaf1 = split + 1u == last;
             const uint32_t k0 = leaf0 ? t : split - base, k1 = leaf1 ? t : split + 1u - base;
@@ -427,8 +428,8 @@ __global__ void __launch_bounds__(kSpanThreads) span_kernel(LEAVES leaf, uint32_
         if (!DERIVED) {
             const Box x0 = box_range(leaf, s, n, first, split), x1 = box_range(leaf, s, n, split + 1u, last);
             if (lane == 0)
-                store_record<false>(reinterpret_cast<float4 *>(nodes) + 4 * (size_t)g, box_a(x0), box_b(x0, 0u), box_a(x1),
-                                    box_b(x1, 0u), split, other);
+                store_record<LEAVES::kOwnNodes>(reinterpret_cast<float4 *>(nodes) + 4 * (size_t)g, box_a(x0), box_b(x0, 0u),
+                                                box_a(x1), box_b(x1, 0u), split, other);
             continue;
         }
         // the grandchildren's boxes; the children's are their unions
