@@ -45,7 +45,7 @@ constexpr int kTriFloats = 16;  // a sorted triangle's stride (64 bytes: aligned
 // Incoherent Ray Traversal on GPUs Through Compressed Wide BVHs", HPG 2017.) A binary walk over
 // 64-byte nodes was bound by its scattered loads (93% of the L1 data pipe, 87 loads a segment);
 // this one is bound by instructions (70% of the issue slots at 32 warps per SM, L1 at 53%). 8.3e6
-// segments against 2^18 triangles, scene build included: 6.35 ms, now 4.20 to 4.45.
+// segments against 2^18 triangles, scene build included: 6.35 ms, now 4.20 to 4.48.
 constexpr uint32_t kNodeWords = 32;
 constexpr uint32_t kTriangle = 0x80000000u;
 // A direction component counts as at least 1e-30 (the margin of the triangles' boxes covers the
